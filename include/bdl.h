@@ -159,8 +159,9 @@ int bdl_knn_noalloc(bdl_forest *f, const int32_t *q_dev, int64_t m, int k, int32
  * (0 = the default 32): each warp answers that many consecutive queries in
  * the order the call processes them, 32 at a time.  Used by bdl_knn,
  * bdl_knn_noalloc, bdl_knn_count, and by the batched calls and plans whose
- * forests[0] is f (a plan keeps the shape it was made with).  Results do not
- * depend on the shape.  Other values: BDL_EINVAL, shape unchanged.  Host
+ * forests[0] is f (a plan keeps the shape it was made with), where they take
+ * the thread-per-query kernel (small batches and high dimensions take one warp
+ * per query, which has one shape).  Results do not depend on the shape.  Other values: BDL_EINVAL, shape unchanged.  Host
  * only; no device work. */
 int bdl_set_knn_shape(bdl_forest *f, int block_threads, int queries_per_warp);
 

@@ -191,11 +191,39 @@ __host__ __device__ constexpr int rec_ints(int dim) { return (dim + 1 + 3) / 4 *
 // for the root and one for every internal node at a depth t with h - t even
 // (t > 0); a record describes its node's four descendants two levels down
 // (the root of an odd h: its two children), each an internal node that has a
-// record of its own or a leaf.  Ints of a record: the four entries' codes
-// (record slot, or -1 - leaf index), their live counts, then per coordinate
-// c the four entries' low bounds and the four high bounds, so that one
-// 16-byte load gives one bound of every entry.  32-byte aligned for every dim.
+// record of its own or a leaf.  8 + 8 dim ints, 32-byte aligned for every dim:
+// the four entries' codes (record slot, or -1 - leaf index), their live counts
+// and their (low, high) bounds of every coordinate, in one of two layouts.
+//  * dim <= 3: codes[4], lives[4], then per coordinate low[4], high[4]: the
+//    thread-per-query kernel, which looks at all four entries in one lane,
+//    reads the record in 16-byte loads and uses each word as it arrives (1M
+//    queries on 10M 3-D points: 2.76 ms, with the other layout 2.86; the
+//    warp-per-query kernel is 8% faster with that one).
+//  * dim >= 4, searched mostly by the warp-per-query kernel, with an entry's
+//    words in one lane: an entry is (low, high) per coordinate and (code, live),
+//    for odd dim the pair first, for even dim in a place of its own at the end,
+//    so that the bounds fill 16-byte words; word i of entry 0 .. 3 lie together,
+//    so that the four lanes of a record read 64 consecutive bytes at a time.
+//    A bound x is stored as the bits of the float 2^23 + x, so that the gap to
+//    a query is one exact float subtraction without a conversion.
+constexpr int32_t kBias = 0x4B000000;
+constexpr float kBiasF = 8388608.f;   // 2^23
 __host__ __device__ constexpr int packed_node_ints(int dim) { return 8 + 8 * dim; }
+__host__ __device__ constexpr bool packed_by_entry(int dim) { return dim >= 4; }
+__host__ __device__ constexpr int packed_code_at(int dim, int a) {
+  return !packed_by_entry(dim) ? a : (dim & 1) ? 4 * a : 8 * dim + 2 * a;
+}
+__host__ __device__ constexpr int packed_live_at(int dim, int a) {
+  return packed_code_at(dim, a) + (packed_by_entry(dim) ? 1 : 4);
+}
+// int i of entry a's 16-byte words (dim >= 4)
+__host__ __device__ constexpr int packed_quad_at(int a, int i) { return 16 * (i >> 2) + 4 * a + (i & 3); }
+__host__ __device__ constexpr int packed_lo_at(int dim, int a, int c) {
+  return !packed_by_entry(dim) ? 8 + 8 * c + a : packed_quad_at(a, 2 * c + ((dim & 1) ? 2 : 0));
+}
+__host__ __device__ constexpr int packed_hi_at(int dim, int a, int c) {
+  return packed_lo_at(dim, a, c) + (packed_by_entry(dim) ? 1 : 4);
+}
 
 __host__ __device__ inline int64_t quad_count(int H) {   // (4^H - 1) / 3 nodes in H 4-ary levels
   return (((int64_t)1 << (2 * H)) - 1) / 3;
@@ -621,6 +649,12 @@ struct KnnJob {
   int32_t *oi;
   int64_t *od;
 };
+// One forest's job and tree views as kernel parameters, read through the
+// constant cache (the per-tree fields are warp-uniform).
+struct KnnOne {
+  KnnJob job;
+  TreeView trees[kMaxLevel];
+};
 // Device bytes the job table of `calls` needs (0 for a single call, whose job
 // travels as kernel parameters; `table` may then be null).
 size_t knn_table_bytes(const std::vector<KnnCall> &calls);
@@ -632,6 +666,14 @@ int upload_knn_table(const std::vector<KnnCall> &calls, void *table, int64_t *wa
                      cudaStream_t s);
 int launch_knn_table(const void *table, int njobs, int64_t warps, int dim, int k, const KnnShape &sh,
                      unsigned long long *stats, cudaStream_t s);
+// The kernel with one warp per query (knn_warp.cu): whether a launch of m
+// queries on n points takes it, and its launches (the table's job prefix
+// counts one warp per query: upload_knn_table with qpw = 1).
+bool knn_by_warp(int dim, int k, int64_t m, int64_t n);
+// The same for the calls of one launch together.
+bool knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k);
+int launch_knn_warp_one(const KnnOne &P, int dim, int k, cudaStream_t s);
+int launch_knn_warp_table(const void *table, int njobs, int64_t warps, int dim, int k, cudaStream_t s);
 // k-NN for every call (all of dimension `dim`) in one launch; the job table
 // is uploaded to `table` (knn_table_bytes of device memory) on stream s.
 int launch_knn_jobs(const std::vector<KnnCall> &calls, int dim, int k, const KnnShape &sh, void *table,

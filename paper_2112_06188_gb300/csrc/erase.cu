@@ -129,7 +129,7 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
         const int e = d == 1 ? 1 : 2;
         const int64_t at = leaf_at >> (T.h - d);   // the node's index at depth d
         const int64_t r = packed_slot(T.h, d - e, at >> e);
-        atomicSub(&T.pk[r * rec + 4 + (int)(at & ((1 << e) - 1))], cnt);
+        atomicSub(&T.pk[r * rec + packed_live_at(F.dim, (int)(at & ((1 << e) - 1)))], cnt);
       }
     }
   }
@@ -545,13 +545,19 @@ __global__ void k_pack_lives_many(const TreeSeg *segs, const int64_t *pre, int n
     lv.z = g.live[veb_slot(g.h + 1, t + st, (i << st) + 2)];
     lv.w = g.live[veb_slot(g.h + 1, t + st, (i << st) + 3)];
   }
-  int4 *dst = reinterpret_cast<int4 *>(g.pk + packed_slot(g.h, t, i) * packed_node_ints(g.dim) + 4);
-  if (!g.err) {
-    *dst = lv;
-  } else {
-    const int4 have = *dst;
-    if (have.x != lv.x || have.y != lv.y || have.z != lv.z || have.w != lv.w) atomicOr(g.err, kErrLiveCount);
+  int32_t *r = g.pk + packed_slot(g.h, t, i) * packed_node_ints(g.dim);
+  if (!packed_by_entry(g.dim) && !g.err) {   // the four counts are one 16-byte word
+    *reinterpret_cast<int4 *>(r + packed_live_at(g.dim, 0)) = lv;
+    return;
   }
+  const int32_t v[4] = {lv.x, lv.y, lv.z, lv.w};
+  bool differ = false;
+  for (int a = 0; a < 4; ++a) {
+    int32_t *dst = r + packed_live_at(g.dim, a);
+    if (!g.err) *dst = v[a];
+    else differ = differ || *dst != v[a];
+  }
+  if (differ) atomicOr(g.err, kErrLiveCount);
 }
 
 // One CTA per forest: keep its buffer ids that are still alive, in order;

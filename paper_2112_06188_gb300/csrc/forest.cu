@@ -1472,6 +1472,7 @@ struct bdl_knn_plan {
     void *table;
     unsigned long long *stats;
     bdl::KnnShape shape;
+    bool by_warp;
   };
   struct Sort {
     const int32_t *q;
@@ -1542,8 +1543,9 @@ static int knn_plan_make(bdl_forest *const *F, int nf, const int32_t *const *q, 
     unsigned long long *stats = nullptr;
     for (int i = 0; i < nf; ++i)
       if (F[i]->dim == d && F[i]->knn_stats) stats = F[i]->knn_stats;
-    bdl_knn_plan::Part part{d, (int)groups[gi].size(), 0, p, stats, F[0]->knn_shape};
-    st = upload_knn_table(groups[gi], p, &part.warps, part.shape.qpw, s);
+    bdl_knn_plan::Part part{d, (int)groups[gi].size(), 0, p, stats, F[0]->knn_shape,
+                            !stats && knn_by_warp(groups[gi], d, k)};
+    st = upload_knn_table(groups[gi], p, &part.warps, part.by_warp ? 1 : part.shape.qpw, s);
     if (st) return st;
     p += a256(knn_table_bytes_always(groups[gi]));
     P->parts.push_back(part);
@@ -1561,7 +1563,9 @@ static int knn_plan_launch(bdl_knn_plan *P, cudaStream_t s) {
       return set_error(BDL_EINVAL, "a forest changed since the k-NN plan was made");
   for (auto &so : P->sorts) launch_query_sort(so.q, so.m, so.dim, so.scratch, so.perm, s);
   for (auto &part : P->parts) {
-    const int st = launch_knn_table(part.table, part.njobs, part.warps, part.dim, P->k, part.shape, part.stats, s);
+    const int st = part.by_warp
+                       ? launch_knn_warp_table(part.table, part.njobs, part.warps, part.dim, P->k, s)
+                       : launch_knn_table(part.table, part.njobs, part.warps, part.dim, P->k, part.shape, part.stats, s);
     if (st) return st;
   }
   return BDL_OK;

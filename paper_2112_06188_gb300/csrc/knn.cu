@@ -1,5 +1,7 @@
 // knn.cu -- kNN_L (Alg. 5): exact k nearest neighbours of a batch of queries
-// over every static tree (largest first, Sec. V-B) and the buffer.
+// over every static tree (largest first, Sec. V-B) and the buffer: the
+// thread-per-query kernel, for large batches in low dimensions (knn_by_warp;
+// the others go to knn_warp.cu), the packed records and the query order.
 //
 // GPU design:
 //  * One thread per query walks the trees one after another with its own
@@ -205,8 +207,8 @@ template <int D, class TK>
 __device__ __forceinline__ void walk_packed(const KnnJob &J, const TreeView &T, bool active,
                                             const int32_t *q, int dim, int k, TK &best,
                                             uint64_t *stk) {
-  const int rec = packed_node_ints(dim);
-  const int rs = rec_ints(dim);
+  constexpr int rec = packed_node_ints(D);
+  constexpr int rs = rec_ints(D);
   const float kInf = __int_as_float(0x7f800000);
   unsigned long long unused = 0;
   int sp = 0;
@@ -249,12 +251,13 @@ __device__ __forceinline__ void walk_packed(const KnnJob &J, const TreeView &T, 
       atomicOr(J.err, code >= nrec ? kErrChild : kErrStack);
     } else {
       const int32_t *r = T.pk + (int64_t)code * rec;
-      const int4 cd = *reinterpret_cast<const int4 *>(r);
-      const int4 lv = *reinterpret_cast<const int4 *>(r + 4);
+      int4 cd, lv;
       float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;   // box distances (see box_dist_f)
+      if constexpr (!packed_by_entry(D)) {
+        cd = *reinterpret_cast<const int4 *>(r);
+        lv = *reinterpret_cast<const int4 *>(r + 4);
 #pragma unroll
-      for (int c = 0; c < (D ? D : kMaxDim); ++c) {
-        if (c < dim) {
+        for (int c = 0; c < D; ++c) {
           const int4 lo = *reinterpret_cast<const int4 *>(r + 8 + 8 * c);
           const int4 hi = *reinterpret_cast<const int4 *>(r + 12 + 8 * c);
           const int32_t x = q[c];
@@ -268,6 +271,32 @@ __device__ __forceinline__ void walk_packed(const KnnJob &J, const TreeView &T, 
           s2 = fmaf(g2, g2, s2);
           s3 = fmaf(g3, g3, s3);
         }
+      } else {
+        int32_t v[8 + 8 * D];
+#pragma unroll
+        for (int i = 0; i < 8 + 8 * D; i += 4) {
+          const int4 w = *reinterpret_cast<const int4 *>(r + i);
+          v[i] = w.x;
+          v[i + 1] = w.y;
+          v[i + 2] = w.z;
+          v[i + 3] = w.w;
+        }
+        float sv[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+          const int32_t x = q[c] + kBias;
+#pragma unroll
+          for (int a = 0; a < 4; ++a) {
+            const float g = (float)max(max(v[packed_lo_at(D, a, c)] - x, x - v[packed_hi_at(D, a, c)]), 0);
+            sv[a] = fmaf(g, g, sv[a]);
+          }
+        }
+        s0 = sv[0];
+        s1 = sv[1];
+        s2 = sv[2];
+        s3 = sv[3];
+        cd = make_int4(v[packed_code_at(D, 0)], v[packed_code_at(D, 1)], v[packed_code_at(D, 2)], v[packed_code_at(D, 3)]);
+        lv = make_int4(v[packed_live_at(D, 0)], v[packed_live_at(D, 1)], v[packed_live_at(D, 2)], v[packed_live_at(D, 3)]);
       }
       // entries without live points (and the two unused ones of an odd
       // tree's root) are never visited
@@ -409,7 +438,7 @@ __device__ __forceinline__ void knn_query(const KnnJob &J, const TreeView *trees
     }
     const TreeView &T = *tp;
     if (T.live[0] <= 0) continue;
-    if (STATS) walk_nodes<D>(J, T, q, dim, k, best, stk, nvisit, npts);
+    if constexpr (STATS) walk_nodes<D>(J, T, q, dim, k, best, stk, nvisit, npts);
     else walk_packed<D>(J, T, active, q, dim, k, best, stk);
   }
   if (!active) return;
@@ -468,13 +497,7 @@ __global__ void __launch_bounds__(GEN ? kKnnMaxThreads : kKnnThreads, GEN ? 6 : 
   }
 }
 
-// One forest: its job and tree views travel as kernel parameters, read
-// through the constant cache (the per-tree fields are warp-uniform).
-struct KnnOne {
-  KnnJob job;
-  TreeView trees[kMaxLevel];
-};
-
+// One forest: its job and tree views travel as kernel parameters.
 template <int D, bool STATS, bool GEN>
 __global__ void __launch_bounds__(GEN ? kKnnMaxThreads : kKnnThreads, GEN ? 6 : 12)
     k_knn_one(const __grid_constant__ KnnOne P, int k, int qpw, unsigned long long *stats) {
@@ -499,7 +522,10 @@ int knn_block_for(const KnnShape &sh, int k) {
   return b;
 }
 
-template <int D>
+// The timed instances exist for dim 1 .. 7 (higher dimensions always take the
+// warp-per-query kernel, see knn_by_warp); the counting ones for 2, 3, 5, 7
+// and any (0).
+template <int D, bool STATS>
 void launch_d(const KnnJob *jobs, const int64_t *job_warp, int njobs, int64_t warps, int k,
               const KnnShape &sh, unsigned long long *stats, cudaStream_t s) {
   const int bt = knn_block_for(sh, k);
@@ -507,32 +533,26 @@ void launch_d(const KnnJob *jobs, const int64_t *job_warp, int njobs, int64_t wa
   const unsigned grid = (unsigned)((warps * 32 + bt - 1) / bt);
   const bool gen = bt != kKnnThreads || sh.qpw != 32;
   void (*fn)(const KnnJob *, const int64_t *, int, int, int, unsigned long long *) =
-      stats ? (gen ? k_knn<D, true, true> : k_knn<D, true, false>)
-            : (gen ? k_knn<D, false, true> : k_knn<D, false, false>);
+      gen ? k_knn<D, STATS, true> : k_knn<D, STATS, false>;
   // the kernel's own shared memory (the warps' job and tree slots) comes on
   // top of the top-k slots: past the default 48 KB per block (k = 32 at 128
   // threads) the launch needs the opt-in
   if (smem > 40 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  KScope ks_(stats ? kK_knn_count : kK_knn, s);
+  KScope ks_(STATS ? kK_knn_count : kK_knn, s);
   fn<<<grid, bt, smem, s>>>(jobs, job_warp, njobs, k, sh.qpw, stats);
 }
 
-template <int D>
+template <int D, bool STATS>
 void launch_one(const KnnOne &P, int k, const KnnShape &sh, unsigned long long *stats, cudaStream_t s) {
   const int bt = knn_block_for(sh, k);
   const size_t smem = (size_t)k * bt * 12;
-  KScope ks_(stats ? kK_knn_count : kK_knn, s);
+  KScope ks_(STATS ? kK_knn_count : kK_knn, s);
   const int64_t warps = (P.job.m + sh.qpw - 1) / sh.qpw;
   const unsigned grid = (unsigned)((warps * 32 + bt - 1) / bt);
-  const bool gen = bt != kKnnThreads || sh.qpw != 32;
-  if (stats && gen)
-    k_knn_one<D, true, true><<<grid, bt, smem, s>>>(P, k, sh.qpw, stats);
-  else if (stats)
-    k_knn_one<D, true, false><<<grid, bt, smem, s>>>(P, k, sh.qpw, stats);
-  else if (gen)
-    k_knn_one<D, false, true><<<grid, bt, smem, s>>>(P, k, sh.qpw, stats);
+  if (bt != kKnnThreads || sh.qpw != 32)
+    k_knn_one<D, STATS, true><<<grid, bt, smem, s>>>(P, k, sh.qpw, stats);
   else
-    k_knn_one<D, false, false><<<grid, bt, smem, s>>>(P, k, sh.qpw, stats);
+    k_knn_one<D, STATS, false><<<grid, bt, smem, s>>>(P, k, sh.qpw, stats);
 }
 
 // ---------------------------------------------------------------------------
@@ -565,11 +585,12 @@ __global__ void k_pack_nodes(const TreeSeg *segs, const int64_t *pre, int nseg) 
       lv = live[v];
       bx = box + v * 2 * dim;
     }
-    r[a] = code;
-    r[4 + a] = lv;
+    r[packed_code_at(dim, a)] = code;
+    r[packed_live_at(dim, a)] = lv;
+    const uint32_t bias = packed_by_entry(dim) ? kBias : 0;
     for (int c = 0; c < dim; ++c) {
-      r[8 + 8 * c + a] = bx ? bx[c] : INT32_MAX;
-      r[12 + 8 * c + a] = bx ? bx[dim + c] : INT32_MIN;
+      r[packed_lo_at(dim, a, c)] = bx ? (int32_t)((uint32_t)bx[c] + bias) : INT32_MAX;
+      r[packed_hi_at(dim, a, c)] = bx ? (int32_t)((uint32_t)bx[dim + c] + bias) : INT32_MIN;
     }
   }
 }
@@ -773,6 +794,15 @@ size_t batch_query_sort_bytes(const std::vector<KnnCall> &calls) {
          ((size_t)nb * 4 + 255) / 256 * 256 + ((size_t)n * 8 + 255) / 256 * 256 + (size_t)(n + 1) * 8 + 256;
 }
 
+bool knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k) {
+  int64_t m = 0, n = 0;
+  for (const auto &c : calls) {
+    m += c.m;
+    for (int t = 0; t < c.fv->ntrees; ++t) n += c.fv->tree[t].size;
+  }
+  return knn_by_warp(dim, k, m, n);
+}
+
 size_t knn_table_bytes(const std::vector<KnnCall> &calls) {
   if (calls.size() == 1) return 0;   // one forest: no table (kernel parameters)
   return knn_table_bytes_always(calls);
@@ -823,12 +853,25 @@ int launch_knn_table(const void *table, int njobs, int64_t warps, int dim, int k
   if (warps == 0) return BDL_OK;
   const KnnJob *dj = (const KnnJob *)table;
   const int64_t *dw = (const int64_t *)((const char *)table + njobs * sizeof(KnnJob));
+  if (!stats) {
+    switch (dim) {
+      case 1: launch_d<1, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
+      case 2: launch_d<2, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
+      case 3: launch_d<3, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
+      case 4: launch_d<4, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
+      case 5: launch_d<5, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
+      case 6: launch_d<6, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
+      case 7: launch_d<7, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
+      default: return set_error(BDL_EINTERNAL, "no thread-per-query k-NN kernel for this dimension");
+    }
+    return cuda_check(cudaGetLastError(), "knn kernel");
+  }
   switch (dim) {
-    case 2: launch_d<2>(dj, dw, njobs, warps, k, sh, stats, s); break;
-    case 3: launch_d<3>(dj, dw, njobs, warps, k, sh, stats, s); break;
-    case 5: launch_d<5>(dj, dw, njobs, warps, k, sh, stats, s); break;
-    case 7: launch_d<7>(dj, dw, njobs, warps, k, sh, stats, s); break;
-    default: launch_d<0>(dj, dw, njobs, warps, k, sh, stats, s); break;
+    case 2: launch_d<2, true>(dj, dw, njobs, warps, k, sh, stats, s); break;
+    case 3: launch_d<3, true>(dj, dw, njobs, warps, k, sh, stats, s); break;
+    case 5: launch_d<5, true>(dj, dw, njobs, warps, k, sh, stats, s); break;
+    case 7: launch_d<7, true>(dj, dw, njobs, warps, k, sh, stats, s); break;
+    default: launch_d<0, true>(dj, dw, njobs, warps, k, sh, stats, s); break;
   }
   return cuda_check(cudaGetLastError(), "knn kernel");
 }
@@ -853,18 +896,34 @@ int launch_knn_jobs(const std::vector<KnnCall> &calls, int dim, int k, const Knn
     P.job.oi = c.oi;
     P.job.od = c.od;
     for (int t = 0; t < c.fv->ntrees; ++t) P.trees[t] = c.fv->tree[t];
+    if (!stats && knn_by_warp(calls, dim, k)) return launch_knn_warp_one(P, dim, k, s);
+    if (!stats) {
+      switch (dim) {
+        case 1: launch_one<1, false>(P, k, sh, stats, s); break;
+        case 2: launch_one<2, false>(P, k, sh, stats, s); break;
+        case 3: launch_one<3, false>(P, k, sh, stats, s); break;
+        case 4: launch_one<4, false>(P, k, sh, stats, s); break;
+        case 5: launch_one<5, false>(P, k, sh, stats, s); break;
+        case 6: launch_one<6, false>(P, k, sh, stats, s); break;
+        case 7: launch_one<7, false>(P, k, sh, stats, s); break;
+        default: return set_error(BDL_EINTERNAL, "no thread-per-query k-NN kernel for this dimension");
+      }
+      return cuda_check(cudaGetLastError(), "knn kernel");
+    }
     switch (dim) {
-      case 2: launch_one<2>(P, k, sh, stats, s); break;
-      case 3: launch_one<3>(P, k, sh, stats, s); break;
-      case 5: launch_one<5>(P, k, sh, stats, s); break;
-      case 7: launch_one<7>(P, k, sh, stats, s); break;
-      default: launch_one<0>(P, k, sh, stats, s); break;
+      case 2: launch_one<2, true>(P, k, sh, stats, s); break;
+      case 3: launch_one<3, true>(P, k, sh, stats, s); break;
+      case 5: launch_one<5, true>(P, k, sh, stats, s); break;
+      case 7: launch_one<7, true>(P, k, sh, stats, s); break;
+      default: launch_one<0, true>(P, k, sh, stats, s); break;
     }
     return cuda_check(cudaGetLastError(), "knn kernel");
   }
   int64_t warps = 0;
-  int st = upload_knn_table(calls, table, &warps, sh.qpw, s);
+  const bool by_warp = !stats && knn_by_warp(calls, dim, k);
+  int st = upload_knn_table(calls, table, &warps, by_warp ? 1 : sh.qpw, s);
   if (st) return st;
+  if (by_warp) return launch_knn_warp_table(table, (int)n, warps, dim, k, s);
   return launch_knn_table(table, (int)n, warps, dim, k, sh, stats, s);
 }
 

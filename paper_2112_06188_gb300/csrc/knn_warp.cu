@@ -1,0 +1,513 @@
+// knn_warp.cu -- kNN_L (Alg. 5) with one warp per query.
+//
+// The thread-per-query kernel (knn.cu) walks one query's tree nodes and leaf
+// points one after another in one lane: a small batch leaves most of the GPU
+// idle and waits for the longest such chain.  Here the 32 lanes of a warp work
+// on one query together:
+//  * a node round takes up to eight records off the query's stack at once and
+//    gives each of their 32 entries to a lane (box distance, prune test);
+//  * a leaf round gives 32 leaf points, of up to four leaves, a lane each;
+//  * the k <= 32 best candidates live in registers, lane i holding the i-th
+//    best; a few candidates enter one by one by a ballot (the rank) and a
+//    shift, more than ten are sorted across the warp and merged;
+//  * all trees of the forest are walked together: the stack starts with every
+//    tree's root, the largest tree's on top, and an entry names its tree.
+// The answer does not depend on the order of the walk: every subtree whose
+// box is not strictly farther than the k-th distance is visited, and the k
+// best by (d2, id) of all points seen are unique.
+//
+// What bounds it: small batches by the chain of about 2 x 20 rounds per query
+// (a dependent L2 read each); large ones by instruction issue (about 3,900
+// warp instructions per query on 2M 3-D points, 10,000 on 2M 7-D ones, 65 to
+// 78% of the issue slots) and by the shared/L1 data pipe (53 to 67%).
+// Measured against the thread-per-query kernel (1M 5-D points, k = 10, 316
+// queries: 1,014 -> 51 us; 50K 16-D points, k = 8, 1,000 queries: 1,495 -> 59;
+// 500K 4-D points, k = 32, 100K queries: 3,620 -> 850; 10M 7-D points of 100
+// clusters, k = 5, 1M queries: 31.4 -> 20.4 ms).
+#include "bdl_internal.cuh"
+
+#include <algorithm>
+
+namespace bdl {
+
+namespace {
+
+constexpr int kWarpsPerBlock = 4;
+constexpr int kWStack = 256;    // node stack entries per warp
+constexpr int kWLeaves = 80;    // leaf stack entries per warp
+constexpr int kWTrees = kMaxLevel + 1;
+// Past this depth records are taken one at a time, each adding at most three
+// entries per 4-ary level (14 levels): 190 + 24 + 42 <= kWStack.
+constexpr int kWWide = 190;
+constexpr float kWBoundUp = 1.00000393390655517578125f;   // see TopK in knn.cu
+
+// What a walk needs of a tree.
+struct WTree {
+  const int32_t *pk, *pts, *leaf_off;
+  int64_t size;
+  int32_t nrec, nleaf;
+};
+
+struct __align__(16) WarpMem {
+  int32_t q[kMaxDim];        // the query
+  uint64_t node[kWStack];    // (box distance bits, low 6 bits: tree) << 32 | record
+  uint64_t leaf[kWLeaves];   // (box distance bits, low 6 bits: tree) << 32 | leaf
+  uint64_t sel[8];           // the records of this round
+};
+
+// The k best candidates, lane i holding the i-th of the best 32.
+struct WarpTop {
+  uint64_t d;
+  int32_t id;
+  float kdf;       // pruning bound: k-th distance rounded up, scaled up (see box_dist_f in knn.cu)
+  uint64_t kd;     // k-th pair
+  int32_t kid;
+};
+
+__device__ __forceinline__ void top_bound(WarpTop &b, int k) {
+  b.kd = __shfl_sync(0xffffffffu, b.d, k - 1);
+  b.kid = __shfl_sync(0xffffffffu, b.id, k - 1);
+  b.kdf = b.kd == ~0ull ? __int_as_float(0x7f800000) : __fmul_ru(__ull2float_ru(b.kd), kWBoundUp);
+}
+
+__device__ __forceinline__ bool pair_less(uint64_t d, int32_t i, uint64_t e, int32_t j) {
+  return d < e || (d == e && i < j);
+}
+
+// The candidates (d, id) of the lanes with `have` join the list.
+__device__ __forceinline__ void top_add(WarpTop &b, int k, bool have, uint64_t d, int32_t id) {
+  const int lane = threadIdx.x & 31;
+  unsigned mask = __ballot_sync(0xffffffffu, have);
+  if (!mask) return;
+  if (__popc(mask) > 10) {
+    // many at once: sort them across the warp, then merge the two sorted
+    // lists (the smaller of element i and element 31 - i, a bitonic sequence)
+    const bool empty = __shfl_sync(0xffffffffu, b.d, 0) == ~0ull;
+    if (!have) {
+      d = ~0ull;
+      id = INT32_MAX;
+    }
+#pragma unroll
+    for (int size = 2; size <= 64; size <<= 1) {
+      if (size == 64) {
+        if (empty) break;
+        const uint64_t rd = __shfl_xor_sync(0xffffffffu, d, 31);
+        const int32_t ri = __shfl_xor_sync(0xffffffffu, id, 31);
+        const bool mine = pair_less(b.d, b.id, rd, ri);
+        d = mine ? b.d : rd;
+        id = mine ? b.id : ri;
+      }
+#pragma unroll
+      for (int stride = size == 64 ? 16 : size >> 1; stride > 0; stride >>= 1) {
+        const uint64_t od = __shfl_xor_sync(0xffffffffu, d, stride);
+        const int32_t oi = __shfl_xor_sync(0xffffffffu, id, stride);
+        const bool up = size >= 32 || (lane & size) == 0;
+        const bool keep_min = ((lane & stride) == 0) == up;
+        if (pair_less(od, oi, d, id) == keep_min) {
+          d = od;
+          id = oi;
+        }
+      }
+    }
+    b.d = d;
+    b.id = id;
+  } else {
+    do {
+      const int src = __ffs(mask) - 1;
+      mask &= mask - 1;
+      const uint64_t cd = __shfl_sync(0xffffffffu, d, src);
+      const int32_t ci = __shfl_sync(0xffffffffu, id, src);
+      const bool less = pair_less(b.d, b.id, cd, ci);
+      const int pos = __popc(__ballot_sync(0xffffffffu, less));
+      const uint64_t ud = __shfl_up_sync(0xffffffffu, b.d, 1);
+      const int32_t ui = __shfl_up_sync(0xffffffffu, b.id, 1);
+      if (!less) {
+        b.d = lane == pos ? cd : ud;
+        b.id = lane == pos ? ci : ui;
+      }
+    } while (mask);
+  }
+  top_bound(b, k);
+}
+
+// Query row qi of job J against the nt trees of the table (smallest first),
+// whose views are views[nt - 1 .. 0], then the buffer.  Called by a whole warp.
+template <int D>
+__device__ __forceinline__ void warp_query(const KnnJob &J, WarpMem &W, const WTree *tree, int nt,
+                                           const TreeView *views, int64_t qi, int k) {
+  constexpr int DM = D ? D : kMaxDim;
+  const int dim = D ? D : J.dim;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1;
+  const float kInf = __int_as_float(0x7f800000);
+  __syncwarp();
+  if (lane < dim) W.q[lane] = J.q[qi * dim + lane];
+  __syncwarp();
+  // the query as floats 2^23 + x, exact on the grid and well beyond it
+  float q[DM];
+#pragma unroll
+  for (int c = 0; c < DM; ++c)
+    if (c < dim) q[c] = (float)W.q[c] + kBiasF;
+  WarpTop best;
+  best.d = ~0ull;
+  best.id = INT32_MAX;
+  best.kd = ~0ull;
+  best.kid = INT32_MAX;
+  best.kdf = kInf;
+  int sp = 0, ls = 0;
+  // the roots, largest tree last (on top)
+  for (int b = 0; b < nt; b += 32) {
+    const int ti = b + lane;
+    bool ok = ti < nt;
+    float s = 0.f;
+    bool leaf = false;
+    if (ok) {
+      const TreeView &V = views[nt - 1 - ti];
+      leaf = V.h == 0;
+      ok = V.live[0] > 0;
+#pragma unroll
+      for (int c = 0; c < DM; ++c)
+        if (c < dim) {
+          const float lo = (float)V.box[c] + kBiasF, hi = (float)V.box[dim + c] + kBiasF;
+          const float g = fmaxf(fmaxf(lo - q[c], q[c] - hi), 0.f);
+          s = fmaf(g, g, s);
+        }
+    }
+    const uint64_t e = ((uint64_t)((__float_as_uint(s) & ~63u) | (unsigned)ti) << 32);
+    const unsigned nm = __ballot_sync(0xffffffffu, ok && !leaf), lm = __ballot_sync(0xffffffffu, ok && leaf);
+    if (ok && !leaf) W.node[sp + __popc(nm & lt)] = e;
+    if (ok && leaf) W.leaf[ls + __popc(lm & lt)] = e;
+    sp += __popc(nm);
+    ls += __popc(lm);
+  }
+  __syncwarp();
+  const int rs = rec_ints(dim), rec = packed_node_ints(dim);
+  while (sp > 0 || ls > 0) {
+    // ---- leaf rounds: the points of up to four leaves, 32 at a time ----
+    while (ls >= 2 || (sp == 0 && ls > 0)) {
+      const int nl = min(ls, 4);
+      uint32_t key = 0;    // box distance bits, low 6 bits: tree
+      int pa = 0, n = 0;
+      if (lane < nl) {
+        const uint64_t e = W.leaf[ls - 1 - lane];
+        key = (uint32_t)(e >> 32);
+        if (!(__uint_as_float(key & ~63u) > best.kdf)) {
+          const WTree &T = tree[key & 63u];
+          const uint32_t lf = (uint32_t)e;
+          int pz = 0;
+          unsigned long long bad = kErrChild;
+          if (lf < (uint32_t)T.nleaf) {
+            pa = T.leaf_off[lf];
+            pz = T.leaf_off[lf + 1];
+            bad = pa < 0 || pz > T.size || pa > pz ? kErrLeaf : 0;
+          }
+          if (bad) atomicOr(J.err, bad);
+          else n = pz - pa;
+        }
+      }
+      ls -= nl;
+      // each leaf's first place among the round's points
+      int inc = n;
+      int y = __shfl_up_sync(0xffffffffu, inc, 1);
+      if (lane >= 1) inc += y;
+      y = __shfl_up_sync(0xffffffffu, inc, 2);
+      if (lane >= 2) inc += y;
+      const int total = __shfl_sync(0xffffffffu, inc, 3);
+      const int start = inc - n;
+      const int s1 = __shfl_sync(0xffffffffu, start, 1);
+      const int s2 = __shfl_sync(0xffffffffu, start, 2);
+      const int s3 = __shfl_sync(0xffffffffu, start, 3);
+      const int off = pa - start;
+      for (int b = 0; b < total; b += 32) {
+        const int x = b + lane;
+        const int own = (x >= s1) + (x >= s2) + (x >= s3);
+        const int po = __shfl_sync(0xffffffffu, off, own) + x;
+        const uint32_t pk = __shfl_sync(0xffffffffu, key, own);
+        bool have = false;
+        uint64_t s = 0;
+        int32_t id = 0;
+        if (x < total && !(__uint_as_float(pk & ~63u) > best.kdf)) {
+          const int32_t *src = tree[pk & 63u].pts + (int64_t)po * rs;
+          int32_t p[D ? rec_ints(D) : rec_ints(kMaxDim)];
+#pragma unroll
+          for (int c4 = 0; c4 < (D ? rec_ints(D) : rec_ints(kMaxDim)); c4 += 4)
+            if (c4 < rs) {
+              const int4 v = *reinterpret_cast<const int4 *>(src + c4);
+              p[c4] = v.x;
+              p[c4 + 1] = v.y;
+              p[c4 + 2] = v.z;
+              p[c4 + 3] = v.w;
+            }
+          id = D ? p[D ? D : 0] : src[dim];
+          float sf = 0.f;
+#pragma unroll
+          for (int c = 0; c < DM; ++c)
+            if (c < dim) {
+              const float g = q[c] - __int_as_float(p[c] | kBias);
+              sf = fmaf(g, g, sf);
+            }
+          if (!(sf > best.kdf) && id >= 0) {
+#pragma unroll
+            for (int c4 = 0; c4 < DM; c4 += 4) {
+              const int4 x4 = *reinterpret_cast<const int4 *>(W.q + c4);
+              const int32_t xq[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                if (c4 + e < DM && c4 + e < dim) {
+                  const int32_t g = xq[e] - p[c4 + e];
+                  s += (uint64_t)((int64_t)g * g);
+                }
+            }
+            have = pair_less(s, id, best.kd, best.kid);
+          }
+        }
+        top_add(best, k, have, s, id);
+      }
+    }
+    if (sp == 0) continue;
+    // ---- node round: the entries of up to eight records ----
+    const int win = min(sp, 32);
+    const uint64_t e0 = lane < win ? W.node[sp - 1 - lane] : 0;
+    const bool ok0 = lane < win && !(__uint_as_float((uint32_t)(e0 >> 32) & ~63u) > best.kdf);
+    const unsigned om = __ballot_sync(0xffffffffu, ok0);
+    const int ord = __popc(om & lt);
+    const bool tk0 = ok0 && ord < (sp > kWWide ? 1 : 8);
+    if (tk0) W.sel[ord] = e0;
+    const unsigned tk = __ballot_sync(0xffffffffu, tk0);
+    // what leaves the stack: the records taken and the pruned ones above them
+    sp -= tk == om ? win : 32 - __clz(tk);
+    if (tk == 0) continue;
+    __syncwarp();
+    const int r = lane >> 2, a = lane & 3;
+    uint32_t b = 0x7f800000u | a;   // box distance bits, low 2 bits: the entry's number
+    int32_t code = 0;
+    uint32_t tr = 0;
+    if (r < __popc(tk)) {
+      const uint64_t e = W.sel[r];
+      tr = (uint32_t)(e >> 32) & 63u;
+      const WTree &T = tree[tr];
+      if ((uint32_t)e >= (uint32_t)T.nrec) {
+        atomicOr(J.err, kErrChild);
+      } else {
+        const int32_t *rp = T.pk + (int64_t)(uint32_t)e * rec;
+        float s = 0.f;
+        int32_t lv;
+        auto gap = [&](int c, float lo, float hi) {
+          const float g = fmaxf(fmaxf(lo - q[c], q[c] - hi), 0.f);
+          s = fmaf(g, g, s);
+        };
+        if (D && !packed_by_entry(D)) {
+          code = rp[packed_code_at(D, a)];
+          lv = rp[packed_live_at(D, a)];
+#pragma unroll
+          for (int c = 0; c < DM; ++c)
+            gap(c, __int_as_float(rp[packed_lo_at(D, a, c)] | kBias), __int_as_float(rp[packed_hi_at(D, a, c)] | kBias));
+        } else if (dim & 1) {
+          const int4 w0 = *reinterpret_cast<const int4 *>(rp + packed_quad_at(a, 0));
+          code = w0.x;
+          lv = w0.y;
+          gap(0, __int_as_float(w0.z), __int_as_float(w0.w));
+#pragma unroll
+          for (int c = 1; c + 1 < DM; c += 2)
+            if (c < dim) {
+              const float4 w = *reinterpret_cast<const float4 *>(rp + packed_quad_at(a, 2 + 2 * c));
+              gap(c, w.x, w.y);
+              gap(c + 1, w.z, w.w);
+            }
+        } else {
+          const int2 cl = *reinterpret_cast<const int2 *>(rp + packed_code_at(dim, a));
+          code = cl.x;
+          lv = cl.y;
+#pragma unroll
+          for (int c = 0; c + 1 < DM; c += 2)
+            if (c < dim) {
+              const float4 w = *reinterpret_cast<const float4 *>(rp + packed_quad_at(a, 2 * c));
+              gap(c, w.x, w.y);
+              gap(c + 1, w.z, w.w);
+            }
+        }
+        if (lv > 0 && !(s > best.kdf)) b = (__float_as_uint(s) & ~3u) | a;
+      }
+    }
+    // the entries that stay go onto their stack, the nearest of a record
+    // last, the record nearest the old stack's top last of all
+    const uint32_t b1 = __shfl_xor_sync(0xffffffffu, b, 1), b2 = __shfl_xor_sync(0xffffffffu, b, 2),
+                   b3 = __shfl_xor_sync(0xffffffffu, b, 3);
+    const int near = (b1 < b) + (b2 < b) + (b3 < b);   // entries that do not stay compare greater
+    const bool in = b < 0x7f800000u;
+    const unsigned nm = __ballot_sync(0xffffffffu, in && code >= 0);
+    const unsigned lm = __ballot_sync(0xffffffffu, in && code < 0);
+    const unsigned from = 0xffffffffu << (lane & ~3);   // this record's lanes and those taken after it
+    const uint64_t e = ((uint64_t)((b & ~63u) | tr) << 32) | (uint32_t)(code < 0 ? ~code : code);
+    if (in) {
+      uint64_t *dst = code < 0 ? &W.leaf[ls + __popc(lm & from)] : &W.node[sp + __popc(nm & from)];
+      dst[-1 - near] = e;
+    }
+    sp += __popc(nm);
+    ls += __popc(lm);
+    __syncwarp();
+  }
+  // the buffer's points, where they have no tree
+  for (int64_t b = 0; b < J.nbuf; b += 32) {
+    const int64_t j = b + lane;
+    bool have = false;
+    uint64_t s = 0;
+    int32_t id = 0;
+    if (j < J.nbuf) {
+      id = J.buf[j];
+      const int32_t *p = J.idtab + (int64_t)id * dim;
+      for (int c = 0; c < dim; ++c) {
+        const int32_t g = W.q[c] - p[c];
+        s += (uint64_t)((int64_t)g * g);
+      }
+      have = pair_less(s, id, best.kd, best.kid);
+    }
+    top_add(best, k, have, s, id);
+  }
+  if (lane < k) {
+    const bool ok = best.d != ~0ull;
+    J.oi[qi * k + lane] = ok ? best.id : -1;
+    J.od[qi * k + lane] = ok ? (int64_t)best.d : INT64_MAX;
+  }
+}
+
+// The walk's tree table (smallest tree first) from the nt views.
+__device__ __forceinline__ void fill_trees(WTree *tree, const TreeView *views, int nt, int at, int step) {
+  for (int ti = at; ti < nt; ti += step) {
+    const TreeView &V = views[nt - 1 - ti];
+    WTree w;
+    w.pk = V.pk;
+    w.pts = V.pts;
+    w.leaf_off = V.leaf_off;
+    w.size = V.size;
+    w.nrec = (int32_t)packed_nrec(V.h);
+    w.nleaf = (int32_t)((int64_t)1 << V.h);
+    tree[ti] = w;
+  }
+}
+
+// One forest: every warp answers `per` consecutive queries of the processing
+// order.
+template <int D>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+    k_knn_warp_one(const __grid_constant__ KnnOne P, int k, int per) {
+  __shared__ WarpMem W[kWarpsPerBlock];
+  __shared__ WTree tree[kWTrees];
+  fill_trees(tree, P.trees, P.job.ntrees, threadIdx.x, blockDim.x);
+  __syncthreads();
+  const int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
+  const int64_t t1 = min(t0 + per, P.job.m);
+  for (int64_t t = t0; t < t1; ++t)
+    warp_query<D>(P.job, W[threadIdx.x >> 5], tree, P.job.ntrees, P.trees, P.job.perm ? P.job.perm[t] : t, k);
+}
+
+// Many forests: warp w answers query w - job_warp[j] of its job j.
+template <int D>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+    k_knn_warp(const KnnJob *jobs, const int64_t *job_warp, int njobs, int k) {
+  __shared__ WarpMem W[kWarpsPerBlock];
+  __shared__ WTree tree[kWarpsPerBlock][kWTrees];
+  __shared__ KnnJob s_job[kWarpsPerBlock];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= job_warp[njobs]) return;
+  int lo = 0, hi = njobs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (job_warp[mid] <= w) lo = mid;
+    else hi = mid - 1;
+  }
+  KnnJob &J = s_job[warp];
+  if (lane == 0) J = jobs[lo];
+  __syncwarp();
+  const int64_t t = w - job_warp[lo];
+  fill_trees(tree[warp], J.trees, J.ntrees, lane, 32);
+  __syncwarp();
+  warp_query<D>(J, W[warp], tree[warp], J.ntrees, J.trees, J.perm ? J.perm[t] : t, k);
+}
+
+template <int D>
+void warp_one(const KnnOne &P, int k, cudaStream_t s) {
+  // up to eight neighbouring queries per warp, which find their paths in L1
+  // (10M 7-D points, 1M queries: 23.5 -> 21.5 ms), while that leaves about six
+  // times the warps the GPU can hold
+  const int per = (int)std::min<int64_t>(8, std::max<int64_t>(1, P.job.m / 30000));
+  const int64_t blk = (int64_t)kWarpsPerBlock * per;
+  KScope ks_(kK_knn, s);
+  k_knn_warp_one<D><<<(unsigned)((P.job.m + blk - 1) / blk), kWarpsPerBlock * 32, 0, s>>>(P, k, per);
+}
+
+template <int D>
+void warp_table(const KnnJob *jobs, const int64_t *job_warp, int njobs, int64_t warps, int k, cudaStream_t s) {
+  KScope ks_(kK_knn, s);
+  k_knn_warp<D><<<(unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock), kWarpsPerBlock * 32, 0, s>>>(
+      jobs, job_warp, njobs, k);
+}
+
+}  // namespace
+
+// Where the two kernels cost the same.  The warp-per-query kernel's time grows
+// with the queries (3 to 20 ns each) from a few dozen microseconds; the
+// thread-per-query kernel's stays near that of its slowest warps until about
+// 130,000 queries fill the GPU, and then grows more slowly in low dimensions
+// (neighbouring queries share their walk) and for small k (its top-k lists
+// take 12 k bytes of shared memory per thread: past k = 16 they cost it
+// resident warps).  Measured for n = 10^4 .. 10^7 points, uniform and
+// clustered; thread / warp in us:
+//   dim 1, k = 8:  16K queries 86 / 56, 65K 109 / 215
+//   dim 2, k = 5:  16K 116 / 78, 33K 133 / 159;   k = 32: 131K 867 / 764
+//   dim 3, k = 1:  16K 126 / 77, 33K 125 / 158;   k = 10: 33K 325 / 203, 66K 328 / 369
+//          k = 24: 262K 1719 / 1734;              k = 32: 1M 7885 / 7074
+//   dim 4, k = 1:  66K 400 / 293, 131K 468 / 542; k = 10: 262K 1696 / 1611
+//   dim 5, k = 1:  262K 1095 / 1091;              k = 10: 1M 8569 / 7992
+//   dim 6, k = 1:  262K 2128 / 1233, 1M 3313 / 4229; k = 10: 1M 11838 / 11479
+//   dim 7, k = 1:  1M queries on 100K points 4350 / 4399 (clusters 2503 / 3404),
+//                  on 10M 11182 / 7054;           k = 5: 1M on 1M 20953 / 12524
+bool knn_by_warp(int dim, int k, int64_t m, int64_t n) {
+  struct Line {
+    double base, slope;   // k <= 16: most queries (thousands) = base + slope k
+    double k24, k32;      // for k = 17 .. 24 and above
+  };
+  constexpr double kAll = 1e12;
+  static constexpr Line kLine[7] = {{9, 1.8, 52, 67},      {14, 3, 86, 110},        {20, 4.5, 250, 1000},
+                                    {80, 12, 500, kAll},   {140, 40, kAll, kAll},   {250, 70, kAll, kAll},
+                                    {700, 0, kAll, kAll}};
+  if (dim > 7 || (dim == 7 && (k > 2 || m < n))) return true;
+  const Line &L = kLine[dim - 1];
+  return (double)m <= 1e3 * (k <= 16 ? L.base + L.slope * k : k <= 24 ? L.k24 : L.k32);
+}
+
+int launch_knn_warp_one(const KnnOne &P, int dim, int k, cudaStream_t s) {
+  switch (dim) {
+    case 1: warp_one<1>(P, k, s); break;
+    case 2: warp_one<2>(P, k, s); break;
+    case 3: warp_one<3>(P, k, s); break;
+    case 4: warp_one<4>(P, k, s); break;
+    case 5: warp_one<5>(P, k, s); break;
+    case 6: warp_one<6>(P, k, s); break;
+    case 7: warp_one<7>(P, k, s); break;
+    case 8: warp_one<8>(P, k, s); break;
+    default: warp_one<0>(P, k, s); break;
+  }
+  return cuda_check(cudaGetLastError(), "knn kernel");
+}
+
+int launch_knn_warp_table(const void *table, int njobs, int64_t warps, int dim, int k, cudaStream_t s) {
+  if (warps == 0) return BDL_OK;
+  const KnnJob *jobs = (const KnnJob *)table;
+  const int64_t *job_warp = (const int64_t *)((const char *)table + njobs * sizeof(KnnJob));
+  switch (dim) {
+    case 1: warp_table<1>(jobs, job_warp, njobs, warps, k, s); break;
+    case 2: warp_table<2>(jobs, job_warp, njobs, warps, k, s); break;
+    case 3: warp_table<3>(jobs, job_warp, njobs, warps, k, s); break;
+    case 4: warp_table<4>(jobs, job_warp, njobs, warps, k, s); break;
+    case 5: warp_table<5>(jobs, job_warp, njobs, warps, k, s); break;
+    case 6: warp_table<6>(jobs, job_warp, njobs, warps, k, s); break;
+    case 7: warp_table<7>(jobs, job_warp, njobs, warps, k, s); break;
+    case 8: warp_table<8>(jobs, job_warp, njobs, warps, k, s); break;
+    default: warp_table<0>(jobs, job_warp, njobs, warps, k, s); break;
+  }
+  return cuda_check(cudaGetLastError(), "knn kernel");
+}
+
+}  // namespace bdl

@@ -72,6 +72,7 @@ struct Group {
 };
 
 constexpr int64_t kMixQueries = 1 << 15;   // a k-NN run that mixes k stays this small
+constexpr auto kGather = std::chrono::microseconds(300);   // see exec_loop
 
 }  // namespace
 }  // namespace bdl
@@ -92,6 +93,7 @@ struct bdl_server {
   int64_t staged = 0;               // device bytes of admitted requests
   int64_t groups = 0;
   bool stop = false;
+  bdl::Clock::time_point last_knn;  // when the last k-NN group was formed
   std::thread th_admit, th_exec, th_done;
   std::vector<cudaEvent_t> spare_events;
 };
@@ -371,6 +373,23 @@ void run_group(bdl_server *S, Group *g) {
   cudaEventRecord(g->ev_out, S->s_out);
 }
 
+// Whether the execution thread should wait for more k-NN requests to join the
+// next group (caller holds S->mu): every admitted request is a small k-NN one,
+// nothing else is waiting behind them, and some other request has not been
+// collected yet, so that the client is not waiting for these alone.
+bool gather_more(const bdl_server *S) {
+  if (S->stop || S->cfg.serial || S->live.size() <= S->admitted.size()) return false;
+  if (S->inflight >= S->cfg.max_inflight) return false;
+  for (const Req *q : S->submitted)
+    if (q->r.kind != BDL_REQ_KNN) return false;
+  int64_t n = 0;
+  for (const Req *q : S->admitted) {
+    if (q->res.status || q->r.kind != BDL_REQ_KNN) return false;
+    n += q->r.n;
+  }
+  return n < kMixQueries;
+}
+
 void exec_loop(bdl_server *S) {
   cudaSetDevice(S->f->device);
   std::unique_lock<std::mutex> lk(S->mu);
@@ -378,7 +397,15 @@ void exec_loop(bdl_server *S) {
     S->cv_exec.wait(lk, [&] { return !S->admitted.empty() || (S->stop && S->submitted.empty() &&
                                                               S->inflight == 0); });
     if (S->admitted.empty()) return;
+    // A small k-NN group runs for tens of microseconds, about as long as the
+    // host needs to submit one request: launched as they come, the requests
+    // of a burst would run one by one, each paying a group's launches and
+    // copies.  So small k-NN groups are formed at most every kGather; a
+    // request that comes later than that after the last one, or whose client
+    // has nothing else outstanding, goes at once.
+    S->cv_exec.wait_until(lk, S->last_knn + kGather, [&] { return !gather_more(S); });
     Group *g = form_group(S);
+    if (g->reqs[0]->r.kind == BDL_REQ_KNN) S->last_knn = Clock::now();
     lk.unlock();
     run_group(S, g);
     lk.lock();

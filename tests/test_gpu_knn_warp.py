@@ -1,0 +1,116 @@
+"""The k-NN kernel with one warp per query (small batches, high dimensions)
+against brute force, and the thread-per-query kernel (large batches) against
+it, bit for bit: every dimension class, leaf sizes from 2 to 64, k at both
+ends of its range and at a list longer than the live set, duplicates, erased
+points, a part-filled buffer, and leaves far larger than a warp (the spatial
+median on duplicates)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle.threads import bruteforce_knn_threads
+from paper_2112_06188_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2112_06188_gb300 import build_lib
+    build_lib.build()
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def forest_of(dim, n, seed, leaf=16, split="object", distinct=0, X=256):
+    """A forest after a build, an insert and an erase, and its live points."""
+    from paper_2112_06188_gb300.forest import Forest
+    draw = (lambda m, s: inputs.duplicate_heavy_points(m, dim, s, distinct)) if distinct else \
+           (lambda m, s: inputs.uniform_points(m, dim, s))
+    f = Forest(dim, leaf_size=leaf, buffer_size=X, split=split)
+    live = inputs.LiveSet(dim)
+    for m, s in ((n, seed), (n // 7 + 3, seed + 1)):
+        p = draw(m, s)
+        f.insert(dev(p))
+        live.insert(p)
+    gone = inputs.sample_ids(live.live_ids(), len(live.live_ids()) // 9, seed + 2)
+    assert f.erase(dev(gone)) == live.erase(gone)
+    return f, live
+
+
+def check(f, live, q, k):
+    gi, gd = f.knn(dev(q), k)
+    pts, ids = live.live_points()
+    bi, bd = bruteforce_knn_threads(pts, ids, q, k)
+    assert np.array_equal(gd.cpu().numpy(), bd) and np.array_equal(gi.cpu().numpy(), bi)
+    assert f.poll_error() == 0
+
+
+@pytest.mark.parametrize("dim", [1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 16])
+@pytest.mark.parametrize("k", [1, 10, 32])
+def test_dims(dim, k):
+    leaf = {1: 8, 10: 16, 32: 64}[k]
+    f, live = forest_of(dim, 6_000, 40 * dim + k, leaf=leaf)
+    lp, _ = live.live_points()
+    q = np.concatenate([inputs.queries_from(lp, 33, 7), inputs.uniform_points(40, dim, 8)])
+    check(f, live, q, k)
+    check(f, live, q[:1], k)
+    # queries off the grid (the C ABI asks for grid points; nothing depends on it)
+    check(f, live, q[:5] - (1 << 20), k)
+
+
+@pytest.mark.parametrize("dim,distinct", [(2, 3), (3, 1), (5, 40)])
+@pytest.mark.parametrize("split", ["object", "spatial"])
+def test_ties_and_huge_leaves(dim, distinct, split):
+    f, live = forest_of(dim, 4_000, 77, split=split, distinct=distinct)
+    lp, _ = live.live_points()
+    q = np.concatenate([inputs.queries_from(lp, 9, 7), inputs.uniform_points(9, dim, 8)])
+    for k in (1, 32):
+        check(f, live, q, k)
+
+
+def test_padding_and_buffer_only():
+    for n in (5, 40, 300):
+        f, live = forest_of(3, n, 90 + n)
+        check(f, live, inputs.uniform_points(7, 3, 5), 32)
+
+
+def test_deep_trees_with_little_pruning():
+    """Leaves of two points in 16 dimensions: the node stack reaches the depth
+    from which records are taken one at a time."""
+    f, live = forest_of(16, 150_000, 11, leaf=2, X=1024)
+    check(f, live, inputs.uniform_points(3, 16, 12), 32)
+
+
+# just above and below the size from which each dimension takes the
+# thread-per-query kernel (k = 1), with the launch shapes that kernel has
+@pytest.mark.parametrize("dim,m", [(1, 10_700), (2, 16_900), (3, 24_400), (4, 91_900), (5, 179_900), (6, 319_900),
+                                   (7, 699_900)])
+def test_thread_kernel_gives_the_same_rows(dim, m):
+    from paper_2112_06188_gb300.forest import KnnPlan, knn_batch
+    f, live = forest_of(dim, 3_000, 60 + dim)
+    lp, _ = live.live_points()
+    q = dev(np.concatenate([inputs.queries_from(lp, m // 2, 7), inputs.uniform_points(m + 200 - m // 2, dim, 8)]))
+    wi, wd = (torch.cat(x) for x in zip(*(f.knn(c, 1) for c in q.split(5_000))))
+    for n in (m, m + 200):
+        gi, gd = f.knn(q[:n], 1)
+        assert torch.equal(gi, wi[:n]) and torch.equal(gd, wd[:n])
+    half = q.shape[0] // 2
+    for (gi, gd), want in zip(knn_batch([f, f], [q[:half], q[half:]], 1), (slice(0, half), slice(half, None))):
+        assert torch.equal(gi, wi[want]) and torch.equal(gd, wd[want])
+    if dim == 3:
+        for block in (64, 128, 256):
+            for per in (32, 64, 128):
+                f.set_knn_shape(block, per)
+                plan = KnnPlan([f], [q], 1)
+                for gi, gd in (f.knn(q, 1), plan.launch()[0]):
+                    assert torch.equal(gi, wi) and torch.equal(gd, wd)
+                plan.close()
+        wi, wd = (torch.cat(x) for x in zip(*(f.knn(c, 16) for c in q.repeat(4, 1).split(20_000))))
+        gi, gd = f.knn(q.repeat(4, 1), 16)
+        assert torch.equal(gi, wi) and torch.equal(gd, wd)
+    assert f.poll_error() == 0
