@@ -16,6 +16,70 @@ namespace {
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// Leaves of more points than this (only spatial-median trees have them) are
+// scanned by the whole warp.
+constexpr int kLaneLeaf = 64;
+constexpr int kMapWords = 64;   // per warp: 2,048 bits
+
+// The lanes with `big` look for their id among the points [a, z) of tree ti:
+// the lanes that look in one leaf do so together, 32 points at a time, a
+// bitmap of their ids' hashes keeping the points that none of them wants
+// out.  Called by the whole warp; true where a lane's id was found (and
+// tombstoned).  The ids of a spatially ordered list meet in the same leaves:
+// a lane scanning its leaf alone took as long as the largest leaf (1M 2-D
+// points of 100 clusters, 100K ids: 1,065 us for the launch, this way 86).
+__device__ __forceinline__ bool scan_big_leaves(const EraseJob &F, int rs, bool big, int ti, int a, int z,
+                                                int32_t id) {
+  __shared__ uint32_t s_map[4][kMapWords];
+  unsigned todo = __ballot_sync(0xffffffffu, big);
+  if (!todo) return false;
+  const int lane = threadIdx.x & 31;
+  uint32_t *map = s_map[threadIdx.x >> 5];
+  bool hit = false;
+  while (todo) {
+    const int src = __ffs(todo) - 1;
+    const int t = __shfl_sync(0xffffffffu, ti, src), la = __shfl_sync(0xffffffffu, a, src),
+              lz = __shfl_sync(0xffffffffu, z, src);
+    const bool mine = big && ti == t && a == la;
+    const unsigned grp = __ballot_sync(0xffffffffu, mine);
+    todo &= ~grp;
+    auto bit = [](int32_t x) { return ((uint32_t)x * 0x9E3779B1u) >> 21; };
+    map[lane] = 0;
+    map[lane + 32] = 0;
+    __syncwarp();
+    if (mine) atomicOr(&map[bit(id) >> 5], 1u << (bit(id) & 31));
+    __syncwarp();
+    int32_t *pts = F.trees[t].pts + F.dim;
+    int left = __popc(grp);
+    for (int b = la; b < lz && left > 0; b += 128) {
+      int32_t p[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = b + 32 * u + lane;
+        p[u] = j < lz ? pts[(int64_t)j * rs] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool may = p[u] >= 0 && ((map[bit(p[u]) >> 5] >> (bit(p[u]) & 31)) & 1);
+        unsigned cm = __ballot_sync(0xffffffffu, may);
+        while (cm) {
+          const int s = __ffs(cm) - 1;
+          cm &= cm - 1;
+          const int32_t x = __shfl_sync(0xffffffffu, p[u], s);
+          const bool is = mine && id == x;
+          if (__any_sync(0xffffffffu, is)) {
+            if (lane == s) pts[(int64_t)(b + 32 * u + lane) * rs] = (int32_t)((uint32_t)x | kTomb);
+            hit |= is;
+            left--;
+          }
+        }
+      }
+    }
+    __syncwarp();
+  }
+  return hit;
+}
+
 // K6b + K7: for each erased id and each tree (largest first) probe the bloom
 // filter (one 32-byte sector); on a hit descend by the composite key to the
 // unique leaf, find the id, tombstone it and decrement the live counts along
@@ -67,44 +131,51 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
   int fti = 0;            // the tree that held the id
   int64_t leaf_at = 0;    // its leaf's index among that tree's 2^h leaves
   uint64_t mm = pending ? maybe_mask : 0;
-  while (mm) {
-    const int ti = __ffsll((long long)mm) - 1;
-    mm &= mm - 1;
-    const TreeView &T = F.trees[ti];
-    int v = 0, depth = 0;
-    Node nd;
-    bool ok = true;
-    while (true) {
-      path[depth] = v;
-      nd = T.node[v];
-      if (nd.l < 0) break;
-      uint64_t key = comp_key(xq[depth % F.dim], id);
-      v = key > nd.key ? nd.r : nd.l;
-      depth++;
-      if (v < 0 || v >= T.nnodes || depth > T.h) { ok = false; break; }
-    }
-    const int leaf = -1 - nd.l;
-    int a = 0, z = 0;
-    if (ok && leaf < ((int64_t)1 << T.h)) {
-      a = T.leaf_off[leaf];
-      z = T.leaf_off[leaf + 1];
-      if (a < 0 || z > T.size || a > z) { a = z = 0; atomicOr(F.err, kErrLeaf); }
-    } else {
-      atomicOr(F.err, kErrChild);
-    }
-    const int rs = rec_ints(F.dim);
-    for (int j = a; j < z; ++j) {
-      int32_t *slot = T.pts + (int64_t)j * rs + F.dim;
-      if (*slot == id) {
-        *slot = (int32_t)((uint32_t)id | kTomb);
-        found = true;
-        break;
+  const int rs = rec_ints(F.dim);
+  while (__any_sync(0xffffffffu, mm != 0)) {
+    int ti = -1, leaf = 0, a = 0, z = 0;
+    if (mm) {
+      ti = __ffsll((long long)mm) - 1;
+      mm &= mm - 1;
+      const TreeView &T = F.trees[ti];
+      int v = 0, depth = 0;
+      Node nd;
+      bool ok = true;
+      while (true) {
+        path[depth] = v;
+        nd = T.node[v];
+        if (nd.l < 0) break;
+        uint64_t key = comp_key(xq[depth % F.dim], id);
+        v = key > nd.key ? nd.r : nd.l;
+        depth++;
+        if (v < 0 || v >= T.nnodes || depth > T.h) { ok = false; break; }
+      }
+      leaf = -1 - nd.l;
+      if (ok && leaf < ((int64_t)1 << T.h)) {
+        a = T.leaf_off[leaf];
+        z = T.leaf_off[leaf + 1];
+        if (a < 0 || z > T.size || a > z) { a = z = 0; atomicOr(F.err, kErrLeaf); }
+      } else {
+        atomicOr(F.err, kErrChild);
       }
     }
-    if (found) {
+    bool hit = false;
+    if (z - a <= kLaneLeaf) {
+      for (int j = a; j < z; ++j) {
+        int32_t *slot = F.trees[ti].pts + (int64_t)j * rs + F.dim;
+        if (*slot == id) {
+          *slot = (int32_t)((uint32_t)id | kTomb);
+          hit = true;
+          break;
+        }
+      }
+    }
+    hit |= scan_big_leaves(F, rs, z - a > kLaneLeaf, ti, a, z, id);
+    if (hit) {
+      found = true;
       fti = ti;
       leaf_at = leaf;
-      break;
+      mm = 0;
     }
   }
   // live counts on the path: the nodes', and (when the job keeps them) the
