@@ -406,6 +406,7 @@ struct BuildTree {
   unsigned long long *err; // the forest's error word
   int64_t base = 0;        // set by build_trees: first staging position
   int g = 0;               // set by build_trees: levels split by the global kernels
+  unsigned long long *skew = nullptr;   // spatial builds: mapped word for the sum of squared leaf sizes
 };
 
 struct Scratch;            // allocation helper (forest.cu)
@@ -447,6 +448,10 @@ struct bdl_forest {
   uint64_t version = 0;          // bumped by every change of the trees or the buffer
   cudaEvent_t ev_flags = nullptr;  // recorded behind the insert flags' copy
   bdl::KnnShape knn_shape;         // launch shape of its k-NN calls
+  // spatial-median forests: per tree (kMaxLevel: the buffer's) the sum of its
+  // squared leaf sizes, written by the build to mapped page-locked memory
+  // whenever it gets there: a hint for the choice of k-NN kernel
+  volatile unsigned long long *skew = nullptr;
   // per static-tree level: the block of the level's last cleared tree, kept
   // for its next tree (forests without an hbm budget; freed by bdl_destroy)
   struct SpareBlock {
@@ -481,6 +486,10 @@ void *pinned_get(size_t bytes);
 void pinned_put(void *p);
 // The device address of mapped page-locked host memory (nullptr if none).
 void *mapped(void *host);
+// Whether a point of the (spatial-median) forest lies, on average, in a leaf
+// of more than kSkewedLeaf points, as far as its builds have reported.
+constexpr double kSkewedLeaf = 128;
+bool skewed_leaves(const bdl_forest *f);
 ForestView forest_view(const bdl_forest *f);
 // The view k-NN uses: the static trees plus the buffer's kd-tree.  With
 // build = true a stale buffer tree is rebuilt first (this allocates); with
@@ -505,6 +514,9 @@ int erase_lists(bdl_forest *f, const std::vector<const int32_t *> &ids, const st
                 int64_t *counts, cudaStream_t s);
 
 // ---- build.cu ----
+// A cooperative launch of fn(params) with every block that fits on the device
+// at once, or fewer where `items` work items need fewer threads.
+int launch_coop(const void *fn, int threads, int64_t items, void *params, int kid, double bytes, cudaStream_t s);
 struct ClearedSrc {        // a cleared tree whose live points join a new tree
   const int32_t *pts;      // point records
   int64_t size;
@@ -634,6 +646,7 @@ struct KnnCall {
   int64_t m;
   int32_t *oi;             // [m][k]
   int64_t *od;
+  bool skewed = false;     // its points lie in leaves far above the leaf size (skewed_leaves)
 };
 // Device form of a KnnCall (the kernel reads these from a table).
 struct KnnJob {
@@ -669,7 +682,7 @@ int launch_knn_table(const void *table, int njobs, int64_t warps, int dim, int k
 // The kernel with one warp per query (knn_warp.cu): whether a launch of m
 // queries on n points takes it, and its launches (the table's job prefix
 // counts one warp per query: upload_knn_table with qpw = 1).
-bool knn_by_warp(int dim, int k, int64_t m, int64_t n);
+bool knn_by_warp(int dim, int k, int64_t m, int64_t n, bool skewed);
 // The same for the calls of one launch together.
 bool knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k);
 int launch_knn_warp_one(const KnnOne &P, int dim, int k, cudaStream_t s);

@@ -1590,6 +1590,17 @@ int smem_subtree_capacity(int dim) {
   return 2048;
 }
 
+int launch_coop(const void *fn, int threads, int64_t items, void *params, int kid, double bytes, cudaStream_t s) {
+  int g = 0;
+  const int e = coop_grid(fn, threads, &g);
+  if (e) return e;
+  g = (int)std::min<int64_t>(g, std::max<int64_t>(1, ceil_div(std::min<int64_t>(items, (int64_t)1 << 40), threads)));
+  void *args[] = {params};
+  KScope ks_(kid, s, bytes);
+  return cuda_check(cudaLaunchCooperativeKernel(fn, dim3((unsigned)g), dim3((unsigned)threads), args, 0, s),
+                    "cooperative build kernel");
+}
+
 int build_trees(bdl_forest *af, int dim, std::vector<BuildTree> &bt, const std::vector<ClearedSrc> &cl,
                 cudaStream_t s) {
   if (af->cfg.split_rule == BDL_SPLIT_SPATIAL) return build_trees_spatial(af, dim, bt, cl, s);
@@ -1844,15 +1855,6 @@ int build_trees_object(bdl_forest *af, int dim, std::vector<BuildTree> &bt,
     dev_free(af, block, total, s);
     return st;
   }
-  auto coop = [&](const void *fn, int threads, void **args, int kid, double bytes) {
-    int g = 0;
-    int e = coop_grid(fn, threads, &g);
-    if (e) return e;
-    KScope ks_(kid, s, bytes);
-    return cuda_check(cudaLaunchCooperativeKernel(fn, dim3((unsigned)g), dim3((unsigned)threads), args, 0, s),
-                      "cooperative build kernel");
-  };
-
   // ---- gather (K5) and the global levels (K1/K2), one cooperative launch ----
   if (cl_blk.back() || pool_off.back() || gmax) {
     // algorithmic bytes of the gather: every cleared record read, every live
@@ -1871,8 +1873,7 @@ int build_trees_object(bdl_forest *af, int dim, std::vector<BuildTree> &bt,
     B.nlev = gmax;
     B.bar = bar;
     B.err = bt[0].err;
-    void *args[] = {(void *)&B};
-    st = coop((const void *)k_build_levels, kCoopThreads, args, kK_build_levels, gbytes + lv_bytes);
+    st = launch_coop((const void *)k_build_levels, kCoopThreads, INT64_MAX, &B, kK_build_levels, gbytes + lv_bytes, s);
   }
 
   // ---- subtrees on chip: the 1,024-thread launch, then the 256-thread one ----
@@ -1921,8 +1922,7 @@ int build_trees_object(bdl_forest *af, int dim, std::vector<BuildTree> &bt,
     F.bw = (const BoxWork *)(plan + o_bw);
     F.bar = bar + 2;
     F.err = bt[0].err;
-    void *args[] = {(void *)&F};
-    st = coop((const void *)k_build_finish, 256, args, kK_build_finish, 0);
+    st = launch_coop((const void *)k_build_finish, 256, INT64_MAX, &F, kK_build_finish, 0, s);
   }
   if (!st)
     launch_pack_nodes((const TreeSeg *)(plan + o_pk), (const int64_t *)(plan + o_pkpre), (int)pk_segs.size(),

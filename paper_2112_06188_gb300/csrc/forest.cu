@@ -474,6 +474,24 @@ static int alloc_tree(bdl_forest *f, int level, int64_t size, cudaStream_t s, Tr
   return BDL_OK;
 }
 
+bool skewed_leaves(const bdl_forest *f) {
+  if (!f->skew) return false;
+  double sq = 0, n = 0;
+  for (int i = 0; i <= kMaxLevel; ++i) {
+    const Tree *t = i < kMaxLevel ? f->trees[i] : f->btree;
+    if (!t || t->h == 0) continue;
+    sq += (double)f->skew[i];
+    n += (double)t->size;
+  }
+  return sq > kSkewedLeaf * n;
+}
+
+// The device's address of a tree's word in its forest's `skew`.
+static unsigned long long *skew_word(const bdl_forest *f, int level) {
+  unsigned long long *d = f->skew ? (unsigned long long *)mapped((void *)f->skew) : nullptr;
+  return d ? d + level : nullptr;
+}
+
 ForestView forest_view(const bdl_forest *f) {
   ForestView v;
   memset(&v, 0, sizeof(v));
@@ -601,6 +619,7 @@ static int plan_insert(bdl_forest *f, const PoolSrc &pool, int64_t n, InsertPlan
     b.pool_lo = pos;
     b.idtab = f->idtab;
     b.err = f->err;
+    b.skew = skew_word(f, j);
     bt.push_back(b);
     pos += shortfall;
     prev = j;
@@ -813,6 +832,7 @@ static void refresh_btrees(bdl_forest *const *F, int nf, cudaStream_t s) {
     b.pool_lo = 0;
     b.idtab = f->idtab;
     b.err = f->err;
+    b.skew = skew_word(f, kMaxLevel);
     bt.push_back(b);
     owner.push_back(i);
   }
@@ -1420,7 +1440,7 @@ static int knn_many(bdl_forest *const *F, int nf, const int32_t *const *q, const
   for (int i = 0; i < nf; ++i) {
     if (m[i] == 0) continue;
     views[i] = knn_view(F[i], false, s);
-    calls.push_back(KnnCall{&views[i], q[i], perm[i], m[i], oi[i], od[i]});
+    calls.push_back(KnnCall{&views[i], q[i], perm[i], m[i], oi[i], od[i], skewed_leaves(F[i])});
   }
   int st = BDL_OK;
   std::vector<int> dims;
@@ -1508,7 +1528,7 @@ static int knn_plan_make(bdl_forest *const *F, int nf, const int32_t *const *q, 
     if (m[i] == 0) continue;
     views[i] = knn_view(F[i], false, s);
     if (m[i] >= kSortMinQueries) sort_bytes += a256(query_sort_bytes(m[i], F[i]->dim));
-    calls.push_back(KnnCall{&views[i], q[i], nullptr, m[i], oi[i], od[i]});
+    calls.push_back(KnnCall{&views[i], q[i], nullptr, m[i], oi[i], od[i], skewed_leaves(F[i])});
   }
   std::vector<int> dims;
   for (auto &c : calls)
@@ -1740,6 +1760,10 @@ int bdl_create(int dim, const bdl_config *cfg, const int32_t *pts, int64_t n, in
     const char *dbg = getenv("BDL_DEBUG_CHECK");
     f->debug_check = dbg && dbg[0] == '1';
   }
+  if (!st && c.split_rule == BDL_SPLIT_SPATIAL) {   // (no memory for the hint: no hint)
+    f->skew = (volatile unsigned long long *)pinned_get((kMaxLevel + 1) * 8);
+    if (f->skew) memset((void *)f->skew, 0, (kMaxLevel + 1) * 8);
+  }
   void *buf = nullptr;
   if (!st) st = dev_alloc(f, &buf, (size_t)c.buffer_size * 4, s);
   f->buf = (int32_t *)buf;
@@ -1880,6 +1904,7 @@ int bdl_destroy(bdl_forest *f) {
   cudaStreamSynchronize(s);
   if (f->ev_flags) cudaEventDestroy(f->ev_flags);
   if (f->pinned) cudaFreeHost(f->pinned);
+  pinned_put((void *)f->skew);
   delete f;
   return cuda_check(cudaGetLastError(), "destroy");
 }

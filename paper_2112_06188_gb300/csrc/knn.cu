@@ -795,12 +795,13 @@ size_t batch_query_sort_bytes(const std::vector<KnnCall> &calls) {
 }
 
 bool knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k) {
-  int64_t m = 0, n = 0;
+  int64_t m = 0, n = 0, ms = 0;
   for (const auto &c : calls) {
     m += c.m;
+    if (c.skewed) ms += c.m;
     for (int t = 0; t < c.fv->ntrees; ++t) n += c.fv->tree[t].size;
   }
-  return knn_by_warp(dim, k, m, n);
+  return knn_by_warp(dim, k, m, n, 2 * ms > m);
 }
 
 size_t knn_table_bytes(const std::vector<KnnCall> &calls) {
@@ -1045,7 +1046,7 @@ extern "C" int bdl_knn_noalloc(bdl_forest *f, const int32_t *q, int64_t m, int k
       launch_query_sort(q, m, f->dim, (char *)scratch + kNoAllocPermBytes, perm, s);
     }
     // a single forest's job goes by kernel parameters: no table to place
-    std::vector<KnnCall> calls{KnnCall{&fv, q, perm, m, out_ids, out_d2}};
+    std::vector<KnnCall> calls{KnnCall{&fv, q, perm, m, out_ids, out_d2, skewed_leaves(f)}};
     st = finish_call(f, s, launch_knn_jobs(calls, f->dim, k, f->knn_shape, nullptr, f->knn_stats, s));
   }
   if (prev >= 0 && prev != f->device) cudaSetDevice(prev);

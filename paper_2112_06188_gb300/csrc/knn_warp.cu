@@ -463,7 +463,13 @@ void warp_table(const KnnJob *jobs, const int64_t *job_warp, int njobs, int64_t 
 //   dim 6, k = 1:  262K 2128 / 1233, 1M 3313 / 4229; k = 10: 1M 11838 / 11479
 //   dim 7, k = 1:  1M queries on 100K points 4350 / 4399 (clusters 2503 / 3404),
 //                  on 10M 11182 / 7054;           k = 5: 1M on 1M 20953 / 12524
-bool knn_by_warp(int dim, int k, int64_t m, int64_t n) {
+// Leaves of hundreds of points and more (spatial-median trees of clustered
+// points) are scanned by one lane in the thread-per-query kernel, 32 points at
+// a time here.  100 clusters, thread / warp in us: 1M 2-D points, k = 5, 100K
+// queries 4014 / 1062, 1M queries 7174 / 8953; 1M 3-D points, k = 10, 1M
+// queries 16160 / 9937; 10M 3-D points, 1M queries 68980 / 39557.
+bool knn_by_warp(int dim, int k, int64_t m, int64_t n, bool skewed) {
+  if (skewed && (dim > 2 || m <= 600000)) return true;
   struct Line {
     double base, slope;   // k <= 16: most queries (thousands) = base + slope k
     double k24, k32;      // for k = 17 .. 24 and above
