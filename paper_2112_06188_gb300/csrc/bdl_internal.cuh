@@ -326,32 +326,30 @@ enum : unsigned long long {
 };
 
 // Grid-wide barrier of a cooperative launch (every block resident at once):
-// bar[0] counts the blocks that arrived, bar[1] is the generation the last
-// arrival advances.  Writes before the barrier are visible after it (block
-// barrier, then a device-scope fence by the arriving thread, cumulative over
-// the block's writes, and another after the wait).  The wait is bounded:
+// *bar, zero when the launch starts, counts the arrivals; a block waits until
+// all have come `epoch` times (its own count, zero at first).  An arrival is
+// one reduction without an answer, and the wait reads the word that the
+// arrivals change, so the barrier costs a fence and about two trips to L2 (a
+// counter that the last block resets and a generation word behind it took
+// about 6 us with 304 blocks).  Writes before the barrier are visible after it
+// (block barrier, then a device-scope fence by the arriving thread, cumulative
+// over the block's writes, and another after the wait).  The wait is bounded:
 // after kBarrierPolls polls (about a second) the block sets kErrBarrier in
 // *err and goes on, so a lost block never hangs the GPU; the call then fails
 // with BDL_EINTERNAL.
-constexpr unsigned kBarrierPolls = 1u << 24;
-__device__ __forceinline__ void grid_barrier(unsigned *bar, unsigned long long *err) {
+constexpr unsigned kBarrierPolls = 1u << 21;
+__device__ __forceinline__ void grid_barrier(unsigned *bar, unsigned &epoch, unsigned long long *err) {
   __syncthreads();
+  epoch += gridDim.x;
   if (threadIdx.x == 0) {
-    volatile unsigned *gen = bar + 1;
-    const unsigned g = *gen;
     __threadfence();
-    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-      atomicExch(bar, 0u);
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      unsigned polls = 0;
-      while (*gen == g) {
-        if (++polls > kBarrierPolls) {
-          atomicOr(err, kErrBarrier);
-          break;
-        }
-        __nanosleep(64);
+    atomicAdd(bar, 1u);
+    volatile unsigned *seen = bar;
+    unsigned polls = 0;
+    while ((int)(*seen - epoch) < 0) {
+      if (++polls > kBarrierPolls) {
+        atomicOr(err, kErrBarrier);
+        break;
       }
     }
     __threadfence();

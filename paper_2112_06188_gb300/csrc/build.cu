@@ -37,6 +37,7 @@ constexpr int kSubThreads = 1024;  // threads of the subtree kernel
 constexpr int kSmallSubThreads = 256;   // threads of its instance for small subtrees
 constexpr int kSmallSub = 2048;         // subtrees below this many records take that instance
 constexpr int kWarpMode = 64;      // segments this small are sorted by one warp
+constexpr int kCoopThreads = 512;  // threads of the level kernel = tile / kItems for 4096-record tiles
 
 struct SegState {
   unsigned long long cand_n;   // candidates gathered
@@ -354,7 +355,11 @@ __device__ void level_collect(const LvParams &P, int64_t b) {
 }
 
 // One CTA per segment: exact select of the median among its bucket's keys
-// (8-bit digits over the 40-bit candidate key), then the node is written.
+// (8-bit digits over the 40-bit candidate key until at most 32 candidates are
+// left, which a warp ranks), then the node is written.  The other blocks wait
+// for it, so its chain is kept short: ranking the last candidates and finding
+// the node's slots beside the passes took the kernel from 238 to 204 us on 1M
+// 3-D points, together with the cheaper grid barrier.
 __device__ void level_select(const LvParams &P, int64_t gs, uint64_t *keys) {
   __shared__ uint32_t hist[256];
   __shared__ uint64_t s_pre;
@@ -362,6 +367,9 @@ __device__ void level_select(const LvParams &P, int64_t gs, uint64_t *keys) {
   __shared__ uint32_t s_cnt;
   __shared__ uint64_t s_found;
   __shared__ uint32_t s_wsum[32];
+  __shared__ int32_t s_slot[3];
+  __shared__ uint64_t s_few[32];
+  __shared__ unsigned s_nfew;
   const LvTree &T = tree_by_seg(P, gs);
   int64_t idx = gs - T.seg_off;
   int64_t st, sz;
@@ -372,16 +380,29 @@ __device__ void level_select(const LvParams &P, int64_t gs, uint64_t *keys) {
   bool in_smem = n <= 2048;
   if (in_smem)
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) keys[i] = cand[i];
-  if (threadIdx.x == 0) { s_pre = 0; s_rank = S.rank; s_cnt = (uint32_t)n; s_found = ~0ull; }
+  if (threadIdx.x == 0) { s_pre = 0; s_rank = S.rank; s_cnt = (uint32_t)n; s_found = ~0ull; s_nfew = 0; }
+  // the slots of the node and its children, meanwhile, by three lanes of the last warp
+  const int l3 = (int)threadIdx.x - (kCoopThreads - 32);
+  if (l3 >= 0 && l3 < 3) s_slot[l3] = (int32_t)veb_slot(T.h + 1, l3 ? T.t + 1 : T.t, l3 ? 2 * idx + l3 - 1 : idx);
   __syncthreads();
   const int kbits = 31 + kHistShift;   // 40
   int shift = kbits;
   while (true) {
-    if (s_cnt == 1) {
-      // the unique key with this prefix
+    if (s_cnt <= 32) {
+      // few enough for a warp to rank against each other
       for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        uint64_t k = in_smem ? keys[i] : cand[i];
-        if ((k >> shift) == (s_pre >> shift)) s_found = k;
+        const uint64_t k = in_smem ? keys[i] : cand[i];
+        if ((k >> shift) != (s_pre >> shift)) continue;
+        const unsigned at = atomicAdd(&s_nfew, 1u);
+        if (at < 32) s_few[at] = k;
+      }
+      __syncthreads();
+      const int m = min((int)s_nfew, 32);
+      if ((int)threadIdx.x < m) {
+        const uint64_t k = s_few[threadIdx.x];
+        int less = 0;
+        for (int i = 0; i < m; ++i) less += s_few[i] < k;
+        if (less + 1 == s_rank) s_found = k;
       }
       __syncthreads();
       break;
@@ -434,26 +455,29 @@ __device__ void level_select(const LvParams &P, int64_t gs, uint64_t *keys) {
     uint32_t coord = ((uint32_t)S.bucket << kHistShift) | (uint32_t)(k40 >> 31);
     uint64_t med = comp_key((int32_t)coord, (int32_t)(k40 & 0x7fffffffu));
     S.median = med;
-    const NodeOut &o = T.out;
-    int l = T.h + 1;
-    int64_t v = veb_slot(l, T.t, idx);
-    o.node[v] = Node{med, (int32_t)veb_slot(l, T.t + 1, 2 * idx), (int32_t)veb_slot(l, T.t + 1, 2 * idx + 1)};
+    T.out.node[s_slot[0]] = Node{med, s_slot[1], s_slot[2]};
   }
 }
 
 
 // K2: partition every tile's records around their segment's median into the
 // other staging buffer.  Left records of a segment go to [st, st+ceil(m/2)),
-// right ones after; each CTA reserves its ranges with one atomic per class.
+// right ones after; each CTA reserves its ranges with one atomic per class
+// (segment of the tile, side).  A warp takes 256 consecutive records, 32 at a
+// time, so that the records of one class in such a group go to consecutive
+// places: every array is stored straight to its places, and the tile needs
+// two block barriers instead of two per array for a copy staged in shared
+// memory (the whole kernel, 10M 3-D points: 1,988 -> 1,690 us, 1M 5-D points:
+// 298 -> 254).  What bounds it at 10M points: memory (16 bytes read and written
+// per record and level, 47 us at 6.8 TB/s of the 86 us a level takes); below
+// 1M the latency of a tile's chain and the barriers around it.
 // hnext: shared memory for the next level's histograms of the tile's (up to
 // four) child segments, 16-bit counts packed in pairs (a tile has at most
 // 4096 records).
-__device__ void level_partition(const LvParams &P, int64_t b, int32_t *stage, uint32_t *hnext) {
-  __shared__ unsigned long long wsum[32];
-  __shared__ unsigned long long cbase[4];
-  __shared__ int64_t gdst[4];              // global start of each class's run
-  __shared__ int coff[5];                  // start of each class's run in `stage`
-  __shared__ int cok[4];
+__device__ void level_partition(const LvParams &P, int64_t b, uint32_t *hnext) {
+  constexpr int kW = kCoopThreads / 32;
+  __shared__ int s_cnt[4][kW];             // records of each class in each warp
+  __shared__ int s_dst[4][kW];             // where they go (in the tree), -1: nowhere
   const LvTree &T = tree_by_tile(P, b);
   TileSegs g = tile_segs(P, T, b);
   const int64_t nxt = T.next_seg;
@@ -462,98 +486,103 @@ __device__ void level_partition(const LvParams &P, int64_t b, int32_t *stage, ui
     for (int i = threadIdx.x; i < 4 * kHistBins / 8; i += blockDim.x)
       reinterpret_cast<uint4 *>(hnext)[i] = make_uint4(0, 0, 0, 0);
   const SegState *s0 = &P.seg[T.seg_off + g.idx0];
-  uint64_t med0 = s0[0].median, med1 = g.sz1 ? s0[1].median : 0;
-  const int32_t *xc = P.src + T.c * P.S + T.base;
-  const int32_t *xi = P.src + P.dim * P.S + T.base;
-  int64_t pb = g.p0 + (int64_t)threadIdx.x * kItems;
-  int cls[kItems];
+  const uint64_t med0 = s0[0].median, med1 = g.sz1 ? s0[1].median : 0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1;
+  const int n = (int)(g.p1 - g.p0);                          // records of the tile
+  const int cut = (int)min(g.st1 - g.p0, (int64_t)n);        // the first of its second segment
+  const int x0 = warp * (32 * kItems) + lane;                // this lane's first record of the tile
+  const int32_t *src = P.src + T.base + g.p0 + x0;
   int32_t cv[kItems], iv[kItems];
-  load8(xc, pb, g.p1, cv);
-  load8(xi, pb, g.p1, iv);
-  unsigned long long mine = 0;   // 4 x 16-bit class counts
+  auto load = [&](int c, int32_t *to) {
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) to[j] = x0 + 32 * j < n ? src[c * P.S + 32 * j] : 0;
+  };
+  load(T.c, cv);
+  load(P.dim, iv);
+
+  // class and rank among the warp's records of the class
+  uint32_t cls = 0;                        // 2 bits per item: 2 * (second segment) + right
+  uint32_t rank[kItems / 4] = {0, 0};      // 8 bits per item
+  int cnt[4] = {0, 0, 0, 0};
 #pragma unroll
   for (int j = 0; j < kItems; ++j) {
-    int64_t p = pb + j;
-    cls[j] = -1;
-    if (p < g.p1) {
-      int w = p >= g.st1;
-      uint64_t k = comp_key(cv[j], iv[j]);
-      int c = 2 * w + (k > (w ? med1 : med0));
-      cls[j] = c;
-      mine += 1ull << (16 * c);
-    }
+    const int x = x0 + 32 * j;
+    const bool w = x >= cut;
+    const bool r = comp_key(cv[j], iv[j]) > (w ? med1 : med0);
+    const unsigned mv = __ballot_sync(0xffffffffu, x < n), mw = __ballot_sync(0xffffffffu, w),
+                   mr = __ballot_sync(0xffffffffu, r);
+    const unsigned mine = mv & (w ? mw : ~mw) & (r ? mr : ~mr);
+    const int c = 2 * w + r;
+    const int before = c == 0 ? cnt[0] : c == 1 ? cnt[1] : c == 2 ? cnt[2] : cnt[3];
+    cls |= (uint32_t)c << (2 * j);
+    rank[j / 4] |= (uint32_t)(before + __popc(mine & lt)) << (8 * (j & 3));
+    cnt[0] += __popc(mv & ~mw & ~mr);
+    cnt[1] += __popc(mv & ~mw & mr);
+    cnt[2] += __popc(mv & mw & ~mr);
+    cnt[3] += __popc(mv & mw & mr);
   }
-  // block exclusive scan of the packed counts
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long inc = mine;
-  for (int o = 1; o < 32; o <<= 1) {
-    unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += y;
-  }
-  if (lane == 31) wsum[warp] = inc;
+  if (lane < 4) s_cnt[lane][warp] = lane == 0 ? cnt[0] : lane == 1 ? cnt[1] : lane == 2 ? cnt[2] : cnt[3];
   __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long acc = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { unsigned long long v = wsum[w]; wsum[w] = acc; acc += v; }
-    coff[0] = 0;
-    for (int c = 0; c < 4; ++c) {
-      unsigned long long tot = (acc >> (16 * c)) & 0xffff;
-      cbase[c] = 0;
-      if (tot) {
-        const SegState &S = P.seg[T.seg_off + g.idx0 + (c >> 1)];
-        unsigned long long *cur = (c & 1) ? (unsigned long long *)&S.rcur : (unsigned long long *)&S.lcur;
-        cbase[c] = atomicAdd(cur, tot);
+  if (threadIdx.x < 4 * kW) {
+    // lane group of kW = 16: one class, prefix over the warps
+    const int c = threadIdx.x / kW, w = threadIdx.x % kW;
+    const int mine = s_cnt[c][w];
+    int inc = mine;
+    for (int o = 1; o < kW; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, inc, o, kW);
+      if (w >= o) inc += y;
+    }
+    const int tot = __shfl_sync(0xffffffffu, inc, kW - 1, kW);
+    int at = 0;
+    if (w == 0 && tot) {
+      const SegState &S = P.seg[T.seg_off + g.idx0 + (c >> 1)];
+      unsigned long long *cur = (c & 1) ? (unsigned long long *)&S.rcur : (unsigned long long *)&S.lcur;
+      const int64_t st = (c >> 1) ? g.st1 : g.st0, sz = (c >> 1) ? g.sz1 : g.sz0, half = (sz + 1) >> 1;
+      const int64_t base = (int64_t)atomicAdd(cur, (unsigned long long)tot);
+      if (base + tot > ((c & 1) ? sz - half : half)) {   // the median did not halve the segment
+        atomicOr(T.err, kErrPartition);
+        at = -1;
+      } else {
+        at = (int)(st + ((c & 1) ? half : 0) + base);
       }
-      const int64_t st = (c >> 1) ? g.st1 : g.st0;
-      const int64_t sz = (c >> 1) ? g.sz1 : g.sz0;
-      const int64_t off = (c & 1) ? ((sz + 1) >> 1) : 0;
-      const int64_t lim = (c & 1) ? sz - ((sz + 1) >> 1) : ((sz + 1) >> 1);
-      gdst[c] = st + off + (int64_t)cbase[c];
-      cok[c] = (int64_t)(cbase[c] + tot) <= lim;   // else the median did not halve the segment
-      if (!cok[c]) atomicOr(T.err, kErrPartition);
-      coff[c + 1] = coff[c] + (int)tot;
     }
+    at = __shfl_sync(0xffffffffu, at, 0, kW);
+    s_dst[c][w] = at < 0 ? -1 : at + inc - mine;
   }
   __syncthreads();
-  const unsigned long long ex = inc - mine + wsum[warp];
-  int spos[kItems];                 // position of each item in the tile's output order
-  int run[4] = {0, 0, 0, 0};
+  int dst[kItems];
 #pragma unroll
   for (int j = 0; j < kItems; ++j) {
-    const int c = cls[j];
-    spos[j] = -1;
-    if (c < 0) continue;
-    spos[j] = coff[c] + (int)((ex >> (16 * c)) & 0xffff) + run[c];
-    run[c]++;
+    const int d = s_dst[(cls >> (2 * j)) & 3][warp];
+    dst[j] = x0 + 32 * j < n && d >= 0 ? d + (int)((rank[j / 4] >> (8 * (j & 3))) & 0xffu) : -1;
   }
-  // each array: scatter into shared memory, then write every class's run
-  // with consecutive threads on consecutive addresses; the next level's
-  // split coordinate also goes into its child segment's histogram.  The
-  // next array's items are loaded as soon as this one's are scattered, so
-  // that their loads overlap the barrier and the stores.
-  const int ntile = coff[4];
-  int32_t v[kItems];
-  load8(P.src + T.base, pb, g.p1, v);
-  for (int c = 0; c <= P.dim; ++c) {
+  int32_t *y = P.dst + T.base;
+  // an array's values to their places; the next level's split coordinate
+  // also goes into its child segment's histogram
+  auto store = [&](int c, const int32_t *from) {
 #pragma unroll
     for (int j = 0; j < kItems; ++j)
-      if (spos[j] >= 0) {
-        stage[spos[j]] = v[j];
-        if (c == cn && nxt >= 0) {
-          const int bin = v[j] >> kHistShift;
-          atomicAdd(&hnext[cls[j] * (kHistBins / 2) + (bin >> 1)], 1u << (16 * (bin & 1)));
+      if (dst[j] >= 0) y[c * P.S + dst[j]] = from[j];
+    if (c == cn && nxt >= 0) {
+#pragma unroll
+      for (int j = 0; j < kItems; ++j)
+        if (dst[j] >= 0) {
+          const int bin = from[j] >> kHistShift;
+          atomicAdd(&hnext[((cls >> (2 * j)) & 3) * (kHistBins / 2) + (bin >> 1)], 1u << (16 * (bin & 1)));
         }
-      }
-    if (c < P.dim) load8(P.src + (c + 1) * P.S + T.base, pb, g.p1, v);
-    __syncthreads();
-    int32_t *y = P.dst + c * P.S + T.base;
-    for (int i = threadIdx.x; i < ntile; i += blockDim.x) {
-      const int k = (i >= coff[1]) + (i >= coff[2]) + (i >= coff[3]);
-      if (cok[k]) y[gdst[k] + (i - coff[k])] = stage[i];
     }
-    __syncthreads();
+  };
+  store(T.c, cv);
+  store(P.dim, iv);
+  for (int c = 0; c < P.dim; ++c) {
+    if (c == T.c) continue;
+    int32_t v[kItems];
+    load(c, v);
+    store(c, v);
   }
-  if (nxt >= 0)   // child (segment w, side) of level index idx0 + w is 2 (idx0 + w) + side
+  if (nxt >= 0) {   // child (segment w, side) of level index idx0 + w is 2 (idx0 + w) + side
+    __syncthreads();
     for (int i = threadIdx.x; i < 4 * kHistBins / 2; i += blockDim.x) {
       const int k = i / (kHistBins / 2), wd = i % (kHistBins / 2);
       if ((k >> 1) && !g.sz1) continue;
@@ -563,6 +592,7 @@ __device__ void level_partition(const LvParams &P, int64_t b, int32_t *stage, ui
       if (x & 0xffffu) atomicAdd(h, x & 0xffffu);
       if (x >> 16) atomicAdd(h + 1, x >> 16);
     }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -571,8 +601,6 @@ __device__ void level_partition(const LvParams &P, int64_t b, int32_t *stage, ui
 // blocks, pool entries, tiles, segments), and a grid barrier separates the
 // phases, instead of one launch per phase and level.
 // ---------------------------------------------------------------------------
-
-constexpr int kCoopThreads = 512;   // = tile / kItems for 4096-record tiles
 
 struct LevelWork {                  // one global level, in device memory
   LvParams P;
@@ -594,6 +622,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_build_levels(const LevelsPa
   // the partition's staging; the next level's histograms), 16 KB each
   __shared__ __align__(16) uint32_t s_big[2 * kHistBins];
   __shared__ __align__(16) uint32_t s_next[2 * kHistBins];
+  unsigned epoch = 0;
   for (int64_t b = blockIdx.x; b < B.cl_blocks; b += gridDim.x) {
     gather_cleared(B.G, b);
     __syncthreads();
@@ -604,7 +633,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_build_levels(const LevelsPa
   if (B.nlev == 0) return;
   // the first level's histograms; every later level's come from the
   // partition of the level before
-  grid_barrier(B.bar, B.err);
+  grid_barrier(B.bar, epoch, B.err);
   for (int64_t b = blockIdx.x; b < B.lv[0].ntile; b += gridDim.x) {
     level_hist(B.lv[0].P, b, reinterpret_cast<uint32_t (*)[kHistBins]>(s_big));
     __syncthreads();
@@ -612,17 +641,17 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_build_levels(const LevelsPa
   for (int it = 0; it < B.nlev; ++it) {
     const LevelWork &W = B.lv[it];
     const LvParams &P = W.P;
-    grid_barrier(B.bar, B.err);
+    grid_barrier(B.bar, epoch, B.err);
     for (int64_t b = blockIdx.x; b < W.ntile; b += gridDim.x) {
       level_collect(P, b);
       __syncthreads();
     }
-    grid_barrier(B.bar, B.err);
+    grid_barrier(B.bar, epoch, B.err);
     for (int64_t gs = blockIdx.x; gs < W.nseg; gs += gridDim.x) {
       level_select(P, gs, reinterpret_cast<uint64_t *>(s_big));
       __syncthreads();
     }
-    grid_barrier(B.bar, B.err);
+    grid_barrier(B.bar, epoch, B.err);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P.nseg_next;
          i += (int64_t)gridDim.x * blockDim.x) {
       P.seg_next[i].cand_n = 0;
@@ -630,7 +659,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_build_levels(const LevelsPa
       P.seg_next[i].rcur = 0;
     }
     for (int64_t b = blockIdx.x; b < W.ntile; b += gridDim.x) {
-      level_partition(P, b, reinterpret_cast<int32_t *>(s_big), s_next);
+      level_partition(P, b, s_next);
       __syncthreads();
     }
   }
@@ -1423,12 +1452,13 @@ __device__ void box_up(const FinishParams &F, const BoxWork &W, int64_t g) {
 }
 
 __global__ void __launch_bounds__(256) k_build_finish(const FinishParams F) {
+  unsigned epoch = 0;
   for (int t = F.nlev - 1; t >= 0; --t) {
     const BoxWork &W = F.bw[t];
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < W.total;
          g += (int64_t)gridDim.x * blockDim.x)
       box_up(F, W, g);
-    if (t > 0) grid_barrier(F.bar, F.err);
+    if (t > 0) grid_barrier(F.bar, epoch, F.err);
   }
 }
 

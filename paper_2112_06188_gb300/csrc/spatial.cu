@@ -438,8 +438,9 @@ __global__ void __launch_bounds__(kT) k_sp_boxes(const SpBoxParams P) {
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
   for (int64_t x = t0 & ~(int64_t)31; x < P.leaf_pre[P.ntree]; x += step) sp_leaf_boxes(P, x);
   const int dim = P.dim;
+  unsigned epoch = 0;
   for (int t = P.hmax - 1; t >= 0; --t) {
-    grid_barrier(P.bar, P.err);
+    grid_barrier(P.bar, epoch, P.err);
     for (int64_t s = t0; s < P.depth[t]; s += step) {
       const SpTree &tr = P.T[s >> t];
       const int64_t i = s & (((int64_t)1 << t) - 1);
