@@ -105,6 +105,25 @@ __host__ __device__ inline int64_t veb_slot(int l, int t, int64_t i) {
   return off;
 }
 
+// veb_slot in 32-bit arithmetic (nodes are numbered in 31 bits): the smallest
+// power of two >= l/2 is the highest one in l - 1.
+__device__ inline int veb_slot32(int l, int t, int i) {
+  int off = 0;
+  while (l > 1) {
+    const int lb = 1 << (31 - __clz(l - 1)), lt = l - lb;
+    if (t < lt) {
+      l = lt;
+    } else {
+      const int tt = t - lt, j = i >> tt;
+      off += ((1 << lt) - 1) + j * ((1 << lb) - 1);
+      i &= (1 << tt) - 1;
+      t = tt;
+      l = lb;
+    }
+  }
+  return off;
+}
+
 // Point range of segment `idx` at depth t of a tree over s points, where every
 // split gives the left child ceil(m/2) points.  O(t).
 __host__ __device__ inline void seg_range(int64_t s, int t, int64_t idx, int64_t &start,

@@ -720,9 +720,29 @@ __device__ __forceinline__ void warp_sort64(uint64_t &x0, uint64_t &x1, int lane
   }
 }
 
+// The same for 32-bit words.
+__device__ __forceinline__ uint32_t warp_sort32w(uint32_t x, int lane) {
+#pragma unroll
+  for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      const uint32_t y = __shfl_xor_sync(0xffffffffu, x, stride);
+      const bool keep_min = ((lane & stride) == 0) == ((lane & size) == 0);
+      x = keep_min ? min(x, y) : max(x, y);
+    }
+  return x;
+}
+
 __device__ __forceinline__ uint64_t skey(const int32_t *sc, const int32_t *sid, int cap, int c,
                                          int it) {
   return comp_key(sc[c * cap + it], sid[it]);
+}
+
+// The w bits of record it's key below its `sh` open ones (fewer where fewer are
+// open).
+__device__ __forceinline__ int key_digit(const int32_t *sc, const int32_t *sid, int cap, int c, int it, int sh, int w) {
+  const int ns = max(0, sh - w);
+  return (int)((skey(sc, sid, cap, c, it) >> ns) & ((1u << (sh - ns)) - 1));
 }
 
 // seg_range for a subtree (m < 2^31 points).
@@ -748,6 +768,15 @@ __device__ __forceinline__ int open_key_bits(int32_t lo, int32_t hi) {
   return 31 + (lo == hi ? 0 : 32 - __clz(lo ^ hi));
 }
 
+// What bounds it: issue (61% of the slots on 8,192-record 3-D subtrees) and
+// the block barriers around the few-thread phases between the passes.  Of
+// about 245,000 cycles per such subtree the partitions take a quarter, the
+// digit passes 15%, the bin scans 15%, the two warp-sorted levels 18%, the
+// boxes 7%.  10M 3-D points: 1,308 -> 1,116 us by working out the radix levels'
+// slots once in 32 bits, starting the children's searches a warp per segment
+// instead of in a phase of their own, wide reads of bins and digits, the
+// median and the last sort on 32-bit words, and a leaf's record numbers kept
+// in registers for its box.
 // TH threads per CTA (1024, or 256 for subtrees of fewer than 2048 records):
 // 2 * TH histogram bins per pass, TH / 8 segments per radix level at most.
 template <int TH>
@@ -758,15 +787,16 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
   constexpr int MS = TH / 8;                   // segments of a radix level (cap / 64 <= 8 TH / 64)
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ uint64_t s_pre[MS], s_res[MS];
-  __shared__ int32_t s_st[MS], s_sz[MS], s_rank[MS],
-      s_cnt2[MS], s_lb[MS], s_dig[MS],
+  __shared__ int32_t s_range[2][2][MS];     // this level's and the next one's segments: start, size
+  __shared__ int32_t s_rank[MS], s_cnt2[MS], s_lb[MS],
+      s_dig[MS],                            // the digit chosen last, -1: the segment's search is over
       s_bel[MS], s_wq[MS];
   __shared__ unsigned char s_done[MS];
   __shared__ uint32_t s_w[32], s_base[8];
   __shared__ int s_ncand;
-  // key bits still open per segment (the digits below them are the next to
-  // decide): this level's, and the next level's set by the partition
-  __shared__ int32_t s_sh[MS], s_shn[MS];
+  // key bits still open per segment (the digits below them are the next to decide)
+  __shared__ int32_t s_sh[MS];
+  __shared__ int32_t s_slot[2 * MS];        // vEB slots of the radix levels' nodes and their children, by heap index
 
   const int cap = P.cap, dim = P.dim;
   int b = blockIdx.x;
@@ -842,33 +872,40 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
   uint16_t *cur = perm0, *nxt = perm1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
 
+  int32_t *s_st = s_range[0][0], *s_sz = s_range[0][1], *n_st = s_range[1][0], *n_sz = s_range[1][1];
+  // Segment ch of a level (its range, and the bounds [lo, hi] of its
+  // coordinates in the level's split dimension) before its median search: the
+  // key bits above the open ones are the bounds' common prefix, the same for
+  // every record of the segment.
+  auto begin_seg = [&](int ch, int st, int sz, int32_t lo, int32_t hi, int32_t *to_st, int32_t *to_sz) {
+    const int sh = open_key_bits(lo, hi);
+    to_st[ch] = st;
+    to_sz[ch] = sz;
+    s_sh[ch] = sh;
+    s_pre[ch] = sh >= kKeyBits ? 0 : ((uint64_t)lo >> (sh - 31)) << sh;
+    s_rank[ch] = (sz + 1) >> 1;
+    s_cnt2[ch] = 0;
+    s_done[ch] = 0;
+  };
+  for (int x = threadIdx.x + 1; x < min(2 * MS, 2 * nleaf); x += blockDim.x) {
+    const int ux = 31 - __clz(x);
+    s_slot[x] = veb_slot32(l, t0 + ux, ((int)i0 << ux) + (x - (1 << ux)));
+  }
+  if (threadIdx.x == 0) {
+    const int c0 = t0 % dim;
+    begin_seg(0, 0, m0, bcur[2 * c0], bcur[2 * c0 + 1], s_st, s_sz);
+    s_ncand = 0;
+  }
+  __syncthreads();
+
   for (int u = 0; u < U; ++u) {
     const int t = t0 + u;
     const int c = t % dim;
     const int nseg = 1 << u;
-    int64_t st_, sz_;
-    seg_range(m0, u, 0, st_, sz_);
-    const int mmax = (int)sz_;
+    const int mmax = (m0 + nseg - 1) >> u;   // the largest segment (every left child takes the larger half)
     if (mmax > kWarpMode) {
       // ---------------- radix mode: all segments of the level together ----
       const int w = LB - u;      // nseg << w == HB bins
-      for (int s = threadIdx.x; s < nseg; s += blockDim.x) {
-        int64_t a, z;
-        seg_range(m0, u, s, a, z);
-        s_st[s] = (int)a;
-        s_sz[s] = (int)z;
-        // the key bits above the open ones are the bounds' common prefix,
-        // the same for every record of the segment
-        const int32_t lo = bcur[(s * dim + c) * 2], hi = bcur[(s * dim + c) * 2 + 1];
-        const int sh = open_key_bits(lo, hi);
-        s_sh[s] = sh;
-        s_pre[s] = sh >= kKeyBits ? 0 : ((uint64_t)lo >> (sh - 31)) << sh;
-        s_rank[s] = (int)((z + 1) >> 1);
-        s_cnt2[s] = 0;
-        if (s == 0) s_ncand = 0;
-        s_done[s] = 0;
-      }
-      __syncthreads();
       // Every pass decides the next w open bits of each segment's median
       // key (the digit below its s_sh open bits) from a histogram of the
       // records that still match the segment's prefix.  Pass 0 counts every
@@ -887,9 +924,7 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
           if (!hist_ready) {
             for (int q = threadIdx.x; q < m0; q += blockDim.x) {
               const int s = segid[q], it = cur[q];
-              const uint64_t k = skey(sc, sid, cap, c, it);
-              const int sh = s_sh[s], ns = max(0, sh - w);
-              const int dg = (int)((k >> ns) & ((1u << (sh - ns)) - 1));
+              const int dg = key_digit(sc, sid, cap, c, it, s_sh[s], w);
               binq[q] = (uint16_t)dg;
               wit[(s << w) + dg] = (uint16_t)it;
               atomicAdd(&hist[(s << w) + dg], 1u);
@@ -897,16 +932,27 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
             __syncthreads();
           }
         } else if (pass == 1) {
-          for (int q = threadIdx.x; q < m0; q += blockDim.x) {
-            const int s = segid[q];
-            if (s_done[s] || binq[q] != s_dig[s]) continue;
+          const int ipt = cap / TH, q1 = threadIdx.x * ipt;   // consecutive positions of a thread
+          auto one = [&](int q, int s, int dg1) {
+            if (q >= m0 || s_dig[s] != dg1) return;
             cand[atomicAdd(&s_ncand, 1)] = (uint16_t)q;
             const int it = cur[q];
-            const uint64_t k = skey(sc, sid, cap, c, it);
-            const int sh = s_sh[s], ns = max(0, sh - w);
-            const int dg = (int)((k >> ns) & ((1u << (sh - ns)) - 1));
+            const int dg = key_digit(sc, sid, cap, c, it, s_sh[s], w);
             wit[(s << w) + dg] = (uint16_t)it;
             atomicAdd(&hist[(s << w) + dg], 1u);
+          };
+          if (ipt == 8) {
+            // eight positions in one read of their digits and one of their
+            // segments
+            const uint4 bq = *reinterpret_cast<const uint4 *>(binq + q1);
+            const uint2 sv = *reinterpret_cast<const uint2 *>(segid + q1);
+            const uint32_t b4[4] = {bq.x, bq.y, bq.z, bq.w}, s2[2] = {sv.x, sv.y};
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              one(q1 + j, (int)((s2[j >> 2] >> (8 * (j & 3))) & 0xffu), (int)((b4[j >> 1] >> (16 * (j & 1))) & 0xffffu));
+          } else {
+            for (int j = 0; j < ipt; ++j)
+              if (q1 + j < m0) one(q1 + j, segid[q1 + j], binq[q1 + j]);
           }
           __syncthreads();
         } else {
@@ -991,15 +1037,33 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
             } else {
               pending = 1;
             }
+            if (s_done[s]) s_dig[s] = -1;
           }
         } else {
           // one warp per segment: a scan of the segment's bins across the lanes
           for (int s = warp; s < nseg; s += nwarps) {
             if (s_done[s]) continue;
+            // the lane's bins in one or two wide reads
             uint32_t *h = hist + (s << w) + lane * per;
-            const int nb = max(0, min(per, nbin - lane * per));
-            uint32_t sum = 0;
-            for (int i = 0; i < nb; ++i) sum += h[i];
+            uint32_t v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+            if (per == 8) {
+              const uint4 x = reinterpret_cast<const uint4 *>(h)[0], y = reinterpret_cast<const uint4 *>(h)[1];
+              v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+              v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+              reinterpret_cast<uint4 *>(h)[0] = reinterpret_cast<uint4 *>(h)[1] = make_uint4(0, 0, 0, 0);
+            } else if (per == 4) {
+              const uint4 x = reinterpret_cast<const uint4 *>(h)[0];
+              v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+              reinterpret_cast<uint4 *>(h)[0] = make_uint4(0, 0, 0, 0);
+            } else if (per == 2) {
+              const uint2 x = reinterpret_cast<const uint2 *>(h)[0];
+              v[0] = x.x; v[1] = x.y;
+              reinterpret_cast<uint2 *>(h)[0] = make_uint2(0, 0);
+            } else if (lane < nbin) {   // per == 1
+              v[0] = h[0];
+              h[0] = 0;
+            }
+            const uint32_t sum = v[0] + v[1] + v[2] + v[3] + v[4] + v[5] + v[6] + v[7];
             uint32_t inc = sum;
             for (int o2 = 1; o2 < 32; o2 <<= 1) {
               const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o2);
@@ -1008,16 +1072,21 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
             const uint32_t r = (uint32_t)s_rank[s];
             const bool mine = inc - sum < r && r <= inc;
             if (mine) {
-              uint32_t below = inc - sum, cj = h[0];
-              int i = 0;
-              while (below + cj < r) {   // ends inside this lane's bins (r <= inc)
-                below += cj;
-                cj = h[++i];
-              }
+              uint32_t below = inc - sum, cj = 0, b0 = 0;
+              int i = -1;
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                if (i < 0) {   // ends inside this lane's bins (r <= inc)
+                  if (r <= below + v[j]) {
+                    i = j;
+                    cj = v[j];
+                    b0 = below;
+                  }
+                  below += v[j];
+                }
               const int ns = max(0, s_sh[s] - w), dg = lane * per + i;
-              s_dig[s] = dg;
               s_pre[s] |= (uint64_t)dg << ns;
-              s_rank[s] = (int)(r - below);
+              s_rank[s] = (int)(r - b0);
               s_sh[s] = ns;
               if (cj == 1) {
                 s_res[s] = skey(sc, sid, cap, c, wit[(s << w) + dg]);
@@ -1028,49 +1097,52 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
               } else {
                 pending = 1;
               }
+              s_dig[s] = s_done[s] ? -1 : dg;
             }
             if (!__any_sync(0xffffffffu, mine) && lane == 0) {   // counts inconsistent with the rank
               atomicOr(T.err, kErrPartition);
               s_done[s] = 1;
+              s_dig[s] = -1;
             }
-            for (int i = 0; i < nb; ++i) h[i] = 0;
           }
         }
         if (!__syncthreads_or(pending)) break;
       }
       hist_ready = false;
-      // node keys
-      for (int s = threadIdx.x; s < nseg; s += blockDim.x) {
-        int64_t bfs = (i0 << u) + s;
-        int64_t v = veb_slot(l, t, bfs);
-        o.node[v] = Node{s_res[s], (int32_t)veb_slot(l, t + 1, 2 * bfs), (int32_t)veb_slot(l, t + 1, 2 * bfs + 1)};
+      // A warp per segment: the node and, when the next level also selects by
+      // radix, the children's bounds -- the parent's, cut at the median's
+      // coordinate in the split dimension (left: coordinates <= v, right: >= v)
+      // -- and their searches' start.  (With a thread per segment, which also
+      // worked out three slots, this took 15% of the kernel while the block
+      // waited.)
+      const bool next_radix = u + 1 < U && ((m0 + 2 * nseg - 1) >> (u + 1)) > kWarpMode;
+      const int wn = LB - 1 - u;             // the next level's digit width, LB - (u + 1)
+      const int cn = (t + 1) % dim;
+      if (threadIdx.x == 0) s_ncand = 0;
+      for (int s = warp; s < nseg; s += nwarps) {
+        const uint64_t med = s_res[s];
+        const int x = nseg + s;   // heap index
+        if (lane == 0) o.node[s_slot[x]] = Node{med, s_slot[2 * x], s_slot[2 * x + 1]};
+        if (next_radix) {
+          const int32_t v = (int32_t)(med >> 31);
+          if (lane < 2 * dim) {              // one coordinate of one child
+            const int side = lane >= dim, cc = side ? lane - dim : lane, ch = 2 * s + side;
+            int32_t lo = bcur[(s * dim + cc) * 2], hi = bcur[(s * dim + cc) * 2 + 1];
+            if (cc == c && side) lo = v;
+            if (cc == c && !side) hi = v;
+            bnxt[(ch * dim + cc) * 2] = lo;
+            bnxt[(ch * dim + cc) * 2 + 1] = hi;
+            if (cc == cn) {
+              const int st = s_st[s], sz = s_sz[s], half = (sz + 1) >> 1;
+              begin_seg(ch, side ? st + half : st, side ? sz - half : half, lo, hi, n_st, n_sz);
+            }
+          }
+        }
       }
       // stable partition by a block scan of the left flags (positions blocked
       // per thread); when the next level also selects by radix, its first
       // pass's histogram (the top bits of the next split coordinate, per
       // child segment) is counted on the way
-      int64_t nst_, nsz_;
-      seg_range(m0, u + 1, 0, nst_, nsz_);
-      const bool next_radix = u + 1 < U && nsz_ > kWarpMode;
-      const int wn = LB - 1 - u;             // the next level's digit width, LB - (u + 1)
-      const int cn = (t + 1) % dim;
-      if (next_radix) {
-        // the children's bounds: the parent's, cut at the median's
-        // coordinate in the split dimension (left: coordinates <= v, right:
-        // >= v); and their open key bits in the next split dimension
-        for (int s = threadIdx.x; s < nseg; s += blockDim.x) {
-          const int32_t v = (int32_t)(s_res[s] >> 31);
-          for (int cc = 0; cc < dim; ++cc) {
-            const int32_t lo = bcur[(s * dim + cc) * 2], hi = bcur[(s * dim + cc) * 2 + 1];
-            bnxt[(2 * s * dim + cc) * 2] = lo;
-            bnxt[(2 * s * dim + cc) * 2 + 1] = cc == c ? v : hi;
-            bnxt[((2 * s + 1) * dim + cc) * 2] = cc == c ? v : lo;
-            bnxt[((2 * s + 1) * dim + cc) * 2 + 1] = hi;
-          }
-          for (int ch = 2 * s; ch <= 2 * s + 1; ++ch)
-            s_shn[ch] = open_key_bits(bnxt[(ch * dim + cn) * 2], bnxt[(ch * dim + cn) * 2 + 1]);
-        }
-      }
       const int ipt = (cap + blockDim.x - 1) / blockDim.x;   // 2, 4 or 8 (cap <= 8 TH)
       const int q0 = threadIdx.x * ipt;
       // this thread's positions' records and segments, read once (one vector
@@ -1155,9 +1227,8 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
               nxt[dst] = (uint16_t)CQ(j);
               segid_n[dst] = (unsigned char)(2 * s + (left ? 0 : 1));   // child segment
               if (next_radix) {   // the child's first digit, below its open key bits
-                const int ch = 2 * s + (left ? 0 : 1), sh = s_shn[ch], ns = max(0, sh - wn);
-                const uint64_t kn = skey(sc, sid, cap, cn, CQ(j));
-                const int dg = (int)((kn >> ns) & ((1u << (sh - ns)) - 1));
+                const int ch = 2 * s + (left ? 0 : 1);
+                const int dg = key_digit(sc, sid, cap, cn, CQ(j), s_sh[ch], wn);
                 binq[dst] = (uint16_t)dg;
                 wit[(ch << wn) + dg] = (uint16_t)CQ(j);
                 atomicAdd(&hist[(ch << wn) + dg], 1u);
@@ -1173,6 +1244,8 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
       hist_ready = next_radix;
       unsigned char *ts = segid; segid = segid_n; segid_n = ts;
       int32_t *tb = bcur; bcur = bnxt; bnxt = tb;
+      int32_t *tr = s_st; s_st = n_st; n_st = tr;
+      tr = s_sz; s_sz = n_sz; n_sz = tr;
     } else {
       // ---------------- warp mode: one warp splits each segment ------------
       // A segment of z <= 64 records.  Above the last level, two per lane
@@ -1191,7 +1264,7 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
       if (!slots_ready && nleaf <= (int)blockDim.x) {
         for (int x = threadIdx.x + 1; x < 2 * nleaf; x += blockDim.x) {
           const int ux = 31 - __clz(x);
-          nslot[x] = (int32_t)veb_slot(l, t0 + ux, (i0 << ux) + (x - (1 << ux)));
+          nslot[x] = veb_slot32(l, t0 + ux, ((int)i0 << ux) + (x - (1 << ux)));
         }
         slots_ready = true;
         __syncthreads();
@@ -1204,7 +1277,16 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
         uint64_t med = 0;
         if (u == U - 1) {
           const int mr = ((z + 1) >> 1) - 1;
-          if (z <= 32) {
+          // coordinates that are all different sort as (coordinate << 5 | lane)
+          // in one word, half the work of the full key
+          const int ri = lane < z ? cur[a + lane] : 0;
+          const uint32_t xs = z > 32 ? 0 : warp_sort32w(lane < z ? ((uint32_t)sc[c * cap + ri] << 5) | lane : ~0u, lane);
+          const uint32_t xp = __shfl_up_sync(0xffffffffu, xs, 1);
+          if (z <= 32 && !__any_sync(0xffffffffu, lane > 0 && lane < z && (xp >> 5) == (xs >> 5))) {
+            const int from = __shfl_sync(0xffffffffu, ri, xs & 31);
+            if (lane < z) nxt[a + lane] = (uint16_t)from;
+            med = skey(sc, sid, cap, c, __shfl_sync(0xffffffffu, from, mr));
+          } else if (z <= 32) {
             uint64_t x = lane < z ? (skey(sc, sid, cap, c, cur[a + lane]) << 13) | cur[a + lane] : ~0ull;
             x = warp_sort32(x, lane);
             if (lane < z) nxt[a + lane] = (uint16_t)(x & 8191u);
@@ -1221,34 +1303,32 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
         } else {
           const bool v0 = lane < z, v1 = 32 + lane < z;
           const int ra = v0 ? cur[a + lane] : 0, rb = v1 ? cur[a + 32 + lane] : 0;
-          const uint64_t k0 = v0 ? skey(sc, sid, cap, c, ra) : 0, k1 = v1 ? skey(sc, sid, cap, c, rb) : 0;
-          // the bits where the keys differ: OR and AND over the records
-          const uint64_t ko = (v0 ? k0 : 0) | (v1 ? k1 : 0), ka = (v0 ? k0 : ~0ull) & (v1 ? k1 : ~0ull);
-          const uint64_t all_or = ((uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)(ko >> 32)) << 32) |
-                                  __reduce_or_sync(0xffffffffu, (unsigned)ko);
-          const uint64_t all_and = ((uint64_t)__reduce_and_sync(0xffffffffu, (unsigned)(ka >> 32)) << 32) |
-                                   __reduce_and_sync(0xffffffffu, (unsigned)ka);
-          const uint64_t diff = all_or ^ all_and;
+          // the coordinate's bits first, then, where records with the median's
+          // coordinate are left over, their ids' bits
           bool c0 = v0, c1 = v1;   // still candidates for the median
           int r = ((z + 1) >> 1) - 1, n = z;
-          for (int bit = diff ? 63 - __clzll(diff) : -1; bit >= 0 && n > 1; --bit) {
-            const bool b0 = (k0 >> bit) & 1, b1 = (k1 >> bit) & 1;
-            const int cz = __popc(__ballot_sync(0xffffffffu, c0 && !b0)) + __popc(__ballot_sync(0xffffffffu, c1 && !b1));
-            if (r < cz) {
-              c0 = c0 && !b0;
-              c1 = c1 && !b1;
-              n = cz;
-            } else {
-              c0 = c0 && b0;
-              c1 = c1 && b1;
-              r -= cz;
-              n -= cz;
+          auto narrow = [&](uint32_t k0, uint32_t k1) {
+            // the bits where the candidates' words differ: OR and AND over them
+            const uint32_t all_or = __reduce_or_sync(0xffffffffu, (c0 ? k0 : 0) | (c1 ? k1 : 0));
+            const uint32_t all_and = __reduce_and_sync(0xffffffffu, (c0 ? k0 : ~0u) & (c1 ? k1 : ~0u));
+            const uint32_t diff = all_or ^ all_and;
+            for (int bit = diff ? 31 - __clz(diff) : -1; bit >= 0 && n > 1; --bit) {
+              const bool b0 = (k0 >> bit) & 1, b1 = (k1 >> bit) & 1;
+              const int cz =
+                  __popc(__ballot_sync(0xffffffffu, c0 && !b0)) + __popc(__ballot_sync(0xffffffffu, c1 && !b1));
+              const bool up = r >= cz;   // the median has a 1 here
+              c0 = c0 && b0 == up;
+              c1 = c1 && b1 == up;
+              r -= up ? cz : 0;
+              n = up ? n - cz : cz;
             }
-          }
+          };
+          narrow(v0 ? (uint32_t)sc[c * cap + ra] : 0, v1 ? (uint32_t)sc[c * cap + rb] : 0);
+          if (n > 1) narrow(v0 ? (uint32_t)sid[ra] : 0, v1 ? (uint32_t)sid[rb] : 0);
           const unsigned m0b = __ballot_sync(0xffffffffu, c0), m1b = __ballot_sync(0xffffffffu, c1);
-          med = __shfl_sync(0xffffffffu, m0b ? k0 : k1, __ffs(m0b ? m0b : m1b) - 1);
+          med = skey(sc, sid, cap, c, __shfl_sync(0xffffffffu, m0b ? ra : rb, __ffs(m0b ? m0b : m1b) - 1));
           // the split: left records first, each side in position order
-          const bool l0 = v0 && k0 <= med, l1 = v1 && k1 <= med;
+          const bool l0 = v0 && skey(sc, sid, cap, c, ra) <= med, l1 = v1 && skey(sc, sid, cap, c, rb) <= med;
           const unsigned L0 = __ballot_sync(0xffffffffu, l0), L1 = __ballot_sync(0xffffffffu, l1);
           const unsigned R0 = __ballot_sync(0xffffffffu, v0 && !l0), R1 = __ballot_sync(0xffffffffu, v1 && !l1);
           const int nl = __popc(L0) + __popc(L1);
@@ -1262,10 +1342,10 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
           if (lane == 0) o.node[nslot[x]] = Node{med, nslot[2 * x], nslot[2 * x + 1]};
         } else {
           // the node's vEB slot and its children's, three lanes at once
-          const int64_t bfs = (i0 << u) + s;
-          const int64_t sl = lane < 3 ? veb_slot(l, lane ? t + 1 : t, lane ? 2 * bfs + lane - 1 : bfs) : 0;
-          const int64_t vl = __shfl_sync(0xffffffffu, sl, 1), vr = __shfl_sync(0xffffffffu, sl, 2);
-          if (lane == 0) o.node[sl] = Node{med, (int32_t)vl, (int32_t)vr};
+          const int bfs = ((int)i0 << u) + s;
+          const int sl = lane < 3 ? veb_slot32(l, lane ? t + 1 : t, lane ? 2 * bfs + lane - 1 : bfs) : 0;
+          const int vl = __shfl_sync(0xffffffffu, sl, 1), vr = __shfl_sync(0xffffffffu, sl, 2);
+          if (lane == 0) o.node[sl] = Node{med, vl, vr};
         }
       }
       __syncthreads();
@@ -1287,7 +1367,7 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
     if (!slots_ready) {
       for (int x = threadIdx.x + 1; x < 2 * nleaf; x += blockDim.x) {
         const int u = 31 - __clz(x);
-        nslot[x] = (int32_t)veb_slot(l, t0 + u, (i0 << u) + (x - (1 << u)));
+        nslot[x] = veb_slot32(l, t0 + u, ((int)i0 << u) + (x - (1 << u)));
       }
       __syncthreads();
     }
@@ -1304,12 +1384,31 @@ __global__ void __launch_bounds__(TH, TH == kSubThreads ? 1 : 3) k_subtree(const
       o.leaf_off[leaf] = (int32_t)(start0 + a);
       if (leaf == nleaves_tree - 1) o.leaf_off[nleaves_tree] = (int32_t)T.s;
     }
+    // a leaf's records, kept in registers over the channels where they are at
+    // most 16 (the last one stands for those it does not have); lanes start at
+    // different places of their leaves, which keeps them off one bank
+    const bool few = ((m0 + nleaf - 1) >> U) <= 16;
+    uint32_t own[8];
+    if (few && has) {
+#pragma unroll
+      for (int j = 0; j < 16; j += 2) {
+        const int p0 = (j + lane) & 15, p1 = (j + 1 + lane) & 15;
+        own[j >> 1] = (uint32_t)cur[a + min(p0, z - 1)] | (uint32_t)cur[a + min(p1, z - 1)] << 16;
+      }
+    }
     const int kw = U < 5 ? U : 5;        // levels combined inside a warp
     for (int ch = -1; ch < dim; ++ch) {  // ch = -1: live counts
       int32_t lo = ch < 0 ? 0 : INT32_MAX, hi = INT32_MIN;
       if (has) {
         if (ch < 0) {
           lo = z;
+        } else if (few) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const int32_t x = sc[ch * cap + (int)((own[j >> 1] >> (16 * (j & 1))) & 0xffffu)];
+            lo = min(lo, x);
+            hi = max(hi, x);
+          }
         } else {
           for (int q = a; q < a + z; ++q) {
             const int32_t x = sc[ch * cap + cur[q]];
