@@ -497,6 +497,8 @@ int small_copy(void *dst, const void *src, size_t bytes, cudaStream_t s);
 // Zero a device buffer with a kernel (not a copy-engine memset), for the
 // same reason.
 int small_zero(void *dst, size_t bytes, cudaStream_t s);
+// h2d and small_zero (16-byte aligned) in one launch.
+int h2d_and_zero(void *dst, const void *src, size_t bytes, void *zero, size_t zero_bytes, cudaStream_t s);
 // Page-locked host scratch for readbacks, from a pool (returned by
 // pinned_put); nullptr if none can be had.
 void *pinned_get(size_t bytes);
@@ -517,9 +519,10 @@ int finish_call(bdl_forest *f, cudaStream_t s, int status);
 constexpr int64_t kSortMinQueries = 1 << 15;   // smaller batches run in input order ...
 constexpr int64_t kBatchSortMinQueries = 1 << 12;   // ... unless a batched call's small jobs
                                                    // hold this many queries together
-constexpr size_t kPinnedWords = 2048;          // a forest's pinned scratch, in int64 words
-constexpr size_t kPinnedFlags = 2040;          // insert-validation flags that fit in it
-constexpr size_t kPinnedErr = 2044;            // where the error word is read back
+constexpr size_t kPinnedWords = 4096;          // a forest's pinned scratch, in int64 words
+constexpr size_t kPinnedFlags = 4080;          // insert-validation flags that fit in it
+constexpr size_t kPinnedErr = 4084;            // where the error word is read back
+constexpr int kSmallCount = 8;                 // dev_small's word for a single erase's count, zero between calls
 constexpr int kBufOutWords = kMaxLevel + 2;    // per forest: buffer size, root live counts, error word
 int smem_subtree_capacity(int dim);
 
@@ -603,15 +606,14 @@ struct FillSeg {           // `count` work items of one kind
   int64_t count;
   const int32_t *src;      // append: coordinates in
   int32_t *dst;            // append / pool tail / iota: out
-  unsigned long long *flag;  // append: set to 1 on a coordinate off the grid
+  volatile unsigned long long *flag;  // append: [0] set to 1 on a coordinate off the grid, [1] see errw
   const int32_t *buf;      // pool tail: the forest's pool ...
   int64_t nbuf;
   const int32_t *arr;
   int64_t first;           // pool tail: range start; iota / alive: first id
   int64_t from;            // pool tail: first pool entry copied
   uint32_t *alive;         // alive: the forest's bitmap
-  const unsigned long long *errw;  // append: the forest's device error word; a set word
-                                   // sets bit 1 of *flag and its bits from bit 8 on
+  const unsigned long long *errw;  // append: the forest's device error word, copied to flag[1]
 };
 struct MarkSeg {           // one erase list of one forest
   uint32_t *alive;
@@ -643,10 +645,23 @@ struct BufSeg {            // one forest's buffer and roots
   int64_t *out;            // out[0] = new nbuf, out[1 + t] = live count of tree t,
                            // out[kMaxLevel + 1] = the forest's device error word
   const unsigned long long *errw;
+  int64_t *count, *count_out;  // if set: *count is copied to *count_out and cleared
   int32_t ntrees, pad_;
   const int32_t *roots[kMaxLevel];
 };
-size_t table_bytes(size_t nseg, size_t seg_size);
+// Segments that travel as kernel parameters instead of a device table.
+template <class T>
+struct InlineSegs;
+template <> struct InlineSegs<FillSeg> { static constexpr int n = 4; };
+template <> struct InlineSegs<MarkSeg> { static constexpr int n = 4; };
+template <> struct InlineSegs<TreeSeg> { static constexpr int n = 16; };
+template <> struct InlineSegs<BufSeg> { static constexpr int n = 1; };
+// Device bytes of the table of nseg segments, 0 where it travels as parameters.
+size_t table_bytes_of(size_t nseg, size_t seg_size, size_t inline_segs);
+template <class T>
+size_t table_bytes(size_t nseg) {
+  return table_bytes_of(nseg, sizeof(T), InlineSegs<T>::n);
+}
 int launch_fill_many(const std::vector<FillSeg> &segs, void *table, cudaStream_t s);
 int launch_erase_mark_many(const std::vector<MarkSeg> &segs, void *table, cudaStream_t s);
 int launch_bloom_build_many(const std::vector<TreeSeg> &segs, void *table,

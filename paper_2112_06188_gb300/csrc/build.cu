@@ -1977,9 +1977,8 @@ int build_trees_object(bdl_forest *af, int dim, std::vector<BuildTree> &bt,
       lv_bytes += (double)L.recs * (8.0 + 8.0 * (dim + 1));
     }
   }
-  st = h2d(plan, img.bytes.data(), img.bytes.size(), s);
-  // segment states, histograms and cursors (contiguous) start at zero
-  if (!st) st = small_zero(seg, seg_bytes + hist_bytes + cursor_bytes, s);
+  // the plan; segment states, histograms and cursors (contiguous) start at zero
+  st = h2d_and_zero(plan, img.bytes.data(), img.bytes.size(), seg, seg_bytes + hist_bytes + cursor_bytes, s);
   if (st) {
     dev_free(af, block, total, s);
     return st;

@@ -28,7 +28,7 @@ constexpr int kMapWords = 64;   // per warp: 2,048 bits
 // tombstoned).  The ids of a spatially ordered list meet in the same leaves:
 // a lane scanning its leaf alone took as long as the largest leaf (1M 2-D
 // points of 100 clusters, 100K ids: 1,065 us for the launch, this way 86).
-__device__ __forceinline__ bool scan_big_leaves(const EraseJob &F, int rs, bool big, int ti, int a, int z,
+__device__ __forceinline__ bool scan_big_leaves(const EraseJob &F, const TreeView *trees, int rs, bool big, int ti, int a, int z,
                                                 int32_t id) {
   __shared__ uint32_t s_map[4][kMapWords];
   unsigned todo = __ballot_sync(0xffffffffu, big);
@@ -49,7 +49,7 @@ __device__ __forceinline__ bool scan_big_leaves(const EraseJob &F, int rs, bool 
     __syncwarp();
     if (mine) atomicOr(&map[bit(id) >> 5], 1u << (bit(id) & 31));
     __syncwarp();
-    int32_t *pts = F.trees[t].pts + F.dim;
+    int32_t *pts = trees[t].pts + F.dim;
     int left = __popc(grp);
     for (int b = la; b < lz && left > 0; b += 128) {
       int32_t p[4];
@@ -87,19 +87,8 @@ __device__ __forceinline__ bool scan_big_leaves(const EraseJob &F, int rs, bool 
 // REC: some job keeps its packed k-NN records' live counts (the instance
 // without that code is used when none does)
 template <bool REC>
-__global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, int njobs) {
-  // every warp belongs to one job (one forest's erase list)
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= job_warp[njobs]) return;
-  int lo = 0, hi = njobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (job_warp[mid] <= w) lo = mid;
-    else hi = mid - 1;
-  }
-  const EraseJob &F = jobs[lo];
+__device__ __forceinline__ void erase_locate(const EraseJob &F, const TreeView *trees, int64_t i) {
   const int lane = threadIdx.x & 31;
-  const int64_t i = (w - job_warp[lo]) * 32 + lane;
   const int64_t n = F.n_dev ? min(*F.n_dev, F.n) : F.n;
   bool pending = i < n;
   int32_t id = pending ? F.list[i] : 0;
@@ -109,7 +98,7 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
   uint64_t maybe_mask = 0;
   if (pending) {
     for (int ti = 0; ti < F.ntrees; ++ti) {
-      const TreeView &T = F.trees[ti];
+      const TreeView &T = trees[ti];
       bool maybe = true;
       if (T.bloom) {
         int64_t blk;
@@ -137,7 +126,7 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
     if (mm) {
       ti = __ffsll((long long)mm) - 1;
       mm &= mm - 1;
-      const TreeView &T = F.trees[ti];
+      const TreeView &T = trees[ti];
       int v = 0, depth = 0;
       Node nd;
       bool ok = true;
@@ -162,7 +151,7 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
     bool hit = false;
     if (z - a <= kLaneLeaf) {
       for (int j = a; j < z; ++j) {
-        int32_t *slot = F.trees[ti].pts + (int64_t)j * rs + F.dim;
+        int32_t *slot = trees[ti].pts + (int64_t)j * rs + F.dim;
         if (*slot == id) {
           *slot = (int32_t)((uint32_t)id | kTomb);
           hit = true;
@@ -170,7 +159,7 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
         }
       }
     }
-    hit |= scan_big_leaves(F, rs, z - a > kLaneLeaf, ti, a, z, id);
+    hit |= scan_big_leaves(F, trees, rs, z - a > kLaneLeaf, ti, a, z, id);
     if (hit) {
       found = true;
       fti = ti;
@@ -183,7 +172,7 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
   // with h - d even: entry (i & 3) of the record two levels up, or (i & 1) of
   // the root's record for d = 1); lanes at the same node of the same tree add
   // up their counts first
-  const int fh = found ? F.trees[fti].h : -1;
+  const int fh = found ? trees[fti].h : -1;
   const int maxh = __reduce_max_sync(0xffffffffu, fh);
   const int rec = packed_node_ints(F.dim);
   for (int d = 0; d <= maxh; ++d) {
@@ -193,7 +182,7 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
     const int v = path[d];
     const unsigned peers = __match_any_sync(am, ((unsigned long long)fti << 32) | (uint32_t)v);
     if (lane == __ffs(peers) - 1) {
-      const TreeView &T = F.trees[fti];
+      const TreeView &T = trees[fti];
       const int cnt = __popc(peers);
       atomicSub(&T.live[v], cnt);
       if (REC && F.records && d >= 1 && ((T.h - d) & 1) == 0) {
@@ -204,6 +193,33 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
       }
     }
   }
+}
+
+// Every warp belongs to one job (one forest's erase list).
+template <bool REC>
+__global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, int njobs) {
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= job_warp[njobs]) return;
+  int lo = 0, hi = njobs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (job_warp[mid] <= w) lo = mid;
+    else hi = mid - 1;
+  }
+  erase_locate<REC>(jobs[lo], jobs[lo].trees, (w - job_warp[lo]) * 32 + (threadIdx.x & 31));
+}
+
+// One job, as kernel parameters with its tree views.
+struct EraseOne {
+  EraseJob job;
+  TreeView trees[kMaxLevel];
+};
+
+template <bool REC>
+__global__ void k_erase_locate_one(const __grid_constant__ EraseOne P) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if ((i & ~(int64_t)31) >= P.job.n) return;   // (whole warps)
+  erase_locate<REC>(P.job, P.trees, i);
 }
 
 // Ordered gather, for many forests at once: mark the live ids of the given
@@ -341,6 +357,7 @@ __global__ void k_emit_ids_many(const BitForest *f, const int64_t *pre, int nf) 
 }  // namespace
 
 size_t erase_table_bytes(const std::vector<EraseCall> &calls) {
+  if (calls.size() == 1) return 0;   // one job: no table (kernel parameters)
   size_t n = calls.size(), views = 0;
   for (const auto &c : calls) views += (size_t)c.fv->ntrees;
   return n * sizeof(EraseJob) + (n + 1) * 8 + views * sizeof(TreeView) + 64;
@@ -349,7 +366,9 @@ size_t erase_table_bytes(const std::vector<EraseCall> &calls) {
 int launch_erase_jobs(const std::vector<EraseCall> &calls, void *table,
                       cudaStream_t s) {
   const size_t n = calls.size();
-  std::vector<unsigned char> img(erase_table_bytes(calls));
+  EraseOne one;
+  std::vector<unsigned char> img(n == 1 ? sizeof(EraseJob) + 16 + kMaxLevel * sizeof(TreeView)
+                                        : erase_table_bytes(calls));
   EraseJob *jobs = (EraseJob *)img.data();
   int64_t *warp = (int64_t *)(img.data() + n * sizeof(EraseJob));
   const size_t views_off = n * sizeof(EraseJob) + (n + 1) * 8;
@@ -374,8 +393,13 @@ int launch_erase_jobs(const std::vector<EraseCall> &calls, void *table,
     warp[j + 1] = warp[j] + (J.n + 31) / 32;
   }
   if (warp[n] == 0) return BDL_OK;
-  int st = h2d(table, img.data(), img.size(), s);
-  if (st) return st;
+  if (n == 1) {
+    one.job = jobs[0];
+    memcpy(one.trees, views, v * sizeof(TreeView));
+  } else {
+    const int st = h2d(table, img.data(), img.size(), s);
+    if (st) return st;
+  }
   bool rec = false;
   for (const auto &c : calls) rec = rec || c.records;
   // algorithmic bytes per erased id: its coordinates (4d), one 32-byte bloom
@@ -399,7 +423,11 @@ int launch_erase_jobs(const std::vector<EraseCall> &calls, void *table,
   const unsigned grid = (unsigned)cdiv(warp[n] * 32, 128);
   const EraseJob *djobs = (const EraseJob *)table;
   const int64_t *jw = (const int64_t *)((char *)table + n * sizeof(EraseJob));
-  if (rec)
+  if (n == 1 && rec)
+    k_erase_locate_one<true><<<grid, 128, 0, s>>>(one);
+  else if (n == 1)
+    k_erase_locate_one<false><<<grid, 128, 0, s>>>(one);
+  else if (rec)
     k_erase_locate<true><<<grid, 128, 0, s>>>(djobs, jw, (int)n);
   else
     k_erase_locate<false><<<grid, 128, 0, s>>>(djobs, jw, (int)n);
@@ -519,7 +547,16 @@ __device__ __forceinline__ int32_t pool_entry(const FillSeg &g, int64_t k) {
   return g.arr ? g.arr[k - g.nbuf] : (int32_t)(g.first + (k - g.nbuf));
 }
 
-__global__ void k_fill_many(const FillSeg *segs, const int64_t *pre, int nseg) {
+// A launch's segments and their work prefix as kernel parameters: a call on
+// one forest has a handful, and a table in device memory costs it a copy
+// launch (about 3 us, half of it the read of host memory) before each kernel.
+template <class T>
+struct InlineTable {
+  int64_t pre[InlineSegs<T>::n + 1];
+  T seg[InlineSegs<T>::n];
+};
+
+__device__ __forceinline__ void fill_many(const FillSeg *segs, const int64_t *pre, int nseg) {
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= pre[nseg]) return;
   const int j = seg_find(pre, nseg, x);
@@ -531,8 +568,8 @@ __global__ void k_fill_many(const FillSeg *segs, const int64_t *pre, int nseg) {
       // an off-grid value is flagged and stored clamped, so that work started
       // before the flag is read back only ever sees grid coordinates
       g.dst[i] = min(max(v, 0), (1 << kCoordBits) - 1);
-      if (v < 0 || v >= (1 << kCoordBits)) atomicOr(g.flag, 1ull);
-      if (i == 0 && g.errw && *g.errw) atomicOr(g.flag, 2ull | (*g.errw << 8));   // with the word's bits
+      if (v < 0 || v >= (1 << kCoordBits)) g.flag[0] = 1;
+      if (i == 0 && g.errw) g.flag[1] = *g.errw;
       break;
     }
     case kFillPoolTail: g.dst[i] = pool_entry(g, g.from + i); break;
@@ -551,7 +588,7 @@ __global__ void k_fill_many(const FillSeg *segs, const int64_t *pre, int nseg) {
 
 // Erase marking for many forests: entries are warp-aligned, so the warp's
 // aggregated append stays inside one forest's list.
-__global__ void k_erase_mark_many(const MarkSeg *segs, const int64_t *pre_warp, int nseg) {
+__device__ __forceinline__ void erase_mark_many(const MarkSeg *segs, const int64_t *pre_warp, int nseg) {
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= pre_warp[nseg]) return;
   const int j = seg_find(pre_warp, nseg, w);
@@ -578,7 +615,7 @@ __global__ void k_erase_mark_many(const MarkSeg *segs, const int64_t *pre_warp, 
   if (own) g.list[base + __popc(m & ((1u << lane) - 1))] = id;
 }
 
-__global__ void k_bloom_build_many(const TreeSeg *segs, const int64_t *pre, int nseg) {
+__device__ __forceinline__ void bloom_build_many(const TreeSeg *segs, const int64_t *pre, int nseg) {
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= pre[nseg]) return;
   const int j = seg_find(pre, nseg, x);
@@ -600,7 +637,7 @@ __global__ void k_bloom_build_many(const TreeSeg *segs, const int64_t *pre, int 
 // tree j's records in level order): its entries' live counts from the nodes'.
 // With segs[j].err set, compare instead of copy and flag a difference (the
 // erase keeps both up to date; this is the debug check of that).
-__global__ void k_pack_lives_many(const TreeSeg *segs, const int64_t *pre, int nseg) {
+__device__ __forceinline__ void pack_lives_many(const TreeSeg *segs, const int64_t *pre, int nseg) {
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= pre[nseg]) return;
   const int j = seg_find(pre, nseg, x);
@@ -633,7 +670,7 @@ __global__ void k_pack_lives_many(const TreeSeg *segs, const int64_t *pre, int n
 
 // One CTA per forest: keep its buffer ids that are still alive, in order;
 // then the live counts of its tree roots.
-__global__ void k_buffer_compact_many(const BufSeg *segs) {
+__device__ __forceinline__ void buffer_compact_many(const BufSeg *segs, const int64_t *, int) {
   __shared__ int wsum[32];
   __shared__ int base;
   const BufSeg &g = segs[blockIdx.x];
@@ -662,52 +699,72 @@ __global__ void k_buffer_compact_many(const BufSeg *segs) {
   if (threadIdx.x == 0) {
     g.out[0] = base;
     g.out[kMaxLevel + 1] = g.errw ? (int64_t)*g.errw : 0;
+    if (g.count) {
+      *g.count_out = *g.count;
+      *g.count = 0;
+    }
   }
   for (int t = threadIdx.x; t < g.ntrees; t += blockDim.x) g.out[1 + t] = g.roots[t][0];
 }
 
-template <class T>
-int upload_table(const std::vector<T> &segs, const std::vector<int64_t> &pre, void *dev,
-                 cudaStream_t s) {
-  std::vector<unsigned char> img(table_bytes(segs.size(), sizeof(T)));
-  memcpy(img.data(), segs.data(), segs.size() * sizeof(T));
-  memcpy(img.data() + (segs.size() * sizeof(T) + 255) / 256 * 256, pre.data(), pre.size() * 8);
-  return h2d(dev, img.data(), img.size(), s);
-}
+// A kernel for each of them, over a table in device memory or in its parameters.
+#define TABLE_KERNELS(name, T)                                                                         \
+  __global__ void k_##name(const T *segs, const int64_t *pre, int nseg) { name(segs, pre, nseg); }     \
+  __global__ void k_##name##_inline(const __grid_constant__ InlineTable<T> A, int nseg) { name(A.seg, A.pre, nseg); }
+TABLE_KERNELS(fill_many, FillSeg)
+TABLE_KERNELS(erase_mark_many, MarkSeg)
+TABLE_KERNELS(bloom_build_many, TreeSeg)
+TABLE_KERNELS(pack_lives_many, TreeSeg)
+TABLE_KERNELS(buffer_compact_many, BufSeg)
+#undef TABLE_KERNELS
 
+// Launches `inl` with the segments as parameters, or uploads them to `dev`
+// and launches `tab`.
 template <class T>
-const int64_t *table_pre(const std::vector<T> &segs, const void *dev) {
-  return (const int64_t *)((const char *)dev + (segs.size() * sizeof(T) + 255) / 256 * 256);
+int launch_table(void (*tab)(const T *, const int64_t *, int), void (*inl)(const InlineTable<T>, int), int kid,
+                 double bytes, unsigned grid, unsigned threads, const std::vector<T> &segs,
+                 const std::vector<int64_t> &pre, void *dev, cudaStream_t s) {
+  if (segs.size() <= (size_t)InlineSegs<T>::n) {
+    InlineTable<T> A;
+    memcpy(A.pre, pre.data(), pre.size() * 8);
+    memcpy(A.seg, segs.data(), segs.size() * sizeof(T));
+    KScope ks_(kid, s, bytes);
+    inl<<<grid, threads, 0, s>>>(A, (int)segs.size());
+    return BDL_OK;
+  }
+  const size_t at = (segs.size() * sizeof(T) + 255) / 256 * 256;
+  std::vector<unsigned char> img(table_bytes<T>(segs.size()));
+  memcpy(img.data(), segs.data(), segs.size() * sizeof(T));
+  memcpy(img.data() + at, pre.data(), pre.size() * 8);
+  const int st = h2d(dev, img.data(), img.size(), s);
+  if (st) return st;
+  KScope ks_(kid, s, bytes);
+  tab<<<grid, threads, 0, s>>>((const T *)dev, (const int64_t *)((const char *)dev + at), (int)segs.size());
+  return BDL_OK;
 }
 
 }  // namespace
 
-size_t table_bytes(size_t nseg, size_t seg_size) {
-  return (nseg * seg_size + 255) / 256 * 256 + (nseg + 1) * 8 + 64;
+size_t table_bytes_of(size_t nseg, size_t seg_size, size_t inline_segs) {
+  return nseg <= inline_segs ? 0 : (nseg * seg_size + 255) / 256 * 256 + (nseg + 1) * 8 + 64;
 }
 
 int launch_fill_many(const std::vector<FillSeg> &segs, void *table, cudaStream_t s) {
   std::vector<int64_t> pre(segs.size() + 1, 0);
   for (size_t j = 0; j < segs.size(); ++j) pre[j + 1] = pre[j] + segs[j].count;
   if (pre.back() == 0) return BDL_OK;
-  int st = upload_table(segs, pre, table, s);
-  if (st) return st;
-  KScope ks_(kK_fill, s);
-  k_fill_many<<<(unsigned)cdiv(pre.back(), 256), 256, 0, s>>>((const FillSeg *)table,
-                                                               table_pre(segs, table), (int)segs.size());
-  return cuda_check(cudaGetLastError(), "fill kernel");
+  const int st = launch_table<FillSeg>(k_fill_many, k_fill_many_inline, kK_fill, 0, (unsigned)cdiv(pre.back(), 256),
+                                       256, segs, pre, table, s);
+  return st ? st : cuda_check(cudaGetLastError(), "fill kernel");
 }
 
 int launch_erase_mark_many(const std::vector<MarkSeg> &segs, void *table, cudaStream_t s) {
   std::vector<int64_t> pre(segs.size() + 1, 0);
   for (size_t j = 0; j < segs.size(); ++j) pre[j + 1] = pre[j] + (segs[j].n + 31) / 32;
   if (pre.back() == 0) return BDL_OK;
-  int st = upload_table(segs, pre, table, s);
-  if (st) return st;
-  KScope ks_(kK_erase_mark, s);
-  k_erase_mark_many<<<(unsigned)cdiv(pre.back() * 32, 256), 256, 0, s>>>(
-      (const MarkSeg *)table, table_pre(segs, table), (int)segs.size());
-  return cuda_check(cudaGetLastError(), "erase mark kernel");
+  const int st = launch_table<MarkSeg>(k_erase_mark_many, k_erase_mark_many_inline, kK_erase_mark, 0,
+                                       (unsigned)cdiv(pre.back() * 32, 256), 256, segs, pre, table, s);
+  return st ? st : cuda_check(cudaGetLastError(), "erase mark kernel");
 }
 
 int launch_bloom_build_many(const std::vector<TreeSeg> &segs, void *table,
@@ -715,35 +772,28 @@ int launch_bloom_build_many(const std::vector<TreeSeg> &segs, void *table,
   std::vector<int64_t> pre(segs.size() + 1, 0);
   for (size_t j = 0; j < segs.size(); ++j) pre[j + 1] = pre[j] + segs[j].size;
   if (pre.back() == 0) return BDL_OK;
-  int st = upload_table(segs, pre, table, s);
-  if (st) return st;
   // algorithmic bytes per point: its id and one 32-byte block
-  KScope ks_(kK_bloom_build, s, (double)pre.back() * 36.0);
-  k_bloom_build_many<<<(unsigned)cdiv(pre.back(), 256), 256, 0, s>>>(
-      (const TreeSeg *)table, table_pre(segs, table), (int)segs.size());
-  return cuda_check(cudaGetLastError(), "bloom kernel");
+  const int st = launch_table<TreeSeg>(k_bloom_build_many, k_bloom_build_many_inline, kK_bloom_build,
+                                       (double)pre.back() * 36.0, (unsigned)cdiv(pre.back(), 256), 256, segs, pre,
+                                       table, s);
+  return st ? st : cuda_check(cudaGetLastError(), "bloom kernel");
 }
 
 int launch_pack_lives_many(const std::vector<TreeSeg> &segs, void *table, cudaStream_t s) {
   std::vector<int64_t> pre(segs.size() + 1, 0);
   for (size_t j = 0; j < segs.size(); ++j) pre[j + 1] = pre[j] + packed_nrec(segs[j].h);
   if (pre.back() == 0) return BDL_OK;
-  int st = upload_table(segs, pre, table, s);
-  if (st) return st;
-  KScope ks_(kK_pack_lives, s);
-  k_pack_lives_many<<<(unsigned)cdiv(pre.back(), 256), 256, 0, s>>>(
-      (const TreeSeg *)table, table_pre(segs, table), (int)segs.size());
-  return cuda_check(cudaGetLastError(), "pack lives kernel");
+  const int st = launch_table<TreeSeg>(k_pack_lives_many, k_pack_lives_many_inline, kK_pack_lives, 0,
+                                       (unsigned)cdiv(pre.back(), 256), 256, segs, pre, table, s);
+  return st ? st : cuda_check(cudaGetLastError(), "pack lives kernel");
 }
 
 int launch_buffer_compact_many(const std::vector<BufSeg> &segs, void *table, cudaStream_t s) {
   if (segs.empty()) return BDL_OK;
   std::vector<int64_t> pre(segs.size() + 1, 0);
-  int st = upload_table(segs, pre, table, s);
-  if (st) return st;
-  KScope ks_(kK_buffer_compact, s);
-  k_buffer_compact_many<<<(unsigned)segs.size(), 1024, 0, s>>>((const BufSeg *)table);
-  return cuda_check(cudaGetLastError(), "buffer compact kernel");
+  const int st = launch_table<BufSeg>(k_buffer_compact_many, k_buffer_compact_many_inline, kK_buffer_compact, 0,
+                                      (unsigned)segs.size(), 1024, segs, pre, table, s);
+  return st ? st : cuda_check(cudaGetLastError(), "buffer compact kernel");
 }
 
 }  // namespace bdl

@@ -231,6 +231,14 @@ __global__ void k_zero(unsigned char *dst, size_t bytes) {
   }
 }
 
+// Both in one launch: dst[0 .. bytes) = src, zero[0 .. zero_bytes) = 0 (all
+// 16-byte aligned, sizes of dst and src rounded up inside their blocks).
+__global__ void k_copy_and_zero(const uint4 *src, uint4 *dst, size_t bytes, uint4 *zero, size_t zero_bytes) {
+  const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = i0; i * 16 < bytes; i += step) dst[i] = src[i];
+  for (size_t i = i0; i * 16 < zero_bytes; i += step) zero[i] = make_uint4(0, 0, 0, 0);
+}
+
 std::mutex g_pin_mu;
 std::vector<std::pair<void *, size_t>> g_pin_free;   // page-locked buffers not in use
 std::vector<std::pair<void *, size_t>> g_pin_used;
@@ -297,8 +305,9 @@ void pinned_put(void *p) {
     }
 }
 
-int h2d(void *dst, const void *src, size_t bytes, cudaStream_t s) {
-  if (bytes == 0) return BDL_OK;
+// h2d, with a zero fill in the same launch where `zero_bytes` > 0.
+static int upload(void *dst, const void *src, size_t bytes, void *zero, size_t zero_bytes, cudaStream_t s) {
+  if (bytes == 0) return small_zero(zero, zero_bytes, s);
   if (((uintptr_t)dst & 15) != 0) return set_error(BDL_EINTERNAL, "table not 16-byte aligned");
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   int st = cuda_check(cudaStreamIsCapturing(s, &cs), "cudaStreamIsCapturing");
@@ -311,14 +320,17 @@ int h2d(void *dst, const void *src, size_t bytes, cudaStream_t s) {
       KScope ks_(kK_put_blob, s);
       k_put_blob<<<1, 256, 0, s>>>(b, (unsigned char *)dst + o, (int)n);
     }
-    return cuda_check(cudaGetLastError(), "table upload");
+    const int e = small_zero(zero, zero_bytes, s);
+    return e ? e : cuda_check(cudaGetLastError(), "table upload");
   }
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 128) return set_error(BDL_EINVAL, "device index out of range");
   const size_t len = a256(bytes);
-  if (len > kRingBytes)   // larger than the ring: plain copy
-    return cuda_check(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s), "table upload");
+  if (len > kRingBytes) {   // larger than the ring: plain copy
+    st = cuda_check(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s), "table upload");
+    return st ? st : small_zero(zero, zero_bytes, s);
+  }
   std::lock_guard<std::mutex> lk(g_ring_mu);
   Ring &R = g_ring[dev];
   if (!R.base) {
@@ -345,7 +357,15 @@ int h2d(void *dst, const void *src, size_t bytes, cudaStream_t s) {
     }
   }
   memcpy(R.base + lo, src, bytes);
-  st = small_copy(dst, R.dbase + lo, bytes, s);   // not behind the caller's transfers on a copy engine
+  if (zero_bytes) {
+    const size_t words = std::max(bytes, zero_bytes) / 16 + 1;
+    KScope ks_(kK_small_copy, s);
+    k_copy_and_zero<<<(unsigned)std::min<size_t>((words + 255) / 256, 2048), 256, 0, s>>>(
+        (const uint4 *)(R.dbase + lo), (uint4 *)dst, bytes, (uint4 *)zero, zero_bytes);
+    st = cuda_check(cudaGetLastError(), "table upload");
+  } else {
+    st = small_copy(dst, R.dbase + lo, bytes, s);   // not behind the caller's transfers on a copy engine
+  }
   if (st) return st;
   cudaEvent_t ev = nullptr;
   if (!R.spare.empty()) {
@@ -367,6 +387,12 @@ int h2d(void *dst, const void *src, size_t bytes, cudaStream_t s) {
   R.busy.push_back(Ring::Use{lo, len, ev});
   R.head = hi;
   return BDL_OK;
+}
+
+int h2d(void *dst, const void *src, size_t bytes, cudaStream_t s) { return upload(dst, src, bytes, nullptr, 0, s); }
+
+int h2d_and_zero(void *dst, const void *src, size_t bytes, void *zero, size_t zero_bytes, cudaStream_t s) {
+  return upload(dst, src, bytes, zero, zero_bytes, s);
 }
 
 // Static trees of a forest without an hbm budget are laid out for their
@@ -718,6 +744,8 @@ struct Temp {
   std::vector<std::pair<void *, size_t>> blocks;
   Temp(bdl_forest *f_, cudaStream_t s_) : f(f_), s(s_) {}
   int get(size_t bytes, void **p) {
+    *p = nullptr;
+    if (bytes == 0) return BDL_OK;
     int st = dev_alloc(f, p, bytes, s);
     if (!st) blocks.push_back({*p, bytes});
     return st;
@@ -762,7 +790,7 @@ static int build_planned(std::vector<InsertPlan> &plans, std::vector<BuildTree> 
   for (auto &ip : plans)
     if (ip.f && (ip.q > 0 ? ip.rem > 0 : ip.n > 0)) fills.push_back(tail_fill(ip));
   void *table = nullptr;
-  if (!st && !fills.empty()) st = tmp.get(table_bytes(fills.size(), sizeof(FillSeg)), &table);
+  if (!st && !fills.empty()) st = tmp.get(table_bytes<FillSeg>(fills.size()), &table);
   if (!st && !fills.empty()) st = launch_fill_many(fills, table, s);
   if (st)
     for (auto &ip : plans) drop_plan(ip, s);
@@ -775,7 +803,7 @@ static int commit_planned(std::vector<InsertPlan> &plans, std::vector<FillSeg> f
                           cudaStream_t s) {
   int st = BDL_OK;
   void *table = nullptr;
-  if (!fills.empty()) st = tmp.get(table_bytes(fills.size(), sizeof(FillSeg)), &table);
+  if (!fills.empty()) st = tmp.get(table_bytes<FillSeg>(fills.size()), &table);
   if (!st && !fills.empty()) st = launch_fill_many(fills, table, s);
   if (st) {
     for (auto &ip : plans) drop_plan(ip, s);
@@ -921,27 +949,30 @@ static int insert_many(bdl_forest *const *F, int nf, const int32_t *const *pts, 
     app.push_back(g);
   }
   if (app.empty()) return BDL_OK;
-  void *flags = nullptr, *table = nullptr;
-  st = tmp.get(app.size() * 8, &flags);
-  if (!st) st = tmp.get(table_bytes(app.size(), sizeof(FillSeg)), &table);
-  if (st) return st;
-  for (size_t j = 0; j < app.size(); ++j) app[j].flag = (unsigned long long *)flags + j;
-  small_zero(flags, app.size() * 8, s);
-  st = launch_fill_many(app, table, s);
   // The append stores off-grid coordinates clamped onto the grid and flags
-  // them.  With room for the flags in the forest's pinned scratch, the build
-  // goes ahead without waiting: it only ever sees grid coordinates, and its
-  // result is installed after the flags have come back clean (else dropped:
-  // nothing it wrote is reachable from the forest).  Without room, wait first.
+  // them.  With room for the flags (two words per entry) in the forest's
+  // pinned scratch, which the kernel writes directly, the build goes ahead
+  // without waiting: it only ever sees grid coordinates, and its result is
+  // installed after the flags have come back clean (else dropped: nothing it
+  // wrote is reachable from the forest).  Without room, wait first.
+  const size_t nflag = 2 * app.size();
+  const bool ahead = nflag <= kPinnedFlags;
   int64_t *hf = F[0]->pinned;
-  const bool ahead = app.size() <= kPinnedFlags;
   std::vector<int64_t> hf_big;
-  if (!ahead) {
-    hf_big.resize(app.size());
+  void *flags = F[0]->pinned_dev, *table = nullptr;
+  if (ahead) {
+    memset(hf, 0, nflag * 8);
+  } else {
+    hf_big.resize(nflag);
     hf = hf_big.data();
+    st = tmp.get(nflag * 8, &flags);
+    if (!st) st = small_zero(flags, nflag * 8, s);
   }
-  if (!st && ahead) st = small_copy(F[0]->pinned_dev, flags, app.size() * 8, s);   // the forest's mapped scratch
-  if (!st && !ahead) st = cuda_check(cudaMemcpyAsync(hf, flags, app.size() * 8, cudaMemcpyDeviceToHost, s), "copy");
+  if (!st) st = tmp.get(table_bytes<FillSeg>(app.size()), &table);
+  if (st) return st;
+  for (size_t j = 0; j < app.size(); ++j) app[j].flag = (unsigned long long *)flags + 2 * j;
+  st = launch_fill_many(app, table, s);
+  if (!st && !ahead) st = cuda_check(cudaMemcpyAsync(hf, flags, nflag * 8, cudaMemcpyDeviceToHost, s), "copy");
   if (!st && ahead) {
     if (!F[0]->ev_flags) st = cuda_check(cudaEventCreateWithFlags(&F[0]->ev_flags, cudaEventDisableTiming),
                                          "cudaEventCreate");
@@ -949,22 +980,21 @@ static int insert_many(bdl_forest *const *F, int nf, const int32_t *const *pts, 
   }
   if (!st && !ahead) st = cuda_check(cudaStreamSynchronize(s), "cudaStreamSynchronize");
   if (st) return st;
-  // flag bit 0: a coordinate off the grid; bit 1: the forest's device error
-  // word was set by earlier work (a kernel found an index outside its
-  // buffers), whose bits follow from bit 8 on
+  // word 0: a coordinate off the grid; word 1: the forest's device error word
+  // as earlier work left it (a kernel found an index outside its buffers)
   auto off_grid = [&]() {
     for (size_t j = 0; j < app.size(); ++j)
-      if (hf[j] & 1) return true;
+      if (hf[2 * j]) return true;
     return false;
   };
   auto dev_error = [&]() {
     for (size_t j = 0; j < app.size(); ++j)
-      if (hf[j] & 2) return true;
+      if (hf[2 * j + 1]) return true;
     return false;
   };
   auto dev_error_msg = [&]() {
     uint64_t bits = 0;
-    for (size_t j = 0; j < app.size(); ++j) bits |= (uint64_t)hf[j] >> 8;
+    for (size_t j = 0; j < app.size(); ++j) bits |= (uint64_t)hf[2 * j + 1];
     return std::string("device error word set by earlier work, code ") + std::to_string(bits);
   };
   if (!ahead && dev_error()) return set_error(BDL_EINTERNAL, dev_error_msg());
@@ -1067,10 +1097,21 @@ static int erase_core(bdl_forest *const *F, int nf, const std::vector<EraseList>
     if (L[j].n > 0 && fa[L[j].forest] >= 0) use.push_back((int)j), total += L[j].n;
   // device counts: one per list taking part, then one total per active forest
   void *lists = nullptr, *counts = nullptr, *table = nullptr;
+  // (one list: a word of the forest that is zero between calls, cleared again
+  // by the compaction, the call's last kernel, or here if that did not run)
+  const bool single = use.size() == 1;
+  struct CountGuard {
+    int64_t *word;
+    cudaStream_t s;
+    ~CountGuard() {
+      if (word) small_zero(word, 8, s);
+    }
+  } count_guard{nullptr, s};
   int st = tmp.get((size_t)total * 4, &lists);
-  if (!st) st = tmp.get((use.size() + na) * 8, &counts);
-  if (!st) st = tmp.get(table_bytes(use.size(), sizeof(MarkSeg)), &table);
+  if (!st && !single) st = tmp.get((use.size() + na) * 8, &counts);
+  if (!st) st = tmp.get(table_bytes<MarkSeg>(use.size()), &table);
   if (st) return st;
+  if (single) counts = F[act_forest[0]]->dev_small + kSmallCount;
   int64_t *lcount = (int64_t *)counts;                 // [use.size()]
   int64_t *ftotal = lcount + use.size();               // [na]
   std::vector<int32_t *> lptr(use.size());
@@ -1084,7 +1125,8 @@ static int erase_core(bdl_forest *const *F, int nf, const std::vector<EraseList>
     rank[u] = seen[e.forest]++;
     nrank = std::max(nrank, rank[u] + 1);
   }
-  small_zero(counts, (use.size() + na) * 8, s);
+  if (single) count_guard.word = lcount;
+  else small_zero(counts, (use.size() + na) * 8, s);
   for (int r = 0; r < nrank && !st; ++r) {
     std::vector<MarkSeg> mk;
     for (size_t u = 0; u < use.size(); ++u) {
@@ -1148,13 +1190,13 @@ static int erase_core(bdl_forest *const *F, int nf, const std::vector<EraseList>
   if (st) return st;
   if (!zeros.empty()) {
     void *zt = nullptr;
-    st = tmp.get(table_bytes(zeros.size(), sizeof(FillSeg)), &zt);
+    st = tmp.get(table_bytes<FillSeg>(zeros.size()), &zt);
     if (!st) st = launch_fill_many(zeros, zt, s);
     if (st) return st;
   }
   if (!blooms.empty()) {
     void *bt = nullptr;
-    st = tmp.get(table_bytes(blooms.size(), sizeof(TreeSeg)), &bt);
+    st = tmp.get(table_bytes<TreeSeg>(blooms.size()), &bt);
     if (!st) st = launch_bloom_build_many(blooms, bt, s);
     if (st) return st;
   }
@@ -1196,8 +1238,16 @@ static int erase_core(bdl_forest *const *F, int nf, const std::vector<EraseList>
   //    descent kept them); compact the buffers; counts back
   std::vector<TreeSeg> lives;
   std::vector<BufSeg> bufs;
-  void *outs = nullptr;
-  st = tmp.get(na * kBufOutWords * 8, &outs);
+  // the counts come back through page-locked memory that the kernels write
+  // (not behind the caller's transfers on a copy engine)
+  const size_t nho = na * kBufOutWords, nhc = use.size() + na;
+  struct PinGuard {
+    void *p;
+    ~PinGuard() { pinned_put(p); }
+  } pin{pinned_get((nho + nhc) * 8)};
+  int64_t *pin_dev = pin.p ? (int64_t *)mapped(pin.p) : nullptr;
+  void *outs = pin_dev;
+  if (!pin_dev) st = tmp.get((nho + nhc) * 8, &outs);
   if (st) return st;
   for (size_t a = 0; a < na; ++a) {
     bdl_forest *f = F[act_forest[a]];
@@ -1208,6 +1258,10 @@ static int erase_core(bdl_forest *const *F, int nf, const std::vector<EraseList>
     b.alive = f->alive;
     b.out = (int64_t *)outs + a * kBufOutWords;
     b.errw = f->err;
+    if (single) {
+      b.count = lcount;
+      b.count_out = (int64_t *)outs + nho;
+    }
     for (int i = kMaxLevel - 1; i >= 0; --i) {
       Tree *t = f->trees[i];
       if (!t) continue;
@@ -1227,35 +1281,25 @@ static int erase_core(bdl_forest *const *F, int nf, const std::vector<EraseList>
   }
   void *lt = nullptr, *bt2 = nullptr;
   if (!lives.empty()) {
-    st = tmp.get(table_bytes(lives.size(), sizeof(TreeSeg)), &lt);
+    st = tmp.get(table_bytes<TreeSeg>(lives.size()), &lt);
     if (!st) st = launch_pack_lives_many(lives, lt, s);
     if (st) return st;
   }
-  st = tmp.get(table_bytes(bufs.size(), sizeof(BufSeg)), &bt2);
+  st = tmp.get(table_bytes<BufSeg>(bufs.size()), &bt2);
   if (!st) st = launch_buffer_compact_many(bufs, bt2, s);
-  // counts back through page-locked scratch written by a kernel (not behind
-  // the caller's transfers on a copy engine)
-  const size_t nho = na * kBufOutWords, nhc = use.size() + na;
-  struct PinGuard {
-    void *p;
-    ~PinGuard() { pinned_put(p); }
-  } pin{pinned_get((nho + nhc) * 8)};
-  std::vector<int64_t> ho_v, hc_v;
-  int64_t *ho, *hc;
-  int64_t *pin_dev = pin.p ? (int64_t *)mapped(pin.p) : nullptr;
+  if (!st) count_guard.word = nullptr;
+  std::vector<int64_t> back;
+  const int64_t *ho = (const int64_t *)pin.p;
   if (pin_dev) {
-    ho = (int64_t *)pin.p;
-    hc = ho + nho;
-    if (!st) st = small_copy(pin_dev, outs, nho * 8, s);
-    if (!st) st = small_copy(pin_dev + nho, counts, nhc * 8, s);
+    if (!st && !single) st = small_copy(pin_dev + nho, counts, nhc * 8, s);
   } else {
-    ho_v.resize(nho);
-    hc_v.resize(nhc);
-    ho = ho_v.data();
-    hc = hc_v.data();
-    if (!st) st = cuda_check(cudaMemcpyAsync(ho, outs, nho * 8, cudaMemcpyDeviceToHost, s), "copy");
-    if (!st) st = cuda_check(cudaMemcpyAsync(hc, counts, nhc * 8, cudaMemcpyDeviceToHost, s), "copy");
+    back.resize(nho + nhc);
+    ho = back.data();
+    if (!st) st = cuda_check(cudaMemcpyAsync(back.data(), outs, (nho + single) * 8, cudaMemcpyDeviceToHost, s), "copy");
+    if (!st && !single)
+      st = cuda_check(cudaMemcpyAsync(back.data() + nho, counts, nhc * 8, cudaMemcpyDeviceToHost, s), "copy");
   }
+  const int64_t *hc = ho + nho;
   if (!st) st = cuda_check(cudaStreamSynchronize(s), "cudaStreamSynchronize");
   if (st) return st;
   // 5. new counts; trees below half capacity are emptied and their points
