@@ -452,6 +452,7 @@ struct bdl_forest {
   bdl::Tree *trees[bdl::kMaxLevel] = {};
   bdl::Tree *btree = nullptr;    // kd-tree over the buffer's points (k-NN only), built lazily
   bool buf_dirty = true;         // the buffer changed since btree was built
+  bool buf_scanned = false;      // ... and a k-NN call has scanned it since (see knn_many)
   uint64_t F = 0;
   int64_t live = 0;              // host mirror of the live count
   int64_t bytes_in_use = 0;

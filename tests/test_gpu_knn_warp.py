@@ -114,3 +114,27 @@ def test_thread_kernel_gives_the_same_rows(dim, m):
         gi, gd = f.knn(q.repeat(4, 1), 16)
         assert torch.equal(gi, wi) and torch.equal(gd, wd)
     assert f.poll_error() == 0
+
+
+@pytest.mark.parametrize("dim,X,n", [(2, 1024, 1023), (3, 64, 5_000), (5, 1024, 20_700), (7, 2048, 33)])
+def test_buffer_scanned_first_then_searched(dim, X, n):
+    """The first small call after an update scans the buffer, the next one
+    searches its tree; both again after the next update."""
+    from paper_2112_06188_gb300.forest import Forest, knn_batch
+    f, live = Forest(dim, buffer_size=X), inputs.LiveSet(dim)
+    for step in range(3):
+        p = inputs.uniform_points(n if step == 0 else 17, dim, 5 + step)
+        f.insert(dev(p))
+        live.insert(p)
+        if step == 2:
+            gone = live.live_ids()[-5:]
+            assert f.erase(dev(gone)) == live.erase(gone)
+        assert len(f.buffer_ids()) > 0
+        lp, ids = live.live_points()
+        q = np.concatenate([inputs.queries_from(lp, 20, 1), inputs.uniform_points(13, dim, 2)])
+        bi, bd = bruteforce_knn_threads(lp, ids, q, 9)
+        for call in range(3):
+            got = [f.knn(dev(q), 9)] if call != 1 else knn_batch([f, f], [dev(q), dev(q)], 9)
+            for gi, gd in got:
+                assert np.array_equal(gi.cpu().numpy(), bi) and np.array_equal(gd.cpu().numpy(), bd)
+    assert f.poll_error() == 0
