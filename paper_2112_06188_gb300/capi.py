@@ -5,6 +5,7 @@ same arguments (device pointers as Python ints, the stream as an int handle);
 all computation happens in the CUDA library.  Loading fails loudly if the
 library has not been built: there is no fallback.
 """
+import array
 import ctypes
 import os
 
@@ -200,11 +201,15 @@ def bdl_knn_noalloc(f, q_dev, m, k, out_ids_dev, out_d2_dev, stream):
 
 
 def _ptr_array(xs):
-    return (ctypes.c_void_p * max(len(xs), 1))(*[x or None for x in xs])
+    """A C array of pointers (None: NULL).  Filled through array.array: ctypes
+    converts item by item, ten times slower."""
+    a = array.array("Q", [x or 0 for x in xs] or [0])
+    return (ctypes.c_void_p * len(a)).from_buffer(a)
 
 
 def _i64_array(xs):
-    return (ctypes.c_int64 * max(len(xs), 1))(*xs)
+    a = array.array("q", xs or [0])
+    return (ctypes.c_int64 * len(a)).from_buffer(a)
 
 
 def bdl_insert_batch(forests, pts_dev, n, out_ids_dev, stream):
@@ -218,7 +223,7 @@ def bdl_erase_batch(forests, ids_dev, n, stream):
     out = (ctypes.c_int64 * max(len(forests), 1))()
     st = load().bdl_erase_batch(_ptr_array(forests), len(forests), _ptr_array(ids_dev),
                                 _i64_array(n), out, stream)
-    return st, [int(out[i]) for i in range(len(forests))]
+    return st, out[:len(forests)]
 
 
 def bdl_knn_batch(forests, q_dev, m, k, out_ids_dev, out_d2_dev, stream):

