@@ -1669,30 +1669,50 @@ int deepened_g(const BuildTree &b, int gmax, int e, int tile) {
   return g;
 }
 
-// Extra global levels for the trees with fewer than the deepest one's: the
-// global kernel runs gmax levels anyway, so splitting such a tree further
-// costs only its records' passes, and its smaller subtrees can fill the last
-// wave of the subtree launch (one CTA per SM, often a few left over).  Of
-// 0, 1, 2 or as many extra levels as allowed (the same for every such tree),
-// the one with the shortest schedule under subtree_cost is applied.
-void balance_subtrees(std::vector<BuildTree> &bt, int gmax, int slots, int tile) {
-  if (gmax == 0) return;
-  double best = 0;
-  int best_e = 0;
-  for (int e : {0, 1, 2, 64}) {
-    std::vector<double> c;
-    for (const auto &b : bt) {
-      const int g = deepened_g(b, gmax, e, tile);
-      const double x = subtree_cost(ceil_div(b.s, (int64_t)1 << g), b.h - g);
-      c.insert(c.end(), (size_t)1 << g, x);
+// The number of global levels of every tree, given the fewest that bring its
+// subtrees on chip (b.g, at most gmax).  More of them split subtrees further:
+//  * for trees with fewer levels than the deepest one the global kernel runs
+//    the levels anyway, so splitting such a tree further costs only its
+//    records' passes, and its smaller subtrees can fill the last wave of the
+//    subtree launch (one CTA per SM, often a few left over);
+//  * a build whose subtrees leave most SMs idle takes one level more for
+//    everyone and halves the subtrees, where they hold more than 6,144 records
+//    and still run in one wave (insert of 8,192 2-D points 224 -> 208 us, of
+//    100,000 3-D ones 336 -> 323; from smaller subtrees, 5,000 3-D points 185
+//    -> 190, or into a second wave, 1M 3-D points 498 -> 507, it is slower).
+// Of 0, 1, 2 or as many extra levels as allowed (the same for every tree),
+// with the deepest tree's count as it is or one more, the choice with the
+// shortest schedule under subtree_cost and the levels' own cost is applied.
+// A level costs about 1.3 units of subtree_cost (13.7 us) for its barriers,
+// the first one 0.7 more, and 0.9 units per million records.
+int balance_subtrees(std::vector<BuildTree> &bt, int gmax, int slots, int tile) {
+  double best = 0, recs = 0;
+  int best_e = 0, best_top = gmax;
+  for (const auto &b : bt) recs += (double)b.s;
+  for (int top = gmax; top <= gmax + 1; ++top)
+    for (int e : {0, 1, 2, 64}) {
+      if (top == 0 && e > 0) continue;   // (no level to go to)
+      std::vector<double> c;
+      int most = 0;
+      int64_t largest = 0;
+      for (const auto &b : bt) {
+        const int g = deepened_g(b, top, e, tile);
+        most = std::max(most, g);
+        largest = std::max(largest, ceil_div(b.s, (int64_t)1 << b.g));
+        const double x = subtree_cost(ceil_div(b.s, (int64_t)1 << g), b.h - g);
+        c.insert(c.end(), (size_t)1 << g, x);
+      }
+      if (most != top) continue;         // the same as with fewer levels
+      if (top > gmax && (largest <= 6144 || (int64_t)c.size() > slots)) continue;
+      const double ms = schedule_makespan(std::move(c), slots) + most * (1.3 + 0.9e-6 * recs) + (most ? 0.7 : 0);
+      if ((top == gmax && e == 0) || ms < best * 0.99) {
+        best = ms;
+        best_e = e;
+        best_top = top;
+      }
     }
-    const double ms = schedule_makespan(std::move(c), slots);
-    if (e == 0 || ms < best * 0.99) {
-      best = ms;
-      best_e = e;
-    }
-  }
-  for (auto &b : bt) b.g = deepened_g(b, gmax, best_e, tile);
+  for (auto &b : bt) b.g = deepened_g(b, best_top, best_e, tile);
+  return best_top;
 }
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
@@ -1764,7 +1784,7 @@ int build_trees_object(bdl_forest *af, int dim, std::vector<BuildTree> &bt,
       const int v = atoi(e);
       if (v > 0) sms = v;
     }
-    balance_subtrees(bt, gmax, std::max(sms, 1), tile);   // one subtree CTA per SM (its shared memory)
+    gmax = balance_subtrees(bt, gmax, std::max(sms, 1), tile);   // one subtree CTA per SM (its shared memory)
   }
 
   // ---- plan arrays ----
