@@ -573,6 +573,7 @@ struct EraseCall {
   uint64_t seed;           // the forest's bloom hash seed
   const int64_t *n_dev;    // if set: the list's length on the device (<= n)
   int records;             // 1: also keep the packed k-NN records' live counts current
+  bool spatial;            // its trees split at the spatial median (leaves of any size)
 };
 struct EraseJob {          // device form of an EraseCall
   const TreeView *trees;

@@ -28,7 +28,7 @@ constexpr int kMapWords = 64;   // per warp: 2,048 bits
 // tombstoned).  The ids of a spatially ordered list meet in the same leaves:
 // a lane scanning its leaf alone took as long as the largest leaf (1M 2-D
 // points of 100 clusters, 100K ids: 1,065 us for the launch, this way 86).
-__device__ __forceinline__ bool scan_big_leaves(const EraseJob &F, const TreeView *trees, int rs, bool big, int ti, int a, int z,
+__device__ __forceinline__ bool scan_big_leaves(const EraseJob &F, int rs, bool big, int ti, int a, int z,
                                                 int32_t id) {
   __shared__ uint32_t s_map[4][kMapWords];
   unsigned todo = __ballot_sync(0xffffffffu, big);
@@ -49,7 +49,7 @@ __device__ __forceinline__ bool scan_big_leaves(const EraseJob &F, const TreeVie
     __syncwarp();
     if (mine) atomicOr(&map[bit(id) >> 5], 1u << (bit(id) & 31));
     __syncwarp();
-    int32_t *pts = trees[t].pts + F.dim;
+    int32_t *pts = F.trees[t].pts + F.dim;
     int left = __popc(grp);
     for (int b = la; b < lz && left > 0; b += 128) {
       int32_t p[4];
@@ -86,8 +86,11 @@ __device__ __forceinline__ bool scan_big_leaves(const EraseJob &F, const TreeVie
 // the path.  A live id that no tree holds is in the buffer.
 // REC: some job keeps its packed k-NN records' live counts (the instance
 // without that code is used when none does)
-template <bool REC>
-__device__ __forceinline__ void erase_locate(const EraseJob &F, const TreeView *trees, int64_t i) {
+// BIG: some job's forest may have leaves of more than kLaneLeaf points (the
+// spatial median); the instance without that code keeps more warps resident
+// (512 forests: 359 us, with it 437).
+template <bool REC, bool BIG>
+__device__ __forceinline__ void erase_locate(const EraseJob &F, int64_t i) {
   const int lane = threadIdx.x & 31;
   const int64_t n = F.n_dev ? min(*F.n_dev, F.n) : F.n;
   bool pending = i < n;
@@ -98,7 +101,7 @@ __device__ __forceinline__ void erase_locate(const EraseJob &F, const TreeView *
   uint64_t maybe_mask = 0;
   if (pending) {
     for (int ti = 0; ti < F.ntrees; ++ti) {
-      const TreeView &T = trees[ti];
+      const TreeView &T = F.trees[ti];
       bool maybe = true;
       if (T.bloom) {
         int64_t blk;
@@ -121,58 +124,75 @@ __device__ __forceinline__ void erase_locate(const EraseJob &F, const TreeView *
   int64_t leaf_at = 0;    // its leaf's index among that tree's 2^h leaves
   uint64_t mm = pending ? maybe_mask : 0;
   const int rs = rec_ints(F.dim);
-  while (__any_sync(0xffffffffu, mm != 0)) {
-    int ti = -1, leaf = 0, a = 0, z = 0;
-    if (mm) {
+  // one tree: down to the id's leaf [a, z) of it, then through its points
+  auto descend = [&](const TreeView &T, int &a, int &z) {
+    int v = 0, depth = 0;
+    Node nd;
+    bool ok = true;
+    while (true) {
+      path[depth] = v;
+      nd = T.node[v];
+      if (nd.l < 0) break;
+      uint64_t key = comp_key(xq[depth % F.dim], id);
+      v = key > nd.key ? nd.r : nd.l;
+      depth++;
+      if (v < 0 || v >= T.nnodes || depth > T.h) { ok = false; break; }
+    }
+    const int leaf = -1 - nd.l;
+    if (ok && leaf < ((int64_t)1 << T.h)) {
+      a = T.leaf_off[leaf];
+      z = T.leaf_off[leaf + 1];
+      if (a < 0 || z > T.size || a > z) { a = z = 0; atomicOr(F.err, kErrLeaf); }
+    } else {
+      atomicOr(F.err, kErrChild);
+    }
+    return leaf;
+  };
+  auto scan = [&](const TreeView &T, int a, int z) {
+    for (int j = a; j < z; ++j) {
+      int32_t *slot = T.pts + (int64_t)j * rs + F.dim;
+      if (*slot == id) {
+        *slot = (int32_t)((uint32_t)id | kTomb);
+        return true;
+      }
+    }
+    return false;
+  };
+  do {
+    bool big = false;     // stopped at a leaf that the whole warp scans
+    int ti = 0, leaf = 0, a = 0, z = 0;
+    while (mm) {
       ti = __ffsll((long long)mm) - 1;
       mm &= mm - 1;
-      const TreeView &T = trees[ti];
-      int v = 0, depth = 0;
-      Node nd;
-      bool ok = true;
-      while (true) {
-        path[depth] = v;
-        nd = T.node[v];
-        if (nd.l < 0) break;
-        uint64_t key = comp_key(xq[depth % F.dim], id);
-        v = key > nd.key ? nd.r : nd.l;
-        depth++;
-        if (v < 0 || v >= T.nnodes || depth > T.h) { ok = false; break; }
+      const TreeView &T = F.trees[ti];
+      a = z = 0;
+      leaf = descend(T, a, z);
+      if (BIG && z - a > kLaneLeaf) {
+        big = true;
+        break;
       }
-      leaf = -1 - nd.l;
-      if (ok && leaf < ((int64_t)1 << T.h)) {
-        a = T.leaf_off[leaf];
-        z = T.leaf_off[leaf + 1];
-        if (a < 0 || z > T.size || a > z) { a = z = 0; atomicOr(F.err, kErrLeaf); }
-      } else {
-        atomicOr(F.err, kErrChild);
+      found = scan(T, a, z);
+      if (found) {
+        fti = ti;
+        leaf_at = leaf;
+        break;
       }
     }
-    bool hit = false;
-    if (z - a <= kLaneLeaf) {
-      for (int j = a; j < z; ++j) {
-        int32_t *slot = trees[ti].pts + (int64_t)j * rs + F.dim;
-        if (*slot == id) {
-          *slot = (int32_t)((uint32_t)id | kTomb);
-          hit = true;
-          break;
-        }
-      }
-    }
-    hit |= scan_big_leaves(F, trees, rs, z - a > kLaneLeaf, ti, a, z, id);
-    if (hit) {
+    if (!BIG || !__any_sync(0xffffffffu, big)) break;
+    if (found) mm = 0;
+    if (scan_big_leaves(F, rs, big, ti, a, z, id)) {
       found = true;
       fti = ti;
       leaf_at = leaf;
       mm = 0;
     }
-  }
+  } while (true);
   // live counts on the path: the nodes', and (when the job keeps them) the
   // packed k-NN record entries' for the nodes that are entries (depth d >= 1
   // with h - d even: entry (i & 3) of the record two levels up, or (i & 1) of
   // the root's record for d = 1); lanes at the same node of the same tree add
   // up their counts first
-  const int fh = found ? trees[fti].h : -1;
+  const int fh = found ? F.trees[fti].h : -1;
   const int maxh = __reduce_max_sync(0xffffffffu, fh);
   const int rec = packed_node_ints(F.dim);
   for (int d = 0; d <= maxh; ++d) {
@@ -182,7 +202,7 @@ __device__ __forceinline__ void erase_locate(const EraseJob &F, const TreeView *
     const int v = path[d];
     const unsigned peers = __match_any_sync(am, ((unsigned long long)fti << 32) | (uint32_t)v);
     if (lane == __ffs(peers) - 1) {
-      const TreeView &T = trees[fti];
+      const TreeView &T = F.trees[fti];
       const int cnt = __popc(peers);
       atomicSub(&T.live[v], cnt);
       if (REC && F.records && d >= 1 && ((T.h - d) & 1) == 0) {
@@ -196,7 +216,7 @@ __device__ __forceinline__ void erase_locate(const EraseJob &F, const TreeView *
 }
 
 // Every warp belongs to one job (one forest's erase list).
-template <bool REC>
+template <bool REC, bool BIG>
 __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, int njobs) {
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= job_warp[njobs]) return;
@@ -206,7 +226,7 @@ __global__ void k_erase_locate(const EraseJob *jobs, const int64_t *job_warp, in
     if (job_warp[mid] <= w) lo = mid;
     else hi = mid - 1;
   }
-  erase_locate<REC>(jobs[lo], jobs[lo].trees, (w - job_warp[lo]) * 32 + (threadIdx.x & 31));
+  erase_locate<REC, BIG>(jobs[lo], (w - job_warp[lo]) * 32 + (threadIdx.x & 31));
 }
 
 // One job, as kernel parameters with its tree views.
@@ -215,11 +235,13 @@ struct EraseOne {
   TreeView trees[kMaxLevel];
 };
 
-template <bool REC>
+template <bool REC, bool BIG>
 __global__ void k_erase_locate_one(const __grid_constant__ EraseOne P) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if ((i & ~(int64_t)31) >= P.job.n) return;   // (whole warps)
-  erase_locate<REC>(P.job, P.trees, i);
+  EraseJob J = P.job;
+  J.trees = P.trees;
+  erase_locate<REC, BIG>(J, i);
 }
 
 // Ordered gather, for many forests at once: mark the live ids of the given
@@ -423,14 +445,18 @@ int launch_erase_jobs(const std::vector<EraseCall> &calls, void *table,
   const unsigned grid = (unsigned)cdiv(warp[n] * 32, 128);
   const EraseJob *djobs = (const EraseJob *)table;
   const int64_t *jw = (const int64_t *)((char *)table + n * sizeof(EraseJob));
-  if (n == 1 && rec)
-    k_erase_locate_one<true><<<grid, 128, 0, s>>>(one);
-  else if (n == 1)
-    k_erase_locate_one<false><<<grid, 128, 0, s>>>(one);
-  else if (rec)
-    k_erase_locate<true><<<grid, 128, 0, s>>>(djobs, jw, (int)n);
-  else
-    k_erase_locate<false><<<grid, 128, 0, s>>>(djobs, jw, (int)n);
+  bool big = false;
+  for (const auto &c : calls) big = big || c.spatial;
+  if (n == 1) {
+    void (*fn)(EraseOne) = rec ? (big ? k_erase_locate_one<true, true> : k_erase_locate_one<true, false>)
+                               : (big ? k_erase_locate_one<false, true> : k_erase_locate_one<false, false>);
+    fn<<<grid, 128, 0, s>>>(one);
+  } else {
+    void (*fn)(const EraseJob *, const int64_t *, int) =
+        rec ? (big ? k_erase_locate<true, true> : k_erase_locate<true, false>)
+            : (big ? k_erase_locate<false, true> : k_erase_locate<false, false>);
+    fn<<<grid, 128, 0, s>>>(djobs, jw, (int)n);
+  }
   return cuda_check(cudaGetLastError(), "erase kernel");
 }
 

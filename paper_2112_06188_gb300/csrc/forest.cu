@@ -1227,7 +1227,8 @@ static int erase_core(bdl_forest *const *F, int nf, const std::vector<EraseList>
         order = (const int32_t *)sorted;
       }
     }
-    calls.push_back(EraseCall{&views[a], order, nj, f->cfg.hash_seed, lcount + u, incremental[a]});
+    calls.push_back(EraseCall{&views[a], order, nj, f->cfg.hash_seed, lcount + u, incremental[a],
+                              f->cfg.split_rule == BDL_SPLIT_SPATIAL});
   }
   {
     void *et = nullptr;
