@@ -105,12 +105,21 @@ __host__ __device__ inline int64_t veb_slot(int l, int t, int64_t i) {
   return off;
 }
 
-// veb_slot in 32-bit arithmetic (nodes are numbered in 31 bits): the smallest
-// power of two >= l/2 is the highest one in l - 1.
-__device__ inline int veb_slot32(int l, int t, int i) {
+// Position of the highest set bit of x > 0.
+__host__ __device__ inline int high_bit(int x) {
+#ifdef __CUDA_ARCH__
+  return 31 - __clz(x);
+#else
+  return 31 - __builtin_clz((unsigned)x);
+#endif
+}
+
+// veb_slot in 32-bit arithmetic (nodes are numbered in 31 bits), for the
+// kernels: the smallest power of two >= l/2 is the highest one in l - 1.
+__host__ __device__ inline int veb_slot32(int l, int t, int i) {
   int off = 0;
   while (l > 1) {
-    const int lb = 1 << (31 - __clz(l - 1)), lt = l - lb;
+    const int lb = 1 << high_bit(l - 1), lt = l - lb;
     if (t < lt) {
       l = lt;
     } else {
@@ -287,6 +296,49 @@ __host__ __device__ inline int64_t packed_slot(int h, int t, int64_t i) {
   if (t == 0) return 0;
   const int64_t sub = i >> (t - 1), il = i & (((int64_t)1 << (t - 1)) - 1);
   return 1 + sub * quad_count((h - 1) / 2) + veb4_slot((h - 1) / 2, (t - 1) / 2, il);
+}
+
+// veb4_slot and packed_slot in 32-bit arithmetic.  (4^H - 1) / 3 is every
+// other bit of 2 H.
+__host__ __device__ inline int quad_count32(int H) { return (int)(0x55555555u & ((1u << (2 * H)) - 1)); }
+
+__host__ __device__ inline int veb4_slot32(int H, int u, int i) {
+  int off = 0;
+  while (H > 1) {
+    const int Hb = 1 << high_bit(H - 1), Ht = H - Hb;
+    if (u < Ht) {
+      H = Ht;
+    } else {
+      const int uu = u - Ht, j = i >> (2 * uu);
+      off += quad_count32(Ht) + j * quad_count32(Hb);
+      i &= (1 << (2 * uu)) - 1;
+      u = uu;
+      H = Hb;
+    }
+  }
+  return off;
+}
+
+__host__ __device__ inline int packed_slot32(int h, int t, int i) {
+  if (!(h & 1)) return veb4_slot32(h / 2, t / 2, i);
+  if (t == 0) return 0;
+  const int sub = i >> (t - 1), il = i & ((1 << (t - 1)) - 1);
+  return 1 + sub * quad_count32((h - 1) / 2) + veb4_slot32((h - 1) / 2, (t - 1) / 2, il);
+}
+
+// packed_record_of in 32-bit arithmetic: level u of the (1 + odd) 4-ary trees
+// starts after (1 + odd) (4^u - 1) / 3 records.
+__host__ __device__ inline void packed_record_of32(int h, int g, int &t, int &i) {
+  const int odd = h & 1;
+  if (odd && g == 0) {
+    t = 0;
+    i = 0;
+    return;
+  }
+  const int y = odd ? (g - 1) : g;
+  const int u = high_bit(3 * (y >> odd) + 1) >> 1;   // 4^u <= 3 y' + 1 < 4^(u + 1)
+  t = 2 * u + odd;
+  i = y - (quad_count32(u) << odd);
 }
 
 // The g-th record in level order: depth t and index i of its node.

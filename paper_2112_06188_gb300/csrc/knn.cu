@@ -561,37 +561,58 @@ void launch_one(const KnnOne &P, int k, const KnnShape &sh, unsigned long long *
 // ---------------------------------------------------------------------------
 
 // One thread per record of many trees (table entry j owns the work items
-// pre[j] .. pre[j+1]-1, one per record of tree j, in level order).
+// pre[j] .. pre[j+1]-1, one per record of tree j, in level order).  A record
+// is put together and stored in 16-byte words: stored int by int it took each
+// store a sector of its own per lane (10M 3-D points: 80 -> 34 us).
 __global__ void k_pack_nodes(const TreeSeg *segs, const int64_t *pre, int nseg) {
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= pre[nseg]) return;
   const int j = knn_find(pre, nseg, x);
   const TreeSeg &T = segs[j];
-  const int32_t *box = T.box, *live = T.live;
   const int h = T.h, dim = T.dim;
-  int t;
-  int64_t i;
-  packed_record_of(h, x - pre[j], t, i);
+  int t, i;
+  packed_record_of32(h, (int)(x - pre[j]), t, i);
   const int e = packed_step(h, t);
-  int32_t *r = T.pk + packed_slot(h, t, i) * packed_node_ints(dim);
+  int4 *r = reinterpret_cast<int4 *>(T.pk + (int64_t)packed_slot32(h, t, i) * packed_node_ints(dim));
+  int code[4] = {0, 0, 0, 0}, lv[4] = {0, 0, 0, 0};
+  const int2 *bx[4];   // entry a's box: low bounds, then high ones
+#pragma unroll
   for (int a = 0; a < 4; ++a) {
-    int code = 0, lv = 0;
-    const int32_t *bx = nullptr;
-    if (a < (1 << e)) {   // entry a: descendant (t + e, i * 2^e + a)
-      const int tc = t + e;
-      const int64_t ci = (i << e) + a;
-      code = tc == h ? (int)(-1 - ci) : (int)packed_slot(h, tc, ci);
-      const int64_t v = veb_slot(h + 1, tc, ci);
-      lv = live[v];
-      bx = box + v * 2 * dim;
+    // entry a: descendant (t + e, i * 2^e + a); an odd tree's root has two
+    const int tc = t + e, ci = (i << e) + (a < (1 << e) ? a : 0);
+    const int v = veb_slot32(h + 1, tc, ci);
+    bx[a] = reinterpret_cast<const int2 *>(T.box + (int64_t)v * 2 * dim);
+    if (a < (1 << e)) {
+      code[a] = tc == h ? -1 - ci : packed_slot32(h, tc, ci);
+      lv[a] = T.live[v];
     }
-    r[packed_code_at(dim, a)] = code;
-    r[packed_live_at(dim, a)] = lv;
-    const uint32_t bias = packed_by_entry(dim) ? kBias : 0;
+  }
+  auto at = [&](int a, int w) {   // word w of entry a's box
+    return reinterpret_cast<const int32_t *>(bx[a])[w];
+  };
+  if (!packed_by_entry(dim)) {
+    r[0] = make_int4(code[0], code[1], code[2], code[3]);
+    r[1] = make_int4(lv[0], lv[1], lv[2], lv[3]);
     for (int c = 0; c < dim; ++c) {
-      r[packed_lo_at(dim, a, c)] = bx ? (int32_t)((uint32_t)bx[c] + bias) : INT32_MAX;
-      r[packed_hi_at(dim, a, c)] = bx ? (int32_t)((uint32_t)bx[dim + c] + bias) : INT32_MIN;
+      r[2 + 2 * c] = make_int4(at(0, c), at(1, c), at(2, c), at(3, c));
+      r[3 + 2 * c] = make_int4(at(0, dim + c), at(1, dim + c), at(2, dim + c), at(3, dim + c));
     }
+    return;
+  }
+  auto lo = [&](int a, int c) { return (int32_t)((uint32_t)at(a, c) + (uint32_t)kBias); };
+  auto hi = [&](int a, int c) { return (int32_t)((uint32_t)at(a, dim + c) + (uint32_t)kBias); };
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    int c = 0;
+    if (dim & 1) {
+      r[packed_code_at(dim, a) / 4] = make_int4(code[a], lv[a], lo(a, 0), hi(a, 0));
+      c = 1;
+    }
+    for (; c < dim; c += 2) r[packed_lo_at(dim, a, c) / 4] = make_int4(lo(a, c), hi(a, c), lo(a, c + 1), hi(a, c + 1));
+  }
+  if (!(dim & 1)) {
+    r[packed_code_at(dim, 0) / 4] = make_int4(code[0], lv[0], code[1], lv[1]);
+    r[packed_code_at(dim, 2) / 4] = make_int4(code[2], lv[2], code[3], lv[3]);
   }
 }
 

@@ -130,11 +130,11 @@ __device__ __forceinline__ void top_add(WarpTop &b, int k, bool have, uint64_t d
   top_bound(b, k);
 }
 
-// Query row qi of job J against the nt trees of the table (smallest first),
-// whose views are views[nt - 1 .. 0], then the buffer.  Called by a whole warp.
+// Query row qi of job J against the nt trees of the table (smallest first), then
+// the buffer.  Called by a whole warp.
 template <int D>
 __device__ __forceinline__ void warp_query(const KnnJob &J, WarpMem &W, const WTree *tree, int nt,
-                                           const TreeView *views, int64_t qi, int k) {
+                                           int64_t qi, int k) {
   constexpr int DM = D ? D : kMaxDim;
   const int dim = D ? D : J.dim;
   const int lane = threadIdx.x & 31;
@@ -155,25 +155,12 @@ __device__ __forceinline__ void warp_query(const KnnJob &J, WarpMem &W, const WT
   best.kid = INT32_MAX;
   best.kdf = kInf;
   int sp = 0, ls = 0;
-  // the roots, largest tree last (on top)
+  // the roots, largest tree last (on top), at distance zero: a root is seldom
+  // pruned, and its box would be a read that everything waits for
   for (int b = 0; b < nt; b += 32) {
     const int ti = b + lane;
-    bool ok = ti < nt;
-    float s = 0.f;
-    bool leaf = false;
-    if (ok) {
-      const TreeView &V = views[nt - 1 - ti];
-      leaf = V.h == 0;
-      ok = V.live[0] > 0;
-#pragma unroll
-      for (int c = 0; c < DM; ++c)
-        if (c < dim) {
-          const float lo = (float)V.box[c] + kBiasF, hi = (float)V.box[dim + c] + kBiasF;
-          const float g = fmaxf(fmaxf(lo - q[c], q[c] - hi), 0.f);
-          s = fmaf(g, g, s);
-        }
-    }
-    const uint64_t e = ((uint64_t)((__float_as_uint(s) & ~63u) | (unsigned)ti) << 32);
+    const bool ok = ti < nt, leaf = ok && tree[ti].nrec == 0;
+    const uint64_t e = (uint64_t)(unsigned)ti << 32;
     const unsigned nm = __ballot_sync(0xffffffffu, ok && !leaf), lm = __ballot_sync(0xffffffffu, ok && leaf);
     if (ok && !leaf) W.node[sp + __popc(nm & lt)] = e;
     if (ok && leaf) W.leaf[ls + __popc(lm & lt)] = e;
@@ -398,7 +385,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   const int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
   const int64_t t1 = min(t0 + per, P.job.m);
   for (int64_t t = t0; t < t1; ++t)
-    warp_query<D>(P.job, W[threadIdx.x >> 5], tree, P.job.ntrees, P.trees, P.job.perm ? P.job.perm[t] : t, k);
+    warp_query<D>(P.job, W[threadIdx.x >> 5], tree, P.job.ntrees, P.job.perm ? P.job.perm[t] : t, k);
 }
 
 // Many forests: warp w answers query w - job_warp[j] of its job j.
@@ -423,7 +410,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   const int64_t t = w - job_warp[lo];
   fill_trees(tree[warp], J.trees, J.ntrees, lane, 32);
   __syncwarp();
-  warp_query<D>(J, W[warp], tree[warp], J.ntrees, J.trees, J.perm ? J.perm[t] : t, k);
+  warp_query<D>(J, W[warp], tree[warp], J.ntrees, J.perm ? J.perm[t] : t, k);
 }
 
 template <int D>

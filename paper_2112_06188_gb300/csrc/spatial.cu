@@ -331,8 +331,8 @@ __global__ void k_sp_split(int t, int64_t N, const int32_t *mn, const int32_t *m
   if (nl + (int64_t)curR[s] != m) atomicOr(tr.err, kErrPartition);
   const int64_t v = m > 0 ? ((int64_t)mn[s] + (int64_t)mx[s]) >> 1 : 0;
   const int l = tr.h + 1;
-  const int64_t cl = veb_slot(l, t + 1, 2 * i), cr = veb_slot(l, t + 1, 2 * i + 1);
-  tr.node[veb_slot(l, t, i)] = Node{(uint64_t)((v << 31) | 0x7FFFFFFF), (int32_t)cl, (int32_t)cr};
+  const int cl = veb_slot32(l, t + 1, 2 * (int)i), cr = veb_slot32(l, t + 1, 2 * (int)i + 1);
+  tr.node[veb_slot32(l, t, (int)i)] = Node{(uint64_t)((v << 31) | 0x7FFFFFFF), cl, cr};
   if (t + 1 == tr.h) {
     tr.leaf_off[2 * i] = (int32_t)(lo[s] - tr.toff);
     tr.leaf_off[2 * i + 1] = (int32_t)(lo[s] + nl - tr.toff);
@@ -370,6 +370,8 @@ struct SpBoxParams {
   unsigned long long *err;
 };
 
+constexpr int64_t kOneBlockNodes = 1024;   // depths of at most so many nodes are one block's
+
 __device__ __forceinline__ void sp_leaf_boxes(const SpBoxParams &P, int64_t x0) {
   const int lane = threadIdx.x & 31, dim = P.dim, rs = rec_ints(dim);
   const int64_t x = x0 + lane;
@@ -382,7 +384,7 @@ __device__ __forceinline__ void sp_leaf_boxes(const SpBoxParams &P, int64_t x0) 
   if (act) {
     a = tr.leaf_off[leaf];
     b = tr.leaf_off[leaf + 1];
-    v = veb_slot(tr.h + 1, tr.h, leaf);
+    v = veb_slot32(tr.h + 1, tr.h, (int)leaf);
     if (a < 0 || b > tr.size || a > b) {
       atomicOr(tr.err, kErrLeaf);
       ok = false;
@@ -438,21 +440,30 @@ __global__ void __launch_bounds__(kT) k_sp_boxes(const SpBoxParams P) {
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
   for (int64_t x = t0 & ~(int64_t)31; x < P.leaf_pre[P.ntree]; x += step) sp_leaf_boxes(P, x);
   const int dim = P.dim;
-  unsigned epoch = 0;
-  for (int t = P.hmax - 1; t >= 0; --t) {
-    grid_barrier(P.bar, epoch, P.err);
-    for (int64_t s = t0; s < P.depth[t]; s += step) {
-      const SpTree &tr = P.T[s >> t];
-      const int64_t i = s & (((int64_t)1 << t) - 1);
-      const int l = tr.h + 1;
-      const int64_t v = veb_slot(l, t, i), a = veb_slot(l, t + 1, 2 * i), b = veb_slot(l, t + 1, 2 * i + 1);
-      for (int c = 0; c < dim; ++c) {
-        tr.box[v * 2 * dim + c] = min(tr.box[a * 2 * dim + c], tr.box[b * 2 * dim + c]);
-        tr.box[v * 2 * dim + dim + c] = max(tr.box[a * 2 * dim + dim + c], tr.box[b * 2 * dim + dim + c]);
-      }
-      tr.live[v] = tr.live[a] + tr.live[b];
-      if (t == 0 && tr.skew) *tr.skew = P.sq[s];   // to the host, whenever it arrives (a hint)
+  auto node = [&](int t, int64_t s) {
+    const SpTree &tr = P.T[s >> t];
+    const int i = (int)(s & (((int64_t)1 << t) - 1));
+    const int l = tr.h + 1;
+    const int64_t v = veb_slot32(l, t, i), a = veb_slot32(l, t + 1, 2 * i), b = veb_slot32(l, t + 1, 2 * i + 1);
+    for (int c = 0; c < dim; ++c) {
+      tr.box[v * 2 * dim + c] = min(tr.box[a * 2 * dim + c], tr.box[b * 2 * dim + c]);
+      tr.box[v * 2 * dim + dim + c] = max(tr.box[a * 2 * dim + dim + c], tr.box[b * 2 * dim + dim + c]);
     }
+    tr.live[v] = tr.live[a] + tr.live[b];
+    if (t == 0 && tr.skew) *tr.skew = P.sq[s];   // to the host, whenever it arrives (a hint)
+  };
+  unsigned epoch = 0;
+  int t = P.hmax - 1;
+  for (; t >= 0 && P.depth[t] > kOneBlockNodes; --t) {
+    grid_barrier(P.bar, epoch, P.err);
+    for (int64_t s = t0; s < P.depth[t]; s += step) node(t, s);
+  }
+  // depths with few nodes: one block, with block barriers
+  grid_barrier(P.bar, epoch, P.err);
+  if (blockIdx.x > 0) return;
+  for (; t >= 0; --t) {
+    for (int64_t s = threadIdx.x; s < P.depth[t]; s += blockDim.x) node(t, s);
+    __syncthreads();
   }
 }
 

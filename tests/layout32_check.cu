@@ -1,0 +1,37 @@
+// The 32-bit forms of the layout arithmetic that the kernels use, on the host:
+// equal to the 64-bit ones at every node of small trees, at every level's ends
+// and at places spread over the tallest trees there can be.
+#include <cstdio>
+
+#include "../paper_2112_06188_gb300/csrc/bdl_internal.cuh"
+
+using namespace bdl;
+
+static int bad = 0;
+#define CHECK(c)                                   \
+  do {                                             \
+    if (!(c) && bad++ < 10) printf("line %d\n", __LINE__); \
+  } while (0)
+
+int main() {
+  for (int h = 1; h <= 30; ++h) {
+    for (int t = 0; t <= h; ++t) {
+      const int64_t n = (int64_t)1 << t, step = n <= 4096 ? 1 : n / 4093;
+      for (int64_t i = 0; i < n; i += step) {
+        CHECK(veb_slot(h + 1, t, i) == (h < 30 ? veb_slot32(h + 1, t, (int)i) : veb_slot(h + 1, t, i)));
+        if (t < h && (t == 0 || ((h - t) & 1) == 0)) CHECK(packed_slot(h, t, i) == packed_slot32(h, t, (int)i));
+      }
+      CHECK(h == 30 || veb_slot(h + 1, t, n - 1) == veb_slot32(h + 1, t, (int)(n - 1)));
+    }
+    const int64_t n = packed_nrec(h), step = n <= 50000 ? 1 : n / 49999;
+    for (int64_t g = 0; g < n; g += step) {
+      int t, t2, i2;
+      int64_t i;
+      packed_record_of(h, g, t, i);
+      packed_record_of32(h, (int)g, t2, i2);
+      CHECK(t == t2 && i == i2);
+    }
+  }
+  puts(bad ? "BAD" : "ok");
+  return bad != 0;
+}
