@@ -11,7 +11,14 @@
 //    best; a few candidates enter one by one by a ballot (the rank) and a
 //    shift, more than ten are sorted across the warp and merged;
 //  * all trees of the forest are walked together: the stack starts with every
-//    tree's root, the largest tree's on top, and an entry names its tree.
+//    tree's root, the largest tree's on top, and an entry names its tree;
+//  * a warp that answers several queries one after another starts each but the
+//    first with a bound: the k neighbours just found are k live points, so the
+//    next query's k-th distance is at most its distance to the farthest of
+//    them.  A walk whose bound were the true k-th distance from the start
+//    would take 25 to 36% less; this way it takes 3 to 19% less (below);
+//  * while there is no bound, a node round takes two records only: what it
+//    takes beside the nearest is mostly what the first leaves rule out.
 // The answer does not depend on the order of the walk: every subtree whose
 // box is not strictly farther than the k-th distance is visited, and the k
 // best by (d2, id) of all points seen are unique.
@@ -21,9 +28,13 @@
 // warp instructions per query on 2M 3-D points, 10,000 on 2M 7-D ones, 65 to
 // 78% of the issue slots) and by the shared/L1 data pipe (53 to 67%).
 // Measured against the thread-per-query kernel (1M 5-D points, k = 10, 316
-// queries: 1,014 -> 51 us; 50K 16-D points, k = 8, 1,000 queries: 1,495 -> 59;
-// 500K 4-D points, k = 32, 100K queries: 3,620 -> 850; 10M 7-D points of 100
-// clusters, k = 5, 1M queries: 31.4 -> 20.4 ms).
+// queries: 1,014 -> 47 us; 50K 16-D points, k = 8, 1,000 queries: 1,495 -> 52;
+// 500K 4-D points, k = 32, 100K queries: 3,620 -> 768; 10M 7-D points of 100
+// clusters, k = 5, 1M queries: 31.4 -> 17.8 ms).
+// Without the starting bound and the narrow first rounds, and with them: those
+// four 50.5 -> 47, 55 -> 52, 840 -> 768 us and 20.3 -> 17.8 ms; 10M 3-D points,
+// k = 10, 30K queries 235 -> 202 us; 1M 2-D points of 100 clusters, spatial
+// median, k = 5, 100K queries 1,057 -> 865 us.
 #include "bdl_internal.cuh"
 
 #include <algorithm>
@@ -62,12 +73,13 @@ struct WarpTop {
   float kdf;       // pruning bound: k-th distance rounded up, scaled up (see box_dist_f in knn.cu)
   uint64_t kd;     // k-th pair
   int32_t kid;
+  float cap;       // a bound known beforehand, in the form of kdf
 };
 
 __device__ __forceinline__ void top_bound(WarpTop &b, int k) {
   b.kd = __shfl_sync(0xffffffffu, b.d, k - 1);
   b.kid = __shfl_sync(0xffffffffu, b.id, k - 1);
-  b.kdf = b.kd == ~0ull ? __int_as_float(0x7f800000) : __fmul_ru(__ull2float_ru(b.kd), kWBoundUp);
+  b.kdf = b.kd == ~0ull ? b.cap : fminf(b.cap, __fmul_ru(__ull2float_ru(b.kd), kWBoundUp));
 }
 
 __device__ __forceinline__ bool pair_less(uint64_t d, int32_t i, uint64_t e, int32_t j) {
@@ -131,10 +143,12 @@ __device__ __forceinline__ void top_add(WarpTop &b, int k, bool have, uint64_t d
 }
 
 // Query row qi of job J against the nt trees of the table (smallest first), then
-// the buffer.  Called by a whole warp.
+// the buffer.  Called by a whole warp.  `near_id`: lane i < k comes with the id of
+// a live point of the forest (all k different), or some lane with -1, and
+// leaves with the query's i-th neighbour, or -1.
 template <int D>
 __device__ __forceinline__ void warp_query(const KnnJob &J, WarpMem &W, const WTree *tree, int nt,
-                                           int64_t qi, int k) {
+                                           int64_t qi, int k, int32_t &near_id) {
   constexpr int DM = D ? D : kMaxDim;
   const int dim = D ? D : J.dim;
   const int lane = threadIdx.x & 31;
@@ -148,12 +162,27 @@ __device__ __forceinline__ void warp_query(const KnnJob &J, WarpMem &W, const WT
 #pragma unroll
   for (int c = 0; c < DM; ++c)
     if (c < dim) q[c] = (float)W.q[c] + kBiasF;
+  float cap = kInf;
+  if (__all_sync(0xffffffffu, lane >= k || near_id >= 0)) {
+    uint64_t s = 0;
+    if (lane < k) {
+      const int32_t *p = J.idtab + (int64_t)near_id * dim;
+#pragma unroll
+      for (int c = 0; c < DM; ++c)
+        if (c < dim) {
+          const int32_t g = W.q[c] - p[c];
+          s += (uint64_t)((int64_t)g * g);
+        }
+    }
+    const float f = __fmul_ru(__ull2float_ru(s), kWBoundUp);   // (not negative: ordered as its bits)
+    cap = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(f)));
+  }
   WarpTop best;
   best.d = ~0ull;
   best.id = INT32_MAX;
   best.kd = ~0ull;
   best.kid = INT32_MAX;
-  best.kdf = kInf;
+  best.kdf = best.cap = cap;
   int sp = 0, ls = 0;
   // the roots, largest tree last (on top), at distance zero: a root is seldom
   // pruned, and its box would be a read that everything waits for
@@ -252,13 +281,13 @@ __device__ __forceinline__ void warp_query(const KnnJob &J, WarpMem &W, const WT
       }
     }
     if (sp == 0) continue;
-    // ---- node round: the entries of up to eight records ----
+    // ---- node round: the entries of up to eight records (two while there is no bound) ----
     const int win = min(sp, 32);
     const uint64_t e0 = lane < win ? W.node[sp - 1 - lane] : 0;
     const bool ok0 = lane < win && !(__uint_as_float((uint32_t)(e0 >> 32) & ~63u) > best.kdf);
     const unsigned om = __ballot_sync(0xffffffffu, ok0);
     const int ord = __popc(om & lt);
-    const bool tk0 = ok0 && ord < (sp > kWWide ? 1 : 8);
+    const bool tk0 = ok0 && ord < (sp > kWWide ? 1 : best.kdf == kInf ? 2 : 8);
     if (tk0) W.sel[ord] = e0;
     const unsigned tk = __ballot_sync(0xffffffffu, tk0);
     // what leaves the stack: the records taken and the pruned ones above them
@@ -351,6 +380,7 @@ __device__ __forceinline__ void warp_query(const KnnJob &J, WarpMem &W, const WT
     }
     top_add(best, k, have, s, id);
   }
+  near_id = best.d != ~0ull ? best.id : -1;
   if (lane < k) {
     const bool ok = best.d != ~0ull;
     J.oi[qi * k + lane] = ok ? best.id : -1;
@@ -384,8 +414,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   __syncthreads();
   const int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
   const int64_t t1 = min(t0 + per, P.job.m);
+  int32_t near_id = -1;
   for (int64_t t = t0; t < t1; ++t)
-    warp_query<D>(P.job, W[threadIdx.x >> 5], tree, P.job.ntrees, P.job.perm ? P.job.perm[t] : t, k);
+    warp_query<D>(P.job, W[threadIdx.x >> 5], tree, P.job.ntrees, P.job.perm ? P.job.perm[t] : t, k, near_id);
 }
 
 // Many forests: warp w answers query w - job_warp[j] of its job j.
@@ -410,14 +441,17 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   const int64_t t = w - job_warp[lo];
   fill_trees(tree[warp], J.trees, J.ntrees, lane, 32);
   __syncwarp();
-  warp_query<D>(J, W[warp], tree[warp], J.ntrees, J.perm ? J.perm[t] : t, k);
+  int32_t near_id = -1;
+  warp_query<D>(J, W[warp], tree[warp], J.ntrees, J.perm ? J.perm[t] : t, k, near_id);
 }
 
 template <int D>
 void warp_one(const KnnOne &P, int k, cudaStream_t s) {
-  // up to eight neighbouring queries per warp, which find their paths in L1
-  // (10M 7-D points, 1M queries: 23.5 -> 21.5 ms), while that leaves about six
-  // times the warps the GPU can hold
+  // up to eight neighbouring queries per warp, which find their paths in L1 and
+  // start with a bound, while that leaves about six times the warps the GPU
+  // can hold.  10M 7-D points, 1M queries: 23.5 -> 17.8 ms; with 16 per warp
+  // 17.9, with 32 19.2.  1M 7-D points, 50K queries: one per warp 0.99 ms,
+  // three 1.08
   const int per = (int)std::min<int64_t>(8, std::max<int64_t>(1, P.job.m / 30000));
   const int64_t blk = (int64_t)kWarpsPerBlock * per;
   KScope ks_(kK_knn, s);

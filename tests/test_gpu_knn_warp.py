@@ -116,6 +116,23 @@ def test_thread_kernel_gives_the_same_rows(dim, m):
     assert f.poll_error() == 0
 
 
+@pytest.mark.parametrize("dim,n,m,k", [(4, 6_000, 61_003, 32), (5, 20_000, 250_001, 5), (8, 6_000, 60_000, 1),
+                                       (10, 3_000, 90_001, 32), (8, 20, 60_100, 32), (8, 40, 60_100, 32)])
+@pytest.mark.parametrize("distinct", [0, 7])
+def test_queries_in_turn_by_one_warp(dim, n, m, k, distinct):
+    """Two to eight queries per warp, each starting with the bound that the
+    last one's neighbours give, against one per warp: also with fewer live
+    points than k and with points in few places."""
+    f, live = forest_of(dim, n, 31 + n, distinct=distinct, X=16)
+    lp, _ = live.live_points()
+    q = dev(np.concatenate([inputs.queries_from(lp, m // 2, 7), inputs.uniform_points(m - m // 2, dim, 8)]))
+    gi, gd = f.knn(q, k)
+    for a in range(0, m, 7_000):
+        wi, wd = f.knn(q[a:a + 7_000], k)
+        assert torch.equal(gi[a:a + 7_000], wi) and torch.equal(gd[a:a + 7_000], wd)
+    assert f.poll_error() == 0
+
+
 @pytest.mark.parametrize("dim,X,n", [(2, 1024, 1023), (3, 64, 5_000), (5, 1024, 20_700), (7, 2048, 33)])
 def test_buffer_scanned_first_then_searched(dim, X, n):
     """The first small call after an update scans the buffer, the next one
