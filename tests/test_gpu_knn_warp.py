@@ -116,6 +116,21 @@ def test_thread_kernel_gives_the_same_rows(dim, m):
     assert f.poll_error() == 0
 
 
+@pytest.mark.parametrize("dim,m,k,leaf", [(1, 30_001, 8, 64), (2, 40_003, 5, 33), (3, 70_001, 10, 64), (3, 30_000, 1, 32)])
+@pytest.mark.parametrize("distinct", [0, 40])
+def test_thread_kernel_with_leaves_over_32_points(dim, m, k, leaf, distinct):
+    f, live = forest_of(dim, 9_000, 71 + leaf, leaf=leaf, distinct=distinct)
+    lp, _ = live.live_points()
+    q = dev(np.concatenate([inputs.queries_from(lp, m // 2, 7), inputs.uniform_points(m - m // 2, dim, 8)]))
+    gi, gd = f.knn(q, k)
+    for a in range(0, m, 5_000):
+        wi, wd = f.knn(q[a:a + 5_000], k)
+        assert torch.equal(gi[a:a + 5_000], wi) and torch.equal(gd[a:a + 5_000], wd)
+    cnt = torch.zeros(3, dtype=torch.int64, device="cuda")
+    ci, cd = f.knn_count(q, k, cnt)
+    assert torch.equal(ci, gi) and torch.equal(cd, gd) and f.poll_error() == 0
+
+
 @pytest.mark.parametrize("dim,n,m,k", [(4, 6_000, 61_003, 32), (5, 20_000, 250_001, 5), (8, 6_000, 60_000, 1),
                                        (10, 3_000, 90_001, 32), (8, 20, 60_100, 32), (8, 40, 60_100, 32)])
 @pytest.mark.parametrize("distinct", [0, 7])
