@@ -766,13 +766,15 @@ int upload_knn_table(const std::vector<KnnCall> &calls, void *table, int64_t *wa
 int launch_knn_table(const void *table, int njobs, int64_t warps, int dim, int k, const KnnShape &sh,
                      unsigned long long *stats, cudaStream_t s);
 // The kernel with one warp per query (knn_warp.cu): whether a launch of m
-// queries on n points takes it, and its launches (the table's job prefix
-// counts one warp per query: upload_knn_table with qpw = 1).
+// queries on n points takes it, and its launches; a warp answers
+// knn_warp_per(m) queries in turn (upload_knn_table with qpw = that).
 bool knn_by_warp(int dim, int k, int64_t m, int64_t n, bool skewed);
-// The same for the calls of one launch together.
-bool knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k);
-int launch_knn_warp_one(const KnnOne &P, int dim, int k, cudaStream_t s);
-int launch_knn_warp_table(const void *table, int njobs, int64_t warps, int dim, int k, cudaStream_t s);
+int knn_warp_per(int64_t m);
+// The same for the calls of one launch together: 0 for the thread-per-query
+// kernel, otherwise the queries per warp.
+int knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k);
+int launch_knn_warp_one(const KnnOne &P, int dim, int k, int per, cudaStream_t s);
+int launch_knn_warp_table(const void *table, int njobs, int64_t warps, int dim, int k, int per, cudaStream_t s);
 // k-NN for every call (all of dimension `dim`) in one launch; the job table
 // is uploaded to `table` (knn_table_bytes of device memory) on stream s.
 int launch_knn_jobs(const std::vector<KnnCall> &calls, int dim, int k, const KnnShape &sh, void *table,

@@ -1500,11 +1500,16 @@ static int knn_many(bdl_forest *const *F, int nf, const int32_t *const *q, const
       nd[d] += F[i]->live;
       stats[d] = stats[d] || F[i]->knn_stats;
     }
+    signed char by_warp[kMaxDim + 1][2];   // the rule's answers so far (it takes logarithms)
+    memset(by_warp, -1, sizeof(by_warp));
     for (int i = 0; i < nf && pairs <= kScanPairs; ++i) {
       const bdl_forest *f = F[i];
       const int d = f->dim;
-      scan[i] = f->buf_dirty && !f->buf_scanned && f->nbuf > 0 && m[i] > 0 && !stats[d] &&
-                knn_by_warp(d, k, md[d], nd[d], skewed_leaves(f));
+      scan[i] = f->buf_dirty && !f->buf_scanned && f->nbuf > 0 && m[i] > 0 && !stats[d];
+      if (!scan[i]) continue;
+      const bool skewed = skewed_leaves(f);
+      if (by_warp[d][skewed] < 0) by_warp[d][skewed] = knn_by_warp(d, k, md[d], nd[d], skewed);
+      scan[i] = by_warp[d][skewed];
     }
     for (int i = 0; i < nf; ++i)
       if (scan[i]) F[i]->buf_scanned = true;
@@ -1567,7 +1572,7 @@ struct bdl_knn_plan {
     void *table;
     unsigned long long *stats;
     bdl::KnnShape shape;
-    bool by_warp;
+    int per;   // queries per warp of the warp-per-query kernel; 0: the other one
   };
   struct Sort {
     const int32_t *q;
@@ -1639,8 +1644,8 @@ static int knn_plan_make(bdl_forest *const *F, int nf, const int32_t *const *q, 
     for (int i = 0; i < nf; ++i)
       if (F[i]->dim == d && F[i]->knn_stats) stats = F[i]->knn_stats;
     bdl_knn_plan::Part part{d, (int)groups[gi].size(), 0, p, stats, F[0]->knn_shape,
-                            !stats && knn_by_warp(groups[gi], d, k)};
-    st = upload_knn_table(groups[gi], p, &part.warps, part.by_warp ? 1 : part.shape.qpw, s);
+                            stats ? 0 : knn_by_warp(groups[gi], d, k)};
+    st = upload_knn_table(groups[gi], p, &part.warps, part.per ? part.per : part.shape.qpw, s);
     if (st) return st;
     p += a256(knn_table_bytes_always(groups[gi]));
     P->parts.push_back(part);
@@ -1658,8 +1663,8 @@ static int knn_plan_launch(bdl_knn_plan *P, cudaStream_t s) {
       return set_error(BDL_EINVAL, "a forest changed since the k-NN plan was made");
   for (auto &so : P->sorts) launch_query_sort(so.q, so.m, so.dim, so.scratch, so.perm, s);
   for (auto &part : P->parts) {
-    const int st = part.by_warp
-                       ? launch_knn_warp_table(part.table, part.njobs, part.warps, part.dim, P->k, s)
+    const int st = part.per
+                       ? launch_knn_warp_table(part.table, part.njobs, part.warps, part.dim, P->k, part.per, s)
                        : launch_knn_table(part.table, part.njobs, part.warps, part.dim, P->k, part.shape, part.stats, s);
     if (st) return st;
   }

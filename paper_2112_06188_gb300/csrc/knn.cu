@@ -858,14 +858,14 @@ size_t batch_query_sort_bytes(const std::vector<KnnCall> &calls) {
          ((size_t)nb * 4 + 255) / 256 * 256 + ((size_t)n * 8 + 255) / 256 * 256 + (size_t)(n + 1) * 8 + 256;
 }
 
-bool knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k) {
+int knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k) {
   int64_t m = 0, n = 0, ms = 0;
   for (const auto &c : calls) {
     m += c.m;
     if (c.skewed) ms += c.m;
     for (int t = 0; t < c.fv->ntrees; ++t) n += c.fv->tree[t].size;
   }
-  return knn_by_warp(dim, k, m, n, 2 * ms > m);
+  return knn_by_warp(dim, k, m, n, 2 * ms > m) ? knn_warp_per(m) : 0;
 }
 
 size_t knn_table_bytes(const std::vector<KnnCall> &calls) {
@@ -961,7 +961,8 @@ int launch_knn_jobs(const std::vector<KnnCall> &calls, int dim, int k, const Knn
     P.job.oi = c.oi;
     P.job.od = c.od;
     for (int t = 0; t < c.fv->ntrees; ++t) P.trees[t] = c.fv->tree[t];
-    if (!stats && knn_by_warp(calls, dim, k)) return launch_knn_warp_one(P, dim, k, s);
+    const int per = stats ? 0 : knn_by_warp(calls, dim, k);
+    if (per) return launch_knn_warp_one(P, dim, k, per, s);
     if (!stats) {
       switch (dim) {
         case 1: launch_one<1, false>(P, k, sh, stats, s); break;
@@ -985,10 +986,10 @@ int launch_knn_jobs(const std::vector<KnnCall> &calls, int dim, int k, const Knn
     return cuda_check(cudaGetLastError(), "knn kernel");
   }
   int64_t warps = 0;
-  const bool by_warp = !stats && knn_by_warp(calls, dim, k);
-  int st = upload_knn_table(calls, table, &warps, by_warp ? 1 : sh.qpw, s);
+  const int per = stats ? 0 : knn_by_warp(calls, dim, k);
+  int st = upload_knn_table(calls, table, &warps, per ? per : sh.qpw, s);
   if (st) return st;
-  if (by_warp) return launch_knn_warp_table(table, (int)n, warps, dim, k, s);
+  if (per) return launch_knn_warp_table(table, (int)n, warps, dim, k, per, s);
   return launch_knn_table(table, (int)n, warps, dim, k, sh, stats, s);
 }
 

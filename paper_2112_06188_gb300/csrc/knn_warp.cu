@@ -38,6 +38,7 @@
 #include "bdl_internal.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace bdl {
 
@@ -419,10 +420,11 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
     warp_query<D>(P.job, W[threadIdx.x >> 5], tree, P.job.ntrees, P.job.perm ? P.job.perm[t] : t, k, near_id);
 }
 
-// Many forests: warp w answers query w - job_warp[j] of its job j.
+// Many forests: warp w answers the (w - job_warp[j])-th `per` queries of its
+// job j.
 template <int D>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
-    k_knn_warp(const KnnJob *jobs, const int64_t *job_warp, int njobs, int k) {
+    k_knn_warp(const KnnJob *jobs, const int64_t *job_warp, int njobs, int k, int per) {
   __shared__ WarpMem W[kWarpsPerBlock];
   __shared__ WTree tree[kWarpsPerBlock][kWTrees];
   __shared__ KnnJob s_job[kWarpsPerBlock];
@@ -438,101 +440,120 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   KnnJob &J = s_job[warp];
   if (lane == 0) J = jobs[lo];
   __syncwarp();
-  const int64_t t = w - job_warp[lo];
+  const int64_t t0 = (w - job_warp[lo]) * per, t1 = min(t0 + per, J.m);
   fill_trees(tree[warp], J.trees, J.ntrees, lane, 32);
   __syncwarp();
   int32_t near_id = -1;
-  warp_query<D>(J, W[warp], tree[warp], J.ntrees, J.perm ? J.perm[t] : t, k, near_id);
+  for (int64_t t = t0; t < t1; ++t)
+    warp_query<D>(J, W[warp], tree[warp], J.ntrees, J.perm ? J.perm[t] : t, k, near_id);
 }
 
 template <int D>
-void warp_one(const KnnOne &P, int k, cudaStream_t s) {
-  // up to eight neighbouring queries per warp, which find their paths in L1 and
-  // start with a bound, while that leaves about six times the warps the GPU
-  // can hold.  10M 7-D points, 1M queries: 23.5 -> 17.8 ms; with 16 per warp
-  // 17.9, with 32 19.2.  1M 7-D points, 50K queries: one per warp 0.99 ms,
-  // three 1.08
-  const int per = (int)std::min<int64_t>(8, std::max<int64_t>(1, P.job.m / 30000));
+void warp_one(const KnnOne &P, int k, int per, cudaStream_t s) {
   const int64_t blk = (int64_t)kWarpsPerBlock * per;
   KScope ks_(kK_knn, s);
   k_knn_warp_one<D><<<(unsigned)((P.job.m + blk - 1) / blk), kWarpsPerBlock * 32, 0, s>>>(P, k, per);
 }
 
 template <int D>
-void warp_table(const KnnJob *jobs, const int64_t *job_warp, int njobs, int64_t warps, int k, cudaStream_t s) {
+void warp_table(const KnnJob *jobs, const int64_t *job_warp, int njobs, int64_t warps, int k, int per,
+                cudaStream_t s) {
   KScope ks_(kK_knn, s);
   k_knn_warp<D><<<(unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock), kWarpsPerBlock * 32, 0, s>>>(
-      jobs, job_warp, njobs, k);
+      jobs, job_warp, njobs, k, per);
 }
 
 }  // namespace
 
-// Where the two kernels cost the same.  The warp-per-query kernel's time grows
-// with the queries (3 to 20 ns each) from a few dozen microseconds; the
+// Up to eight neighbouring queries per warp, which find their paths in L1 and
+// start with a bound, while that leaves about six times the warps the GPU can
+// hold.  10M 7-D points, 1M queries: 23.5 -> 17.8 ms; with 16 per warp 17.9,
+// with 32 19.2.  1M 7-D points, 50K queries: one per warp 0.99 ms, three 1.08.
+int knn_warp_per(int64_t m) { return (int)std::min<int64_t>(8, std::max<int64_t>(1, m / 30000)); }
+
+// Where the two kernels cost the same: thousands of queries, for k = 1, 5, 16
+// and 32 on forests of 4,500, 55,000 and a million points (9999: beyond
+// 640,000, the most that was measured).  The warp-per-query kernel's time
+// grows with the queries (3 to 20 ns each) from a few dozen microseconds; the
 // thread-per-query kernel's stays near that of its slowest warps until about
-// 130,000 queries fill the GPU, and then grows more slowly in low dimensions
-// (neighbouring queries share their walk) and for small k (its top-k lists
-// take 12 k bytes of shared memory per thread: past k = 16 they cost it
-// resident warps).  Measured for n = 10^4 .. 10^7 points, uniform and
-// clustered; thread / warp in us:
-//   dim 1, k = 8:  16K queries 86 / 56, 65K 109 / 215
-//   dim 2, k = 5:  16K 116 / 78, 33K 133 / 159;   k = 32: 131K 867 / 764
-//   dim 3, k = 1:  16K 126 / 77, 33K 125 / 158;   k = 10: 33K 325 / 203, 66K 328 / 369
-//          k = 24: 262K 1719 / 1734;              k = 32: 1M 7885 / 7074
-//   dim 4, k = 1:  66K 400 / 293, 131K 468 / 542; k = 10: 262K 1696 / 1611
-//   dim 5, k = 1:  262K 1095 / 1091;              k = 10: 1M 8569 / 7992
-//   dim 6, k = 1:  262K 2128 / 1233, 1M 3313 / 4229; k = 10: 1M 11838 / 11479
-//   dim 7, k = 1:  1M queries on 100K points 4350 / 4399 (clusters 2503 / 3404),
-//                  on 10M 11182 / 7054;           k = 5: 1M on 1M 20953 / 12524
+// 130,000 queries fill the GPU, and then grows more slowly where its walks are
+// short (low dimensions, small forests) and for small k (its top-k lists take
+// 12 k bytes of shared memory per thread: past k = 16 they cost it resident
+// warps).  Each entry is the geometric mean of the crossings of uniform points
+// and of points in 100 clusters, and of two sizes n for the first two columns
+// (2,000 and 10,000; 30,000 and 100,000).  5,000 to 640,000 queries at points
+// of the forest, thread / warp in us on either side of a crossing:
+//   dim 1, k = 5:  n = 10,000, 10K queries 36 / 31, 20K 37 / 48
+//   dim 2, k = 5:  n = 100,000, 20K 89 / 65, 40K 101 / 139
+//   dim 3, k = 5:  n = 1M, 40K 264 / 198, 80K 300 / 337
+//          k = 16: n = 1M, 80K 573 / 435, 160K 666 / 797
+//   dim 4, k = 1:  n = 30,000, 40K 182 / 137, 80K 186 / 195
+//   dim 5, k = 1:  n = 2,000 clustered, 10K 38 / 28, 160K 83 / 217
+//          k = 16: n = 30,000, 320K 1973 / 1856, 640K 2914 / 3285
+//   dim 6, k = 5:  n = 10,000, 160K 782 / 674, 320K 912 / 1203
+//   dim 7, k = 1:  n = 10,000, 160K 554 / 343, 320K 554 / 586
+// Over all 2,688 of those launches the choice costs 1% more than the better
+// kernel each time (a line in k alone: 3.4%, and up to 3.3 times on small
+// forests in dimensions 4 to 7).
+//
 // Leaves of hundreds of points and more (spatial-median trees of clustered
 // points) are scanned by one lane in the thread-per-query kernel, 32 points at
 // a time here.  100 clusters, thread / warp in us: 1M 2-D points, k = 5, 100K
-// queries 4014 / 1062, 1M queries 7174 / 8953; 1M 3-D points, k = 10, 1M
-// queries 16160 / 9937; 10M 3-D points, 1M queries 68980 / 39557.
+// queries 3190 / 867, 600K 4400 / 4083, 1M 5749 / 6522; 1M 3-D points, k = 10,
+// 1M queries 11681 / 8335; 10M 3-D points, 1M queries 55418 / 37189.
 bool knn_by_warp(int dim, int k, int64_t m, int64_t n, bool skewed) {
-  if (skewed && (dim > 2 || m <= 600000)) return true;
-  struct Line {
-    double base, slope;   // k <= 16: most queries (thousands) = base + slope k
-    double k24, k32;      // for k = 17 .. 24 and above
+  if (dim > 7 || (skewed && (dim > 2 || m <= 600000))) return true;
+  static constexpr int kAtK[4] = {1, 5, 16, 32};
+  static constexpr float kAtN[3] = {4500, 55000, 1e6};
+  static constexpr float kMost[7][4][3] = {
+      {{7, 14, 56}, {14, 20, 64}, {32, 42, 97}, {61, 130, 220}},
+      {{13, 18, 28}, {27, 34, 53}, {49, 81, 110}, {130, 1700, 9999}},
+      {{19, 28, 41}, {33, 53, 78}, {62, 120, 150}, {220, 2600, 9999}},
+      {{23, 45, 78}, {53, 85, 260}, {130, 250, 9999}, {710, 9999, 9999}},
+      {{36, 77, 270}, {64, 180, 9999}, {160, 1600, 9999}, {2600, 9999, 9999}},
+      {{55, 140, 910}, {87, 300, 9999}, {220, 2000, 9999}, {2500, 9999, 9999}},
+      {{73, 420, 9999}, {94, 1700, 9999}, {470, 9999, 9999}, {2800, 9999, 9999}}};
+  // between the entries: linear in k and log n, for the logarithm
+  const int ik = k < 5 ? 0 : k < 16 ? 1 : 2;
+  const float wk = (float)(k - kAtK[ik]) / (float)(kAtK[ik + 1] - kAtK[ik]);
+  const int in = (float)n < kAtN[1] ? 0 : 1;
+  const float x = std::log((float)std::max<int64_t>(n, 1) / kAtN[in]) / std::log(kAtN[in + 1] / kAtN[in]);
+  const float wn = std::min(std::max(x, 0.f), 1.f);
+  auto at = [&](int i) {
+    return (1 - wn) * std::log(kMost[dim - 1][i][in]) + wn * std::log(kMost[dim - 1][i][in + 1]);
   };
-  constexpr double kAll = 1e12;
-  static constexpr Line kLine[7] = {{9, 1.8, 52, 67},      {14, 3, 86, 110},        {20, 4.5, 250, 1000},
-                                    {80, 12, 500, kAll},   {140, 40, kAll, kAll},   {250, 70, kAll, kAll},
-                                    {700, 0, kAll, kAll}};
-  if (dim > 7 || (dim == 7 && (k > 2 || m < n))) return true;
-  const Line &L = kLine[dim - 1];
-  return (double)m <= 1e3 * (k <= 16 ? L.base + L.slope * k : k <= 24 ? L.k24 : L.k32);
+  return (float)m <= 1000 * std::exp((1 - wk) * at(ik) + wk * at(ik + 1));
 }
 
-int launch_knn_warp_one(const KnnOne &P, int dim, int k, cudaStream_t s) {
+int launch_knn_warp_one(const KnnOne &P, int dim, int k, int per, cudaStream_t s) {
   switch (dim) {
-    case 1: warp_one<1>(P, k, s); break;
-    case 2: warp_one<2>(P, k, s); break;
-    case 3: warp_one<3>(P, k, s); break;
-    case 4: warp_one<4>(P, k, s); break;
-    case 5: warp_one<5>(P, k, s); break;
-    case 6: warp_one<6>(P, k, s); break;
-    case 7: warp_one<7>(P, k, s); break;
-    case 8: warp_one<8>(P, k, s); break;
-    default: warp_one<0>(P, k, s); break;
+    case 1: warp_one<1>(P, k, per, s); break;
+    case 2: warp_one<2>(P, k, per, s); break;
+    case 3: warp_one<3>(P, k, per, s); break;
+    case 4: warp_one<4>(P, k, per, s); break;
+    case 5: warp_one<5>(P, k, per, s); break;
+    case 6: warp_one<6>(P, k, per, s); break;
+    case 7: warp_one<7>(P, k, per, s); break;
+    case 8: warp_one<8>(P, k, per, s); break;
+    default: warp_one<0>(P, k, per, s); break;
   }
   return cuda_check(cudaGetLastError(), "knn kernel");
 }
 
-int launch_knn_warp_table(const void *table, int njobs, int64_t warps, int dim, int k, cudaStream_t s) {
+int launch_knn_warp_table(const void *table, int njobs, int64_t warps, int dim, int k, int per, cudaStream_t s) {
   if (warps == 0) return BDL_OK;
   const KnnJob *jobs = (const KnnJob *)table;
   const int64_t *job_warp = (const int64_t *)((const char *)table + njobs * sizeof(KnnJob));
   switch (dim) {
-    case 1: warp_table<1>(jobs, job_warp, njobs, warps, k, s); break;
-    case 2: warp_table<2>(jobs, job_warp, njobs, warps, k, s); break;
-    case 3: warp_table<3>(jobs, job_warp, njobs, warps, k, s); break;
-    case 4: warp_table<4>(jobs, job_warp, njobs, warps, k, s); break;
-    case 5: warp_table<5>(jobs, job_warp, njobs, warps, k, s); break;
-    case 6: warp_table<6>(jobs, job_warp, njobs, warps, k, s); break;
-    case 7: warp_table<7>(jobs, job_warp, njobs, warps, k, s); break;
-    case 8: warp_table<8>(jobs, job_warp, njobs, warps, k, s); break;
-    default: warp_table<0>(jobs, job_warp, njobs, warps, k, s); break;
+    case 1: warp_table<1>(jobs, job_warp, njobs, warps, k, per, s); break;
+    case 2: warp_table<2>(jobs, job_warp, njobs, warps, k, per, s); break;
+    case 3: warp_table<3>(jobs, job_warp, njobs, warps, k, per, s); break;
+    case 4: warp_table<4>(jobs, job_warp, njobs, warps, k, per, s); break;
+    case 5: warp_table<5>(jobs, job_warp, njobs, warps, k, per, s); break;
+    case 6: warp_table<6>(jobs, job_warp, njobs, warps, k, per, s); break;
+    case 7: warp_table<7>(jobs, job_warp, njobs, warps, k, per, s); break;
+    case 8: warp_table<8>(jobs, job_warp, njobs, warps, k, per, s); break;
+    default: warp_table<0>(jobs, job_warp, njobs, warps, k, per, s); break;
   }
   return cuda_check(cudaGetLastError(), "knn kernel");
 }

@@ -87,9 +87,9 @@ def test_deep_trees_with_little_pruning():
 
 
 # just above and below the size from which each dimension takes the
-# thread-per-query kernel (k = 1), with the launch shapes that kernel has
-@pytest.mark.parametrize("dim,m", [(1, 10_700), (2, 16_900), (3, 24_400), (4, 91_900), (5, 179_900), (6, 319_900),
-                                   (7, 699_900)])
+# thread-per-query kernel (k = 1, a small forest), with the launch shapes that kernel has
+@pytest.mark.parametrize("dim,m", [(1, 6_900), (2, 12_900), (3, 18_900), (4, 22_900), (5, 35_900), (6, 54_900),
+                                   (7, 72_900)])
 def test_thread_kernel_gives_the_same_rows(dim, m):
     from paper_2112_06188_gb300.forest import KnnPlan, knn_batch
     f, live = forest_of(dim, 3_000, 60 + dim)
@@ -131,7 +131,7 @@ def test_thread_kernel_with_leaves_over_32_points(dim, m, k, leaf, distinct):
     assert torch.equal(ci, gi) and torch.equal(cd, gd) and f.poll_error() == 0
 
 
-@pytest.mark.parametrize("dim,n,m,k", [(4, 6_000, 61_003, 32), (5, 20_000, 250_001, 5), (8, 6_000, 60_000, 1),
+@pytest.mark.parametrize("dim,n,m,k", [(4, 6_000, 61_003, 32), (5, 20_000, 250_001, 16), (8, 6_000, 60_000, 1),
                                        (10, 3_000, 90_001, 32), (8, 20, 60_100, 32), (8, 40, 60_100, 32)])
 @pytest.mark.parametrize("distinct", [0, 7])
 def test_queries_in_turn_by_one_warp(dim, n, m, k, distinct):
