@@ -50,9 +50,7 @@ enum KernelId : int {
   kK_pack_lives,
   kK_put_blob,
   kK_sp_gather,
-  kK_sp_minmax,
-  kK_sp_scatter,
-  kK_sp_split,
+  kK_sp_levels,
   kK_sp_box,
   kK_knn_count,
   kK_small_copy,

@@ -43,9 +43,7 @@ const char *const kKernelNames[kKernelCount] = {
     "k_pack_lives",
     "k_put_blob",
     "k_sp_gather",
-    "k_sp_minmax",
-    "k_sp_scatter",
-    "k_sp_split",
+    "k_sp_levels",
     "k_sp_box",
     "k_knn_count",
     "k_small_copy",

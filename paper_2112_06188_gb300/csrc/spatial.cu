@@ -11,17 +11,16 @@
 // ordered by height, so the trees still splitting at level t are a prefix of
 // that order and so are their records in the staging buffer.  A record's
 // segment at level t is s = j * 2^t + i (tree j, node i of depth t), and its
-// child's is 2s or 2s + 1.  Per level:
-//   k_sp_minmax  -- min and max of the split coordinate per segment (block-,
-//                   then warp-aggregated atomics), for the first level only;
-//   k_sp_scatter -- left records fill the child's range from its start, right
-//                   ones from its end (aggregated atomic cursors); records of
-//                   a tree whose children are leaves go straight to the tree;
-//                   the others also give their child segment's min and max of
-//                   the next level's split coordinate, so that level needs no
-//                   pass of its own;
-//   k_sp_split   -- the node's key and children, the children's bounds, and
-//                   the leaf offsets of trees that end here.
+// child's is 2s or 2s + 1.  k_sp_levels runs all levels in one cooperative
+// launch.  Per level, with a grid barrier after each:
+//   scatter -- left records fill the child's range from its start, right
+//              ones from its end (aggregated atomic cursors); records of a
+//              tree whose children are leaves go straight to the tree; the
+//              others also give their child segment's min and max of the next
+//              level's split coordinate, so only the first level needs a pass
+//              for its bounds (block-, then warp-aggregated atomics);
+//   split   -- the node's key and children, the children's bounds, and the
+//              leaf offsets of trees that end here.
 // Order inside a child is not kept (the sets are what the rule fixes).  Then
 // leaf boxes, boxes bottom-up and the packed k-NN records.
 #include "bdl_internal.cuh"
@@ -136,41 +135,35 @@ __global__ void k_sp_gather(const SpGather *G, const int64_t *pre, int ng, const
   }
 }
 
-// Level-0 bounds of every splitting tree; the leaf-offset sentinels; the
-// single leaf of a tree with h = 0.
-__global__ void k_sp_roots(const SpTree *T, int ntree, int64_t *lo, int32_t *n) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= ntree) return;
-  const SpTree &tr = T[j];
-  tr.leaf_off[(int64_t)1 << tr.h] = (int32_t)tr.size;
-  if (tr.h == 0) {
-    tr.leaf_off[0] = 0;
-    tr.node[0] = Node{0, -1, 0};
-  } else {
-    lo[j] = tr.toff;
-    n[j] = (int32_t)tr.size;
-  }
-}
+// All levels of the new trees in one cooperative launch.
+//
+// A step's batch is a few microseconds of work per level, so three launches
+// per level (clearing, scatter, split) and an upload per table were what it
+// cost: 100K points into 1M 2-D ones, insert call 380 us, this way 306; 5,000
+// into 100K 250 -> 170; builds of 100K and 1M 2-D points 328 -> 238 and 634 ->
+// 567 us.  Large builds are bound by the records' gathers and scatters and
+// want the warps: 10M 3-D points 3,705 us in launches, here 3,860 at four
+// blocks per SM (58 registers), 3,580 at five, 3,222 at six and 3,345 at eight.
+constexpr int kSpBlocks = 6;
 
-// Cursors of the N segments of this level; empty bounds for the Nb segments
-// whose min and max are gathered next (by k_sp_minmax or by the scatter).
-__global__ void k_sp_level_init(int64_t N, uint32_t *curL, uint32_t *curR, int64_t Nb, int32_t *mn,
-                                int32_t *mx) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < N) {
-    curL[s] = 0;
-    curR[s] = 0;
-  }
-  if (s < Nb) {
-    mn[s] = INT32_MAX;
-    mx[s] = INT32_MIN;
-  }
-}
+struct SpLevels {
+  const SpTree *T;
+  const int64_t *seg_n;    // [hmax] segments of each level
+  const int64_t *rec_n;    // [hmax] records still splitting at each level
+  int ntree, dim, hmax;
+  int32_t *stg[2], *seg[2];
+  int32_t *mn[2], *mx[2];  // split-coordinate bounds of this level's and the next level's segments
+  int64_t *lo[2];
+  int32_t *n[2];
+  uint32_t *curL, *curR;
+  unsigned *bar;
+  unsigned long long *err;
+};
 
-__global__ void __launch_bounds__(kT) k_sp_minmax(const int32_t *stg, const int32_t *seg, int64_t A, int rs,
-                                                  int c, int32_t *mn, int32_t *mx) {
+// First level's bounds from the records [p0, p0 + kT).
+__device__ __forceinline__ void sp_minmax(const int32_t *stg, const int32_t *seg, int64_t p0, int64_t A, int rs,
+                                          int c, int32_t *mn, int32_t *mx) {
   __shared__ int32_t s_mn[kT / 32], s_mx[kT / 32];
-  const int64_t p0 = (int64_t)blockIdx.x * kT;
   const int64_t p = p0 + threadIdx.x;
   const bool act = p < A;
   const int s = act ? seg[p] : -1;
@@ -212,18 +205,21 @@ __global__ void __launch_bounds__(kT) k_sp_minmax(const int32_t *stg, const int3
   }
 }
 
-// Left records fill [lo, lo + nl) from the start, right ones [lo + nl, lo + m)
-// from the end, so neither side needs the other's count first.
-__global__ void __launch_bounds__(kT) k_sp_scatter(const int32_t *stg, const int32_t *seg, int64_t A, int dim,
-                                                   int c, int t, const int32_t *mn, const int32_t *mx,
-                                                   const int64_t *lo, const int32_t *n, uint32_t *curL,
-                                                   uint32_t *curR, const SpTree *T, int32_t *stg_out,
-                                                   int32_t *seg_out, int32_t *mn_next, int32_t *mx_next) {
+// The records [p0, p0 + kT) of level t.  Left records fill [lo, lo + nl) from
+// the start, right ones [lo + nl, lo + m) from the end, so neither side needs
+// the other's count first.
+__device__ __forceinline__ void sp_scatter(const SpLevels &P, int t, int64_t p0, int64_t A) {
+  const int dim = P.dim, c = t % dim;
+  const int32_t *stg = P.stg[t & 1], *seg = P.seg[t & 1], *mn = P.mn[t & 1], *mx = P.mx[t & 1];
+  int32_t *mn_next = P.mn[(t & 1) ^ 1], *mx_next = P.mx[(t & 1) ^ 1];
+  const int64_t *lo = P.lo[t & 1];
+  const int32_t *n = P.n[t & 1];
+  uint32_t *curL = P.curL, *curR = P.curR;
+  const SpTree *T = P.T;
   __shared__ uint32_t s_cnt[2][kT / 32];
   __shared__ uint32_t s_base[2];
   __shared__ int32_t s_bnd[4][kT / 32];   // per warp: left min, left max, right min, right max
   const int rs = rec_ints(dim);
-  const int64_t p0 = (int64_t)blockIdx.x * kT;
   const int64_t p = p0 + threadIdx.x;
   const bool act = p < A;
   const int s = act ? seg[p] : -1;
@@ -311,38 +307,86 @@ __global__ void __launch_bounds__(kT) k_sp_scatter(const int32_t *stg, const int
   if (t + 1 == tr.h) {                    // the children are leaves: into the tree
     copy_rec(tr.pts + (pos - tr.toff) * rs, stg + p * rs, rs);
   } else {
-    copy_rec(stg_out + pos * rs, stg + p * rs, rs);
-    seg_out[pos] = 2 * s + (left ? 0 : 1);
+    copy_rec(P.stg[(t & 1) ^ 1] + pos * rs, stg + p * rs, rs);
+    P.seg[(t & 1) ^ 1][pos] = 2 * s + (left ? 0 : 1);
   }
 }
 
-// Per segment: the node's key and children, the children's bounds for the
-// next level, or the leaves' offsets and records when the children are leaves.
-__global__ void k_sp_split(int t, int64_t N, const int32_t *mn, const int32_t *mx, const int64_t *lo,
-                           const int32_t *n, const uint32_t *curL, const uint32_t *curR, const SpTree *T,
-                           int64_t *lo_next, int32_t *n_next) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= N) return;
+// Segment s of level t: the node's key and children, the children's bounds for
+// the next level, or the leaves' offsets and records when the children are
+// leaves.
+__device__ __forceinline__ void sp_split(const SpLevels &P, int t, int64_t s) {
   const int j = (int)(s >> t);
   const int64_t i = s & (((int64_t)1 << t) - 1);
-  const SpTree &tr = T[j];
-  const int64_t m = n[s];
-  const int64_t nl = curL[s];
-  if (nl + (int64_t)curR[s] != m) atomicOr(tr.err, kErrPartition);
-  const int64_t v = m > 0 ? ((int64_t)mn[s] + (int64_t)mx[s]) >> 1 : 0;
+  const SpTree &tr = P.T[j];
+  const int64_t lo = P.lo[t & 1][s], m = P.n[t & 1][s];
+  const int64_t nl = P.curL[s];
+  if (nl + (int64_t)P.curR[s] != m) atomicOr(tr.err, kErrPartition);
+  const int64_t v = m > 0 ? ((int64_t)P.mn[t & 1][s] + (int64_t)P.mx[t & 1][s]) >> 1 : 0;
   const int l = tr.h + 1;
   const int cl = veb_slot32(l, t + 1, 2 * (int)i), cr = veb_slot32(l, t + 1, 2 * (int)i + 1);
   tr.node[veb_slot32(l, t, (int)i)] = Node{(uint64_t)((v << 31) | 0x7FFFFFFF), cl, cr};
   if (t + 1 == tr.h) {
-    tr.leaf_off[2 * i] = (int32_t)(lo[s] - tr.toff);
-    tr.leaf_off[2 * i + 1] = (int32_t)(lo[s] + nl - tr.toff);
+    tr.leaf_off[2 * i] = (int32_t)(lo - tr.toff);
+    tr.leaf_off[2 * i + 1] = (int32_t)(lo + nl - tr.toff);
     tr.node[cl] = Node{0, (int32_t)(-1 - 2 * i), 0};
     tr.node[cr] = Node{0, (int32_t)(-2 - 2 * i), 0};
   } else {
-    lo_next[2 * s] = lo[s];
+    int64_t *lo_next = P.lo[(t & 1) ^ 1];
+    int32_t *n_next = P.n[(t & 1) ^ 1];
+    lo_next[2 * s] = lo;
     n_next[2 * s] = (int32_t)nl;
-    lo_next[2 * s + 1] = lo[s] + nl;
+    lo_next[2 * s + 1] = lo + nl;
     n_next[2 * s + 1] = (int32_t)(m - nl);
+  }
+}
+
+__global__ void __launch_bounds__(kT, kSpBlocks) k_sp_levels(const __grid_constant__ SpLevels P) {
+  const int64_t t0 = (int64_t)blockIdx.x * kT + threadIdx.x, step = (int64_t)gridDim.x * kT;
+  const int64_t r0 = (int64_t)blockIdx.x * kT;   // the block's first record, a multiple of kT (whole blocks go on)
+  auto clear_cursors = [&](int64_t s) {
+    P.curL[s] = 0;
+    P.curR[s] = 0;
+  };
+  auto clear_bounds = [&](int t, int64_t s) {
+    P.mn[t & 1][s] = INT32_MAX;
+    P.mx[t & 1][s] = INT32_MIN;
+  };
+  // bounds of every splitting tree; the leaf-offset sentinels; the single leaf
+  // of a tree with h = 0
+  for (int64_t j = t0; j < P.ntree; j += step) {
+    const SpTree &tr = P.T[j];
+    tr.leaf_off[(int64_t)1 << tr.h] = (int32_t)tr.size;
+    if (tr.h == 0) {
+      tr.leaf_off[0] = 0;
+      tr.node[0] = Node{0, -1, 0};
+    } else {
+      P.lo[0][j] = tr.toff;
+      P.n[0][j] = (int32_t)tr.size;
+      clear_cursors(j);
+    }
+  }
+  if (P.hmax == 0) return;
+  for (int t = 0; t < min(P.hmax, 2); ++t)
+    for (int64_t s = t0; s < P.seg_n[t]; s += step) clear_bounds(t, s);
+  unsigned epoch = 0;
+  grid_barrier(P.bar, epoch, P.err);
+  for (int64_t p = r0; p < P.rec_n[0]; p += step)
+    sp_minmax(P.stg[0], P.seg[0], p, P.rec_n[0], rec_ints(P.dim), 0, P.mn[0], P.mx[0]);
+  for (int t = 0; t < P.hmax; ++t) {
+    grid_barrier(P.bar, epoch, P.err);
+    const int64_t A = P.rec_n[t], N = P.seg_n[t];
+    for (int64_t p = r0; p < A; p += step) sp_scatter(P, t, p, A);
+    grid_barrier(P.bar, epoch, P.err);
+    // a thread clears for the next levels what it alone reads here (s), and
+    // the places behind N, which nobody reads here: a level has at most twice
+    // the segments of the one before it
+    const int64_t N1 = t + 1 < P.hmax ? P.seg_n[t + 1] : 0, N2 = t + 2 < P.hmax ? P.seg_n[t + 2] : 0;
+    for (int64_t s = t0; s < N; s += step) {
+      sp_split(P, t, s);
+      for (int64_t i = s; i < N1; i += N) clear_cursors(i);
+      for (int64_t i = s; i < N2; i += N) clear_bounds(t, i);
+    }
   }
 }
 
@@ -544,10 +588,14 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   const size_t b_i32 = al256((size_t)Nmax * 4), b_i64 = al256((size_t)Nmax * 8);
   const size_t b_tr = al256(ntree * sizeof(SpTree)), b_ga = al256(ga.size() * sizeof(SpGather));
   const size_t b_gpre = al256(gpre.size() * 8), b_lpre = al256(leaf_pre.size() * 8);
-  // zeroed: gather cursors, sums of squared leaf sizes, the box kernel's barrier
+  // zeroed: gather cursors, sums of squared leaf sizes, the two barriers
   const size_t b_cur = 2 * al256((size_t)ntree * 8) + 256;
   std::vector<int64_t> depth(std::max(hmax, 1), 0);
-  for (int t = 0; t < hmax; ++t) depth[t] = (int64_t)nact[t] << t;
+  std::vector<int64_t> recs(depth.size(), 0);   // records still splitting at each level
+  for (int t = 0; t < hmax; ++t) {
+    depth[t] = (int64_t)nact[t] << t;
+    recs[t] = tr[nact[t] - 1].toff + tr[nact[t] - 1].size;
+  }
   const size_t b_depth = al256(depth.size() * 8);
   std::vector<TreeSeg> pk;
   std::vector<int64_t> pk_pre;
@@ -558,7 +606,7 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   }
   const size_t b_pk = al256(pk.size() * sizeof(TreeSeg)), b_pkpre = al256(pk_pre.size() * 8);
   const size_t total = 2 * b_stg + 2 * b_seg + 6 * b_i32 + 2 * (b_i64 + b_i32) + b_tr + b_ga + b_gpre + b_lpre +
-                       b_cur + b_pk + b_pkpre + b_depth;
+                       b_cur + b_pk + b_pkpre + 2 * b_depth;
   void *block = nullptr;
   int st = dev_alloc(af, &block, total, s);
   if (st) return st;
@@ -585,64 +633,57 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   nn[0] = (int32_t *)take(b_i32);
   lo[1] = (int64_t *)take(b_i64);
   nn[1] = (int32_t *)take(b_i32);
-  SpTree *d_tr = (SpTree *)take(b_tr);
-  SpGather *d_ga = (SpGather *)take(b_ga);
-  int64_t *d_gpre = (int64_t *)take(b_gpre), *d_lpre = (int64_t *)take(b_lpre);
+  // the tables, in one upload
+  std::vector<unsigned char> img;
+  unsigned char *const tables = p;
+  auto table = [&](const void *src, size_t bytes, size_t room) {
+    img.resize((size_t)(p - tables) + bytes);
+    if (bytes) memcpy(img.data() + (p - tables), src, bytes);
+    return take(room);
+  };
+  SpTree *d_tr = (SpTree *)table(tr.data(), ntree * sizeof(SpTree), b_tr);
+  SpGather *d_ga = (SpGather *)table(ga.data(), ga.size() * sizeof(SpGather), b_ga);
+  int64_t *d_gpre = (int64_t *)table(gpre.data(), gpre.size() * 8, b_gpre);
+  int64_t *d_lpre = (int64_t *)table(leaf_pre.data(), leaf_pre.size() * 8, b_lpre);
+  int64_t *d_depth = (int64_t *)table(depth.data(), depth.size() * 8, b_depth);
+  int64_t *d_recs = (int64_t *)table(recs.data(), recs.size() * 8, b_depth);
+  TreeSeg *d_pk = (TreeSeg *)table(pk.data(), pk.size() * sizeof(TreeSeg), b_pk);
+  int64_t *d_pkpre = (int64_t *)table(pk_pre.data(), pk_pre.size() * 8, b_pkpre);
   unsigned long long *cursor = (unsigned long long *)take(b_cur);
   unsigned long long *sq = (unsigned long long *)((char *)cursor + al256((size_t)ntree * 8));
-  unsigned *bar = (unsigned *)((char *)cursor + 2 * al256((size_t)ntree * 8));
-  int64_t *d_depth = (int64_t *)take(b_depth);
-  TreeSeg *d_pk = (TreeSeg *)take(b_pk);
-  int64_t *d_pkpre = (int64_t *)take(b_pkpre);
-  st = h2d(d_tr, tr.data(), ntree * sizeof(SpTree), s);
-  if (!st) st = h2d(d_ga, ga.data(), ga.size() * sizeof(SpGather), s);
-  if (!st) st = h2d(d_gpre, gpre.data(), gpre.size() * 8, s);
-  if (!st) st = h2d(d_lpre, leaf_pre.data(), leaf_pre.size() * 8, s);
-  if (!st && !pk.empty()) st = h2d(d_pk, pk.data(), pk.size() * sizeof(TreeSeg), s);
-  if (!st) st = h2d(d_depth, depth.data(), depth.size() * 8, s);
-  if (!st) st = h2d(d_pkpre, pk_pre.data(), pk_pre.size() * 8, s);
-  if (!st) st = small_zero(cursor, b_cur, s);
+  unsigned *bar = (unsigned *)((char *)cursor + 2 * al256((size_t)ntree * 8));   // and one more 128 bytes on
+  st = h2d_and_zero(tables, img.data(), img.size(), cursor, b_cur, s);
   if (st) {
     dev_free(af, block, total, s);
     return st;
   }
-  // ---- gather, roots ----
+  // ---- gather, levels ----
   if (gpre.back() > 0) {
     KScope ks_(kK_sp_gather, s);
     k_sp_gather<<<(unsigned)cdiv(gpre.back(), kT), kT, 0, s>>>(d_ga, d_gpre, (int)ga.size(), d_tr, dim, stg[0],
                                                                seg[0], cursor);
   }
   {
-    KScope ks_(kK_sp_split, s);
-    k_sp_roots<<<(unsigned)cdiv(ntree, 128), 128, 0, s>>>(d_tr, ntree, lo[0], nn[0]);
-  }
-  // ---- levels ----
-  for (int t = 0; t < hmax; ++t) {
-    const int64_t N = (int64_t)nact[t] << t;
-    const int64_t A = tr[nact[t] - 1].toff + tr[nact[t] - 1].size;   // records still splitting
-    const int c = t % dim;
-    const int cur = t & 1, nxt = cur ^ 1;
-    if (t == 0) {   // the first level's bounds by a pass of their own; later ones come from the scatter
-      KScope ks_(kK_sp_minmax, s);
-      k_sp_level_init<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(0, curL, curR, N, mn[cur], mx[cur]);
-      k_sp_minmax<<<(unsigned)cdiv(A, kT), kT, 0, s>>>(stg[cur], seg[cur], A, rs, c, mn[cur], mx[cur]);
+    SpLevels P;
+    P.T = d_tr;
+    P.seg_n = d_depth;
+    P.rec_n = d_recs;
+    P.ntree = ntree;
+    P.dim = dim;
+    P.hmax = hmax;
+    for (int i = 0; i < 2; ++i) {
+      P.stg[i] = stg[i];
+      P.seg[i] = seg[i];
+      P.mn[i] = mn[i];
+      P.mx[i] = mx[i];
+      P.lo[i] = lo[i];
+      P.n[i] = nn[i];
     }
-    const int64_t Nn = t + 1 < hmax ? (int64_t)nact[t + 1] << (t + 1) : 0;
-    {
-      KScope ks_(kK_sp_minmax, s);
-      k_sp_level_init<<<(unsigned)cdiv(std::max(N, Nn), 256), 256, 0, s>>>(N, curL, curR, Nn, mn[nxt], mx[nxt]);
-    }
-    {
-      KScope ks_(kK_sp_scatter, s);
-      k_sp_scatter<<<(unsigned)cdiv(A, kT), kT, 0, s>>>(stg[cur], seg[cur], A, dim, c, t, mn[cur], mx[cur], lo[cur],
-                                                        nn[cur], curL, curR, d_tr, stg[nxt], seg[nxt], mn[nxt],
-                                                        mx[nxt]);
-    }
-    {
-      KScope ks_(kK_sp_split, s);
-      k_sp_split<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(t, N, mn[cur], mx[cur], lo[cur], nn[cur], curL, curR, d_tr,
-                                                       lo[nxt], nn[nxt]);
-    }
+    P.curL = curL;
+    P.curR = curR;
+    P.bar = bar + 32;
+    P.err = bt[0].err;
+    st = launch_coop((const void *)k_sp_levels, kT, std::max<int64_t>(S, ntree), &P, kK_sp_levels, 0, s);
   }
   // ---- boxes, live counts, packed records ----
   {
@@ -656,7 +697,7 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
     P.hmax = hmax;
     P.bar = bar;
     P.err = bt[0].err;
-    st = launch_coop((const void *)k_sp_boxes, kT, leaves, &P, kK_sp_box, 0, s);
+    if (!st) st = launch_coop((const void *)k_sp_boxes, kT, leaves, &P, kK_sp_box, 0, s);
   }
   launch_pack_nodes(d_pk, d_pkpre, (int)pk.size(), pk_pre.back(), s);
   const int err = st ? st : cuda_check(cudaGetLastError(), "spatial build kernels");
