@@ -61,6 +61,7 @@ def test_dims(dim, k):
     check(f, live, q[:1], k)
     # queries off the grid (the C ABI asks for grid points; nothing depends on it)
     check(f, live, q[:5] - (1 << 20), k)
+    check(f, live, (q[:5] - (1 << 19)) * 1000, k)
 
 
 @pytest.mark.parametrize("dim,distinct", [(2, 3), (3, 1), (5, 40)])
