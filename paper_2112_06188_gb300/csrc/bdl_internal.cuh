@@ -764,10 +764,13 @@ int upload_knn_table(const std::vector<KnnCall> &calls, void *table, int64_t *wa
 int launch_knn_table(const void *table, int njobs, int64_t warps, int dim, int k, const KnnShape &sh,
                      unsigned long long *stats, cudaStream_t s);
 // The kernel with one warp per query (knn_warp.cu): whether a launch of m
-// queries on n points takes it, and its launches; a warp answers
+// queries on forests of n points takes it, and its launches; a warp answers
 // knn_warp_per(m) queries in turn (upload_knn_table with qpw = that).
 bool knn_by_warp(int dim, int k, int64_t m, int64_t n, bool skewed);
 int knn_warp_per(int64_t m);
+// The n that stands for several forests: a query meets forests of mn / m
+// points, n in all.
+int64_t knn_forest_size(double mn, int64_t m, double n);
 // The same for the calls of one launch together: 0 for the thread-per-query
 // kernel, otherwise the queries per warp.
 int knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k);

@@ -1489,13 +1489,15 @@ static int knn_many(bdl_forest *const *F, int nf, const int32_t *const *q, const
   // an update, about 500 points in the buffer: the whole step 493 -> 435 us.
   std::vector<char> scan(nf, 0);
   if (!counts) {
-    int64_t pairs = 0, md[kMaxDim + 1] = {}, nd[kMaxDim + 1] = {};
+    int64_t pairs = 0, md[kMaxDim + 1] = {};
+    double mn[kMaxDim + 1] = {}, nd[kMaxDim + 1] = {};   // the size of forest that a query meets, times md; all points
     bool stats[kMaxDim + 1] = {};
     for (int i = 0; i < nf; ++i) {
       const int d = F[i]->dim;
       pairs += F[i]->buf_dirty ? m[i] * F[i]->nbuf : 0;
       md[d] += m[i];
-      nd[d] += F[i]->live;
+      mn[d] += (double)m[i] * (double)F[i]->live;
+      nd[d] += (double)F[i]->live;
       stats[d] = stats[d] || F[i]->knn_stats;
     }
     signed char by_warp[kMaxDim + 1][2];   // the rule's answers so far (it takes logarithms)
@@ -1506,7 +1508,7 @@ static int knn_many(bdl_forest *const *F, int nf, const int32_t *const *q, const
       scan[i] = f->buf_dirty && !f->buf_scanned && f->nbuf > 0 && m[i] > 0 && !stats[d];
       if (!scan[i]) continue;
       const bool skewed = skewed_leaves(f);
-      if (by_warp[d][skewed] < 0) by_warp[d][skewed] = knn_by_warp(d, k, md[d], nd[d], skewed);
+      if (by_warp[d][skewed] < 0) by_warp[d][skewed] = knn_by_warp(d, k, md[d], knn_forest_size(mn[d], md[d], nd[d]), skewed);
       scan[i] = by_warp[d][skewed];
     }
     for (int i = 0; i < nf; ++i)

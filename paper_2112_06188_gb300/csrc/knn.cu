@@ -859,13 +859,17 @@ size_t batch_query_sort_bytes(const std::vector<KnnCall> &calls) {
 }
 
 int knn_by_warp(const std::vector<KnnCall> &calls, int dim, int k) {
-  int64_t m = 0, n = 0, ms = 0;
+  int64_t m = 0, ms = 0;
+  double mn = 0, n = 0;   // the size of forest that a query meets, times m; all points
   for (const auto &c : calls) {
     m += c.m;
     if (c.skewed) ms += c.m;
-    for (int t = 0; t < c.fv->ntrees; ++t) n += c.fv->tree[t].size;
+    double size = 0;
+    for (int t = 0; t < c.fv->ntrees; ++t) size += (double)c.fv->tree[t].size;
+    mn += (double)c.m * size;
+    n += size;
   }
-  return knn_by_warp(dim, k, m, n, 2 * ms > m) ? knn_warp_per(m) : 0;
+  return knn_by_warp(dim, k, m, knn_forest_size(mn, m, n), 2 * ms > m) ? knn_warp_per(m) : 0;
 }
 
 size_t knn_table_bytes(const std::vector<KnnCall> &calls) {

@@ -473,6 +473,16 @@ void warp_table(const KnnJob *jobs, const int64_t *job_warp, int njobs, int64_t 
 // with 32 19.2.  1M 7-D points, 50K queries: one per warp 0.99 ms, three 1.08.
 int knn_warp_per(int64_t m) { return (int)std::min<int64_t>(8, std::max<int64_t>(1, m / 30000)); }
 
+// Between the size of one forest, which sets the length of a walk, and the size
+// of all, which sets how far apart a warp's queries and its reads lie: their
+// geometric mean.  us by all / by one / by the mean: 64 forests of 10K 3-D
+// points, 1,200 queries each, k = 8: 304 / 257 / 258; 4-D, 3,000 queries, k = 5:
+// 675 / 482 / 483; 5-D, 5,000 queries: 1286 / 1338 / 1338; 32 forests of 12K
+// 7-D points, 10,000 queries, k = 1: 957 / 1333 / 957.
+int64_t knn_forest_size(double mn, int64_t m, double n) {
+  return (int64_t)std::sqrt(mn / (double)std::max<int64_t>(m, 1) * n);
+}
+
 // Where the two kernels cost the same: thousands of queries, for k = 1, 5, 16
 // and 32 on forests of 4,500, 55,000 and a million points (9999: beyond
 // 640,000, the most that was measured).  The warp-per-query kernel's time
