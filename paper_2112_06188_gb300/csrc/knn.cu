@@ -153,16 +153,29 @@ __device__ __forceinline__ void cmp_swap(float &a, int &ca, float &b, int &cb) {
   }
 }
 
-// A point record in registers, by 16-byte words.
+// 32 bytes in one load (src 32-byte aligned).
+__device__ __forceinline__ void read32(const int32_t *src, int32_t (&p)[8]) {
+  asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(p[0]), "=r"(p[1]), "=r"(p[2]), "=r"(p[3]), "=r"(p[4]), "=r"(p[5]), "=r"(p[6]), "=r"(p[7])
+      : "l"(src));
+}
+
+// A point record in registers.
 template <int D>
 __device__ __forceinline__ void read_rec(const int32_t *src, int32_t (&p)[rec_ints(D)]) {
+  // in one load where it has 32 bytes (4-D 799 -> 767 us, 5-D 996 -> 935; 6-D
+  // spills: 1,373 -> 1,530)
+  if constexpr (D == 4 || D == 5) {
+    read32(src, p);
+  } else {
 #pragma unroll
-  for (int c4 = 0; c4 < rec_ints(D); c4 += 4) {
-    const int4 v = *reinterpret_cast<const int4 *>(src + c4);
-    p[c4] = v.x;
-    p[c4 + 1] = v.y;
-    p[c4 + 2] = v.z;
-    p[c4 + 3] = v.w;
+    for (int c4 = 0; c4 < rec_ints(D); c4 += 4) {
+      const int4 v = *reinterpret_cast<const int4 *>(src + c4);
+      p[c4] = v.x;
+      p[c4 + 1] = v.y;
+      p[c4 + 2] = v.z;
+      p[c4 + 3] = v.w;
+    }
   }
 }
 
@@ -176,24 +189,48 @@ __device__ __forceinline__ void read_rec(const int32_t *src, int32_t (&p)[rec_in
 // point, after them it runs about as often as the lane with the most.
 // 10M 3-D points, 1M queries, k = 10: 2,761 -> 2,602 us (the filter unrolled
 // by 2, 3 and 8: 2,740 to 2,685).
+//
+// The lanes' reads lie in lines of their own, so each load costs the L1 data
+// pipe a pass per lane, and that pipe was the busiest unit (79% of its peak).
+// Records of 16 bytes are therefore read in pairs, from an even record on: the
+// one before pa and the one behind pz - 1 are left out of the mask (the array
+// is padded to 256 bytes, so the last pair lies inside it).  2,516 -> 2,468 us,
+// 2-D 997 -> 989 (with two, three, five pairs unrolled 2,755, 2,455, 2,930: the
+// ones that spill lose).
 template <int D, class TK>
 __device__ __forceinline__ void scan_leaf(const TreeView &T, int pa, int pz, const int32_t *q, int k, TK &best) {
   constexpr int rs = rec_ints(D);
-  for (int b = pa; b < pz; b += 32) {
+  constexpr bool kPairs = rs == 4;
+  for (int b = kPairs ? pa & ~1 : pa; b < pz; b += 32) {
     const int n = min(pz - b, 32);
     const int32_t *src = T.pts + (int64_t)b * rs;
     int32_t p[rs];
     unsigned in = 0;
-#pragma unroll 4
-    for (int i = 0; i < n; ++i) {
-      read_rec<D>(src + i * rs, p);
+    auto passes = [&](const int32_t *r) {
       float s = 0.f;
 #pragma unroll
       for (int c = 0; c < D; ++c) {
-        const float g = (float)(q[c] - p[c]);
+        const float g = (float)(q[c] - r[c]);
         s = fmaf(g, g, s);
       }
-      if (!(s > best.kdf) && p[D] >= 0) in |= 1u << i;
+      return !(s > best.kdf) && r[D] >= 0;
+    };
+    if constexpr (kPairs) {
+#pragma unroll 1
+      for (int i = 0; i < n; i += 2) {
+        int32_t w[8];
+        read32(src + i * 4, w);
+        if (passes(w)) in |= 1u << i;
+        if (passes(w + 4)) in |= 2u << i;
+      }
+      if (b < pa) in &= ~1u;
+      if (n < 32) in &= (1u << n) - 1;
+    } else {
+#pragma unroll 4
+      for (int i = 0; i < n; ++i) {
+        read_rec<D>(src + i * rs, p);
+        if (passes(p)) in |= 1u << i;
+      }
     }
     while (in) {
       const int i = __ffs(in) - 1;
@@ -298,12 +335,24 @@ __device__ __forceinline__ void walk_packed(const KnnJob &J, const TreeView &T, 
       int4 cd, lv;
       float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;   // box distances (see box_dist_f)
       if constexpr (!packed_by_entry(D)) {
-        cd = *reinterpret_cast<const int4 *>(r);
-        lv = *reinterpret_cast<const int4 *>(r + 4);
+        // a 3-D record (128 bytes) in four loads: 2,468 -> 2,428 us, 100 clusters
+        // 1,808 -> 1,760 (2-D in three: 989 -> 1,008)
+        auto two = [&](int at, int4 &x, int4 &y) {
+          if constexpr (D == 3) {
+            int32_t w[8];
+            read32(r + at, w);
+            x = make_int4(w[0], w[1], w[2], w[3]);
+            y = make_int4(w[4], w[5], w[6], w[7]);
+          } else {
+            x = *reinterpret_cast<const int4 *>(r + at);
+            y = *reinterpret_cast<const int4 *>(r + at + 4);
+          }
+        };
+        two(0, cd, lv);
 #pragma unroll
         for (int c = 0; c < D; ++c) {
-          const int4 lo = *reinterpret_cast<const int4 *>(r + 8 + 8 * c);
-          const int4 hi = *reinterpret_cast<const int4 *>(r + 12 + 8 * c);
+          int4 lo, hi;
+          two(8 + 8 * c, lo, hi);
           const int32_t x = q[c];
           // the gap to [lo, hi] (lo <= hi): at most one difference is positive
           const float g0 = (float)max(max(lo.x - x, x - hi.x), 0);
