@@ -25,8 +25,8 @@
 //
 // What bounds it: small batches by the chain of about 2 x 20 rounds per query
 // (a dependent L2 read each); large ones by instruction issue (about 3,900
-// warp instructions per query on 2M 3-D points, 10,000 on 2M 7-D ones, 65 to
-// 78% of the issue slots) and by the shared/L1 data pipe (53 to 67%).
+// warp instructions per query on 2M 3-D points, 9,500 on 2M 7-D ones, 67 to
+// 75% of the issue slots) and by the shared/L1 data pipe (53 to 59%).
 // Measured against the thread-per-query kernel (1M 5-D points, k = 10, 316
 // queries: 1,014 -> 47 us; 50K 16-D points, k = 8, 1,000 queries: 1,495 -> 52;
 // 500K 4-D points, k = 32, 100K queries: 3,620 -> 768; 10M 7-D points of 100
