@@ -163,8 +163,8 @@ __device__ __forceinline__ void read32(const int32_t *src, int32_t (&p)[8]) {
 // A point record in registers.
 template <int D>
 __device__ __forceinline__ void read_rec(const int32_t *src, int32_t (&p)[rec_ints(D)]) {
-  // in one load where it has 32 bytes (4-D 799 -> 767 us, 5-D 996 -> 935; 6-D
-  // spills: 1,373 -> 1,530)
+  // in one load where it has 32 bytes (100K points, 500K queries, 4-D, k = 5:
+  // 794 -> 766 us; 1M queries, 5-D, k = 1: 998 -> 934; 6-D spills: 1,373 -> 1,520)
   if constexpr (D == 4 || D == 5) {
     read32(src, p);
   } else {
@@ -206,16 +206,16 @@ __device__ __forceinline__ void scan_leaf(const TreeView &T, int pa, int pz, con
     const int32_t *src = T.pts + (int64_t)b * rs;
     int32_t p[rs];
     unsigned in = 0;
-    auto passes = [&](const int32_t *r) {
-      float s = 0.f;
-#pragma unroll
-      for (int c = 0; c < D; ++c) {
-        const float g = (float)(q[c] - r[c]);
-        s = fmaf(g, g, s);
-      }
-      return !(s > best.kdf) && r[D] >= 0;
-    };
     if constexpr (kPairs) {
+      auto passes = [&](const int32_t *r) {
+        float s = 0.f;
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+          const float g = (float)(q[c] - r[c]);
+          s = fmaf(g, g, s);
+        }
+        return !(s > best.kdf) && r[D] >= 0;
+      };
 #pragma unroll 1
       for (int i = 0; i < n; i += 2) {
         int32_t w[8];
@@ -226,10 +226,17 @@ __device__ __forceinline__ void scan_leaf(const TreeView &T, int pa, int pz, con
       if (b < pa) in &= ~1u;
       if (n < 32) in &= (1u << n) - 1;
     } else {
+      // (the test through a lambda as above: 5-D 934 -> 1,000 us)
 #pragma unroll 4
       for (int i = 0; i < n; ++i) {
         read_rec<D>(src + i * rs, p);
-        if (passes(p)) in |= 1u << i;
+        float s = 0.f;
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+          const float g = (float)(q[c] - p[c]);
+          s = fmaf(g, g, s);
+        }
+        if (!(s > best.kdf) && p[D] >= 0) in |= 1u << i;
       }
     }
     while (in) {
