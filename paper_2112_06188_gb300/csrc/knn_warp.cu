@@ -506,7 +506,8 @@ int64_t knn_forest_size(double mn, int64_t m, double n) {
 //   dim 7, k = 1:  n = 10,000, 160K 554 / 343, 320K 554 / 586
 // Over all 2,688 of those launches the choice costs 1% more than the better
 // kernel each time (a line in k alone: 3.4%, and up to 3.3 times on small
-// forests in dimensions 4 to 7).
+// forests in dimensions 4 to 7).  (Measured before the thread-per-query
+// kernel's 32-byte loads, which took 1 to 8% off its times in 2 to 5 dimensions.)
 //
 // Leaves of hundreds of points and more (spatial-median trees of clustered
 // points) are scanned by one lane in the thread-per-query kernel, 32 points at
