@@ -402,11 +402,21 @@ enum : unsigned long long {
 // counter that the last block resets and a generation word behind it took
 // about 6 us with 304 blocks).  Writes before the barrier are visible after it
 // (block barrier, then a device-scope fence by the arriving thread, cumulative
-// over the block's writes, and another after the wait).  The wait is bounded:
-// after kBarrierPolls polls (about a second) the block sets kErrBarrier in
-// *err and goes on, so a lost block never hangs the GPU; the call then fails
-// with BDL_EINTERNAL.
-constexpr unsigned kBarrierPolls = 1u << 21;
+// over the block's writes, and another after the wait).
+//
+// The wait is bounded by time: between two barriers a block may have much to
+// do (a select over hundreds of millions of equal coordinates in one block
+// takes about a second), so a block gives up after kBarrierNs, far above
+// that.  It then sets kErrBarrier in *err, lets every later wait of the launch
+// through (kBarrierOpen stands above any count of arrivals) and goes on, so a
+// lost block never hangs the GPU; the call then fails with BDL_EINTERNAL.
+constexpr unsigned long long kBarrierNs = 10000000000ull;
+constexpr unsigned kBarrierOpen = 1u << 30;
+__device__ __forceinline__ unsigned long long now_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
 __device__ __forceinline__ void grid_barrier(unsigned *bar, unsigned &epoch, unsigned long long *err) {
   __syncthreads();
   epoch += gridDim.x;
@@ -414,11 +424,14 @@ __device__ __forceinline__ void grid_barrier(unsigned *bar, unsigned &epoch, uns
     __threadfence();
     atomicAdd(bar, 1u);
     volatile unsigned *seen = bar;
-    unsigned polls = 0;
-    while ((int)(*seen - epoch) < 0) {
-      if (++polls > kBarrierPolls) {
+    unsigned long long since = 0;
+    for (unsigned polls = 1; (int)(*seen - epoch) < 0; ++polls) {
+      if (polls % 1024) continue;
+      const unsigned long long t = now_ns();
+      if (since == 0) since = t;
+      if (t - since > kBarrierNs) {
         atomicOr(err, kErrBarrier);
-        break;
+        atomicOr(bar, kBarrierOpen);
       }
     }
     __threadfence();

@@ -401,20 +401,44 @@ __global__ void __launch_bounds__(kT, kSpBlocks) k_sp_levels(const __grid_consta
 // depth and not the leaves, so clustered points leave leaves of thousands,
 // and a lane per leaf took as long as the largest one.  1M 2-D points of 100
 // clusters, a batch of 100K inserted and the buffer's tree: 1,121 us in 24
-// launches, this way 174 in two.
+// launches, this way 174 in two.  Points in one place, or nearly, leave a leaf
+// of any size: those of more than kHugeLeaf points are listed and dealt to
+// all warps in pieces, so that the other blocks never wait at a barrier for
+// one warp to go through a leaf of millions.
 constexpr int kLaneLeaf = 32;
+constexpr int kHugeLeaf = 8192;
+
+struct HugeLeaf {
+  int32_t tree, leaf;
+};
 
 struct SpBoxParams {
   const SpTree *T;
   const int64_t *leaf_pre;  // [ntree + 1] prefix of the trees' leaves
   const int64_t *depth;     // [hmax] nodes of each depth over the trees that have it
   unsigned long long *sq;   // [ntree] sum of the squared leaf sizes (zeroed)
+  HugeLeaf *huge;           // the leaves of more than kHugeLeaf points ...
+  unsigned *nhuge;          // ... and their number (zeroed)
   int ntree, dim, hmax;
   unsigned *bar;
   unsigned long long *err;
 };
 
 constexpr int64_t kOneBlockNodes = 1024;   // depths of at most so many nodes are one block's
+
+// Smallest and largest of x[r * rs] over [a, b), by a whole warp.
+__device__ __forceinline__ void warp_extent(const int32_t *x, int rs, int64_t a, int64_t b, int32_t &lo, int32_t &hi) {
+  lo = INT32_MAX;
+  hi = INT32_MIN;
+#pragma unroll 4
+  for (int64_t r = a + (threadIdx.x & 31); r < b; r += 32) {
+    const int32_t y = x[r * rs];
+    lo = min(lo, y);
+    hi = max(hi, y);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+}
 
 __device__ __forceinline__ void sp_leaf_boxes(const SpBoxParams &P, int64_t x0) {
   const int lane = threadIdx.x & 31, dim = P.dim, rs = rec_ints(dim);
@@ -455,7 +479,15 @@ __device__ __forceinline__ void sp_leaf_boxes(const SpBoxParams &P, int64_t x0) 
   } else if (ok) {
     atomicAdd(&P.sq[j], sq);
   }
-  unsigned big = __ballot_sync(0xffffffffu, ok && !own);
+  const bool huge = ok && b - a > kHugeLeaf;
+  if (huge) {
+    for (int c = 0; c < dim; ++c) {
+      tr.box[v * 2 * dim + c] = INT32_MAX;
+      tr.box[v * 2 * dim + dim + c] = INT32_MIN;
+    }
+    P.huge[atomicAdd(P.nhuge, 1u)] = HugeLeaf{j, (int32_t)leaf};
+  }
+  unsigned big = __ballot_sync(0xffffffffu, ok && !own && !huge);
   while (big) {
     const int src = __ffs(big) - 1;
     big &= big - 1;
@@ -463,20 +495,39 @@ __device__ __forceinline__ void sp_leaf_boxes(const SpBoxParams &P, int64_t x0) 
     const int64_t wa = __shfl_sync(0xffffffffu, a, src), wb = __shfl_sync(0xffffffffu, b, src),
                   wv = __shfl_sync(0xffffffffu, v, src);
     for (int c = 0; c < dim; ++c) {
-      int32_t lo = INT32_MAX, hi = INT32_MIN;
-#pragma unroll 4
-      for (int64_t r = wa + lane; r < wb; r += 32) {
-        const int32_t y = w.pts[r * rs + c];
-        lo = min(lo, y);
-        hi = max(hi, y);
-      }
-      lo = __reduce_min_sync(0xffffffffu, lo);
-      hi = __reduce_max_sync(0xffffffffu, hi);
+      int32_t lo, hi;
+      warp_extent(w.pts + c, rs, wa, wb, lo, hi);
       if (lane == 0) {
         w.box[wv * 2 * dim + c] = lo;
         w.box[wv * 2 * dim + dim + c] = hi;
       }
     }
+  }
+}
+
+// The listed leaves' boxes, empty so far, from their points: kHugeLeaf at a
+// time, the pieces of all leaves one after another to the grid's warps.
+__device__ __forceinline__ void sp_huge_leaf_boxes(const SpBoxParams &P, unsigned nhuge) {
+  const int lane = threadIdx.x & 31, dim = P.dim, rs = rec_ints(dim);
+  const int64_t nwarp = (int64_t)gridDim.x * (kT / 32), warp = (int64_t)blockIdx.x * (kT / 32) + (threadIdx.x >> 5);
+  int64_t first = 0;   // the warp that takes the next leaf's first piece
+  for (unsigned e = 0; e < nhuge; ++e) {
+    const HugeLeaf H = P.huge[e];
+    const SpTree &tr = P.T[H.tree];
+    const int64_t a = tr.leaf_off[H.leaf], b = tr.leaf_off[H.leaf + 1], n = (b - a + kHugeLeaf - 1) / kHugeLeaf;
+    const int64_t v = veb_slot32(tr.h + 1, tr.h, H.leaf);
+    for (int64_t i = warp >= first ? warp - first : warp - first + nwarp; i < n; i += nwarp) {
+      const int64_t p = a + i * kHugeLeaf;
+      for (int c = 0; c < dim; ++c) {
+        int32_t lo, hi;
+        warp_extent(tr.pts + c, rs, p, min(p + kHugeLeaf, b), lo, hi);
+        if (lane == 0) {
+          atomicMin(&tr.box[v * 2 * dim + c], lo);
+          atomicMax(&tr.box[v * 2 * dim + dim + c], hi);
+        }
+      }
+    }
+    first = (first + n) % nwarp;
   }
 }
 
@@ -497,13 +548,18 @@ __global__ void __launch_bounds__(kT) k_sp_boxes(const SpBoxParams P) {
     if (t == 0 && tr.skew) *tr.skew = P.sq[s];   // to the host, whenever it arrives (a hint)
   };
   unsigned epoch = 0;
+  grid_barrier(P.bar, epoch, P.err);
+  const unsigned nhuge = *P.nhuge;   // (final: every leaf has been looked at)
+  if (nhuge > 0) {
+    sp_huge_leaf_boxes(P, nhuge);
+    grid_barrier(P.bar, epoch, P.err);
+  }
   int t = P.hmax - 1;
   for (; t >= 0 && P.depth[t] > kOneBlockNodes; --t) {
-    grid_barrier(P.bar, epoch, P.err);
     for (int64_t s = t0; s < P.depth[t]; s += step) node(t, s);
+    grid_barrier(P.bar, epoch, P.err);
   }
   // depths with few nodes: one block, with block barriers
-  grid_barrier(P.bar, epoch, P.err);
   if (blockIdx.x > 0) return;
   for (; t >= 0; --t) {
     for (int64_t s = threadIdx.x; s < P.depth[t]; s += blockDim.x) node(t, s);
@@ -588,7 +644,8 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   const size_t b_i32 = al256((size_t)Nmax * 4), b_i64 = al256((size_t)Nmax * 8);
   const size_t b_tr = al256(ntree * sizeof(SpTree)), b_ga = al256(ga.size() * sizeof(SpGather));
   const size_t b_gpre = al256(gpre.size() * 8), b_lpre = al256(leaf_pre.size() * 8);
-  // zeroed: gather cursors, sums of squared leaf sizes, the two barriers
+  const size_t b_huge = al256((size_t)(S / kHugeLeaf + 1) * sizeof(HugeLeaf));
+  // zeroed: gather cursors, sums of squared leaf sizes, the two barriers, the number of huge leaves
   const size_t b_cur = 2 * al256((size_t)ntree * 8) + 256;
   std::vector<int64_t> depth(std::max(hmax, 1), 0);
   std::vector<int64_t> recs(depth.size(), 0);   // records still splitting at each level
@@ -606,7 +663,7 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   }
   const size_t b_pk = al256(pk.size() * sizeof(TreeSeg)), b_pkpre = al256(pk_pre.size() * 8);
   const size_t total = 2 * b_stg + 2 * b_seg + 6 * b_i32 + 2 * (b_i64 + b_i32) + b_tr + b_ga + b_gpre + b_lpre +
-                       b_cur + b_pk + b_pkpre + 2 * b_depth;
+                       b_cur + b_pk + b_pkpre + 2 * b_depth + b_huge;
   void *block = nullptr;
   int st = dev_alloc(af, &block, total, s);
   if (st) return st;
@@ -633,6 +690,7 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   nn[0] = (int32_t *)take(b_i32);
   lo[1] = (int64_t *)take(b_i64);
   nn[1] = (int32_t *)take(b_i32);
+  HugeLeaf *huge = (HugeLeaf *)take(b_huge);
   // the tables, in one upload
   std::vector<unsigned char> img;
   unsigned char *const tables = p;
@@ -651,7 +709,7 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   int64_t *d_pkpre = (int64_t *)table(pk_pre.data(), pk_pre.size() * 8, b_pkpre);
   unsigned long long *cursor = (unsigned long long *)take(b_cur);
   unsigned long long *sq = (unsigned long long *)((char *)cursor + al256((size_t)ntree * 8));
-  unsigned *bar = (unsigned *)((char *)cursor + 2 * al256((size_t)ntree * 8));   // and one more 128 bytes on
+  unsigned *bar = (unsigned *)((char *)cursor + 2 * al256((size_t)ntree * 8));   // [0] and [32]; [16]: huge leaves
   st = h2d_and_zero(tables, img.data(), img.size(), cursor, b_cur, s);
   if (st) {
     dev_free(af, block, total, s);
@@ -692,6 +750,8 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
     P.leaf_pre = d_lpre;
     P.depth = d_depth;
     P.sq = sq;
+    P.huge = huge;
+    P.nhuge = bar + 16;
     P.ntree = ntree;
     P.dim = dim;
     P.hmax = hmax;
