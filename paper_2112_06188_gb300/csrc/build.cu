@@ -1530,6 +1530,7 @@ struct BoxWork {               // the nodes of one depth t of the trees with glo
 
 struct FinishParams {
   int dim, nlev;
+  int one;                     // depths 0 .. one - 1 are one block's (one_block_depths)
   const DTree *tree;
   const BoxWork *bw;           // [nlev], by depth
   unsigned *bar;
@@ -1550,14 +1551,10 @@ __device__ void box_up(const FinishParams &F, const BoxWork &W, int64_t g) {
   }
 }
 
-// Depths with few nodes are one block's: a block barrier costs it far less
-// than a grid barrier (10M 3-D points, 11 depths: 74 -> 45 us).
-constexpr int64_t kOneBlockNodes = 1024;
-
 __global__ void __launch_bounds__(256) k_build_finish(const FinishParams F) {
   unsigned epoch = 0;
   int t = F.nlev - 1;
-  for (; t >= 0 && F.bw[t].total > kOneBlockNodes; --t) {
+  for (; t >= F.one; --t) {
     const BoxWork &W = F.bw[t];
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < W.total;
          g += (int64_t)gridDim.x * blockDim.x)
@@ -1565,7 +1562,7 @@ __global__ void __launch_bounds__(256) k_build_finish(const FinishParams F) {
     grid_barrier(F.bar, epoch, F.err);
   }
   if (blockIdx.x > 0) return;
-  for (; t >= 0; --t) {   // (no deeper depth has fewer nodes)
+  for (; t >= 0; --t) {
     const BoxWork &W = F.bw[t];
     for (int64_t g = threadIdx.x; g < W.total; g += blockDim.x) box_up(F, W, g);
     __syncthreads();
@@ -2077,6 +2074,9 @@ int build_trees_object(bdl_forest *af, int dim, std::vector<BuildTree> &bt,
     FinishParams F;
     F.dim = dim;
     F.nlev = gmax;
+    std::vector<int64_t> nodes;
+    for (const auto &L : lv) nodes.push_back(L.nseg);
+    F.one = one_block_depths(nodes.data(), gmax);
     F.tree = d_tree;
     F.bw = (const BoxWork *)(plan + o_bw);
     F.bar = bar + 2;

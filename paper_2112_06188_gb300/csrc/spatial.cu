@@ -420,11 +420,10 @@ struct SpBoxParams {
   HugeLeaf *huge;           // the leaves of more than kHugeLeaf points ...
   unsigned *nhuge;          // ... and their number (zeroed)
   int ntree, dim, hmax;
+  int one;                  // depths 0 .. one - 1 are one block's (one_block_depths)
   unsigned *bar;
   unsigned long long *err;
 };
-
-constexpr int64_t kOneBlockNodes = 1024;   // depths of at most so many nodes are one block's
 
 // Smallest and largest of x[r * rs] over [a, b), by a whole warp.
 __device__ __forceinline__ void warp_extent(const int32_t *x, int rs, int64_t a, int64_t b, int32_t &lo, int32_t &hi) {
@@ -555,11 +554,10 @@ __global__ void __launch_bounds__(kT) k_sp_boxes(const SpBoxParams P) {
     grid_barrier(P.bar, epoch, P.err);
   }
   int t = P.hmax - 1;
-  for (; t >= 0 && P.depth[t] > kOneBlockNodes; --t) {
+  for (; t >= P.one; --t) {
     for (int64_t s = t0; s < P.depth[t]; s += step) node(t, s);
     grid_barrier(P.bar, epoch, P.err);
   }
-  // depths with few nodes: one block, with block barriers
   if (blockIdx.x > 0) return;
   for (; t >= 0; --t) {
     for (int64_t s = threadIdx.x; s < P.depth[t]; s += blockDim.x) node(t, s);
@@ -755,6 +753,7 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
     P.ntree = ntree;
     P.dim = dim;
     P.hmax = hmax;
+    P.one = one_block_depths(depth.data(), hmax);
     P.bar = bar;
     P.err = bt[0].err;
     if (!st) st = launch_coop((const void *)k_sp_boxes, kT, leaves, &P, kK_sp_box, 0, s);

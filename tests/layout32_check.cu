@@ -32,6 +32,13 @@ int main() {
       CHECK(t == t2 && i == i2);
     }
   }
+  // the depths that go to one block: none above them holds more nodes than
+  // that, also where trees of several heights make a shallow depth the largest
+  const int64_t even[] = {1, 2, 4, 8, 16, 32, 64, 128, 256, 512, 1024, 2048, 4096};
+  const int64_t mixed[] = {501, 1002, 2004, 4008, 8016, 16032, 32064, 64128, 128256, 512};
+  const int64_t many[] = {2000, 4000, 512};
+  CHECK(one_block_depths(even, 13) == 11 && one_block_depths(even, 5) == 5);
+  CHECK(one_block_depths(mixed, 10) == 2 && one_block_depths(many, 3) == 0 && one_block_depths(many, 0) == 0);
   puts(bad ? "BAD" : "ok");
   return bad != 0;
 }
