@@ -251,6 +251,15 @@ __host__ __device__ constexpr int packed_hi_at(int dim, int a, int c) {
   return packed_lo_at(dim, a, c) + (packed_by_entry(dim) ? 1 : 4);
 }
 
+// Node stack of the warp-per-query kernel.  A round takes up to eight records
+// off it and puts their 32 entries on; past kWWide entries it takes one record
+// at a time, each adding at most three entries net per level of records below
+// it.  Trees of 2^31 points in leaves of two are the tallest: kMaxHeight levels.
+constexpr int kMaxHeight = 30;
+constexpr int kWStack = 256;
+constexpr int kWWide = 184;
+static_assert(kWWide + 24 + 3 * ((kMaxHeight + 1) / 2) <= kWStack, "node stack of the tallest trees");
+
 __host__ __device__ inline int64_t quad_count(int H) {   // (4^H - 1) / 3 nodes in H 4-ary levels
   return (((int64_t)1 << (2 * H)) - 1) / 3;
 }

@@ -45,12 +45,8 @@ namespace bdl {
 namespace {
 
 constexpr int kWarpsPerBlock = 4;
-constexpr int kWStack = 256;    // node stack entries per warp
 constexpr int kWLeaves = 80;    // leaf stack entries per warp
 constexpr int kWTrees = kMaxLevel + 1;
-// Past this depth records are taken one at a time, each adding at most three
-// entries per 4-ary level (14 levels): 190 + 24 + 42 <= kWStack.
-constexpr int kWWide = 190;
 constexpr float kWBoundUp = 1.00000393390655517578125f;   // see TopK in knn.cu
 
 // What a walk needs of a tree.
@@ -305,8 +301,8 @@ __device__ __forceinline__ void warp_query(const KnnJob &J, WarpMem &W, const WT
       const uint64_t e = W.sel[r];
       tr = (uint32_t)(e >> 32) & 63u;
       const WTree &T = tree[tr];
-      if ((uint32_t)e >= (uint32_t)T.nrec) {
-        atomicOr(J.err, kErrChild);
+      if ((uint32_t)e >= (uint32_t)T.nrec || sp > kWStack - 4) {
+        atomicOr(J.err, (uint32_t)e >= (uint32_t)T.nrec ? kErrChild : kErrStack);
       } else {
         const int32_t *rp = T.pk + (int64_t)(uint32_t)e * rec;
         float s = 0.f;

@@ -39,6 +39,14 @@ int main() {
   const int64_t many[] = {2000, 4000, 512};
   CHECK(one_block_depths(even, 13) == 11 && one_block_depths(even, 5) == 5);
   CHECK(one_block_depths(mixed, 10) == 2 && one_block_depths(many, 3) == 0 && one_block_depths(many, 0) == 0);
+  // the tallest trees there can be (2^31 - 1 points, leaves of two), the levels
+  // of records that a walk goes down in one, and the warp-per-query kernel's
+  // node stack: what a wide round may leave on it and the rest one by one
+  CHECK(tree_height(INT32_MAX, 2) == kMaxHeight);
+  int levels = 0;
+  for (int t = 0; t < kMaxHeight; t += packed_step(kMaxHeight, t)) ++levels;
+  CHECK(kWWide - 8 + 32 + 3 * levels <= kWStack);
+  CHECK(kMaxLevel + 1 + 32 <= kWWide);   // (the walk starts with every tree's root)
   puts(bad ? "BAD" : "ok");
   return bad != 0;
 }
