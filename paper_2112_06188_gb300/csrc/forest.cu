@@ -826,15 +826,28 @@ static int build_and_commit(std::vector<InsertPlan> &plans, std::vector<BuildTre
   return commit_planned(plans, std::move(extra_fills), tmp, s);
 }
 
+// Whether work given to the stream is being recorded into a graph.
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) cudaGetLastError();   // (the launches will say so)
+  return cs != cudaStreamCaptureStatusNone;
+}
+
 // The buffer's points get a small kd-tree of their own for k-NN (the paper's
 // buffer tree), rebuilt when the buffer changed -- for many forests in shared
-// build launches.  A forest whose rebuild cannot get memory keeps scanning.
+// build launches.  A forest whose rebuild cannot get memory keeps scanning, and
+// so does one that is asked while the stream is being captured: a tree built
+// there would exist only once the graph has run, in the graph's own memory.
 static void refresh_btrees(bdl_forest *const *F, int nf, cudaStream_t s, const std::vector<char> *scan = nullptr) {
   std::vector<BuildTree> bt;
   std::vector<int> owner;
-  for (int i = 0; i < nf; ++i) {
+  auto stale = [&](int i) { return F[i]->buf_dirty && !(scan && (*scan)[i]); };
+  int first = 0;
+  while (first < nf && !stale(first)) ++first;
+  if (first == nf || capturing(s)) return;
+  for (int i = first; i < nf; ++i) {
     bdl_forest *f = F[i];
-    if (!f->buf_dirty || (scan && (*scan)[i])) continue;
+    if (!stale(i)) continue;
     f->buf_dirty = false;
     f->version++;
     // the tree's arrays have room for a full buffer and are rebuilt in place
