@@ -147,8 +147,12 @@ int bdl_knn(bdl_forest *f, const int32_t *q_dev, int64_t m, int k, int32_t *out_
  *  - Every call shares the one array and leaves its contents behind: calls
  *    whose work can overlap on the GPU (other streams, other forests on the
  *    same device) race with each other and must be ordered by the caller.
- *  - If the buffer changed since the last bdl_knn, its points are scanned
- *    instead of searched; results are the same as bdl_knn's. */
+ *  - While the buffer has no current tree its points are scanned instead of
+ *    searched; results are the same as bdl_knn's.  The first bdl_knn after a
+ *    change of the buffer builds the tree, with one exception: where the forest
+ *    was asked exactly once between its last two changes (calls of this function
+ *    count), a small batch is scanned too, and the next bdl_knn builds it.
+ *    Making a k-NN plan always builds it; a call in a stream capture never does. */
 int bdl_knn_noalloc(bdl_forest *f, const int32_t *q_dev, int64_t m, int k, int32_t *out_ids_dev,
                     int64_t *out_d2_dev, bdl_stream_t stream);
 
@@ -161,8 +165,8 @@ int bdl_knn_noalloc(bdl_forest *f, const int32_t *q_dev, int64_t m, int k, int32
  * bdl_knn_noalloc, bdl_knn_count, and by the batched calls and plans whose
  * forests[0] is f (a plan keeps the shape it was made with), where they take
  * the thread-per-query kernel (small batches and high dimensions take one warp
- * per query, which has one shape).  Results do not depend on the shape.  Other values: BDL_EINVAL, shape unchanged.  Host
- * only; no device work. */
+ * per query, which has one shape).  Results do not depend on the shape.  Other
+ * values: BDL_EINVAL, shape unchanged.  Host only; no device work. */
 int bdl_set_knn_shape(bdl_forest *f, int block_threads, int queries_per_warp);
 
 /* ---------------------------------------------------------------------

@@ -538,7 +538,11 @@ struct bdl_forest {
   bdl::Tree *trees[bdl::kMaxLevel] = {};
   bdl::Tree *btree = nullptr;    // kd-tree over the buffer's points (k-NN only), built lazily
   bool buf_dirty = true;         // the buffer changed since btree was built
-  bool buf_scanned = false;      // ... and a k-NN call has scanned it since (see knn_many)
+  // k-NN calls since the buffer last changed (0, 1, 2: more), and whether there
+  // was only one the last time there were any between two changes (see knn_many)
+  int knn_calls = 0;
+  bool asks_once = false;
+  bool in_call = false;          // (within knn_many: taking part in this call)
   uint64_t F = 0;
   int64_t live = 0;              // host mirror of the live count
   int64_t bytes_in_use = 0;
@@ -597,6 +601,8 @@ void *mapped(void *host);
 constexpr double kSkewedLeaf = 128;
 bool skewed_leaves(const bdl_forest *f);
 ForestView forest_view(const bdl_forest *f);
+// A k-NN call on the forest, for the choice of whether to build the buffer's tree.
+inline void count_knn_call(bdl_forest *f) { f->knn_calls = std::min(f->knn_calls + 1, 2); }
 // The view k-NN uses: the static trees plus the buffer's kd-tree.  With
 // build = true a stale buffer tree is rebuilt first (this allocates); with
 // build = false a stale one is left alone and the buffer is scanned instead.

@@ -698,6 +698,14 @@ static SortList sort_list(int32_t *ids, int64_t n) {
   return SortList{ids, (int32_t)n, np2};
 }
 
+// The buffer's points are others from here on: its tree is stale, and the k-NN
+// calls so far say whether the caller asks more than once between changes.
+static void buffer_changed(bdl_forest *f) {
+  if (f->knn_calls > 0) f->asks_once = f->knn_calls == 1;
+  f->knn_calls = 0;
+  f->buf_dirty = true;
+}
+
 // After the build and the tail fill: free cleared trees and the old buffer,
 // install the new trees.  A buffer that took reinserted ids is added to
 // `sorts` (it must stay in ascending id order).
@@ -725,8 +733,7 @@ static void commit_insert(InsertPlan &ip, std::vector<SortList> &sorts, cudaStre
     f->nbuf = ip.rem;
     f->F = ip.Fnew;
   }
-  f->buf_dirty = true;
-  f->buf_scanned = false;
+  buffer_changed(f);
   f->version++;
   ip.built.clear();
   ip.newbuf = nullptr;
@@ -1331,10 +1338,7 @@ static int erase_core(bdl_forest *const *F, int nf, const std::vector<EraseList>
     dev_err |= o[kMaxLevel + 1];
     if (ne[a] == 0) continue;   // nothing erased: counts and trees as they were
     f->version++;
-    if (o[0] != f->nbuf) {
-      f->buf_dirty = true;
-      f->buf_scanned = false;
-    }
+    if (o[0] != f->nbuf) buffer_changed(f);
     f->nbuf = o[0];
     int r = 0;
     for (int i = kMaxLevel - 1; i >= 0; --i)
@@ -1496,10 +1500,14 @@ static int knn_many(bdl_forest *const *F, int nf, const int32_t *const *q, const
       launch_query_sort(q[i], m[i], F[i]->dim, (char *)scratch + a256((size_t)m[i] * 4), perm[i], s);
     }
   }
-  // The first small call after an update scans the buffer (a warp per query
-  // reads 32 of its points at a time) instead of building its tree, a chain of
-  // five launches; a second one builds it.  1M 5-D points, 1,009 queries after
-  // an update, about 500 points in the buffer: the whole step 493 -> 435 us.
+  // A tree over the buffer takes a chain of five launches and pays for a caller
+  // who asks more than once between changes of the forest, also without
+  // allocation or in a capture, where no tree can be built.  A caller who
+  // changes and asks once, again and again, gains nothing from it: where
+  // exactly one call came between the last changes, a small first call after a
+  // change scans the buffer instead (a warp per query reads 32 of its points at
+  // a time).  1M 5-D points, 1,009 queries after an update, about 500 points in
+  // the buffer: the whole step 493 -> 435 us.
   std::vector<char> scan(nf, 0);
   if (!counts) {
     int64_t pairs = 0, md[kMaxDim + 1] = {};
@@ -1518,16 +1526,20 @@ static int knn_many(bdl_forest *const *F, int nf, const int32_t *const *q, const
     for (int i = 0; i < nf && pairs <= kScanPairs; ++i) {
       const bdl_forest *f = F[i];
       const int d = f->dim;
-      scan[i] = f->buf_dirty && !f->buf_scanned && f->nbuf > 0 && m[i] > 0 && !stats[d];
+      scan[i] = f->buf_dirty && f->asks_once && f->knn_calls == 0 && f->nbuf > 0 && m[i] > 0 && !stats[d];
       if (!scan[i]) continue;
       const bool skewed = skewed_leaves(f);
       if (by_warp[d][skewed] < 0) by_warp[d][skewed] = knn_by_warp(d, k, md[d], knn_forest_size(mn[d], md[d], nd[d]), skewed);
       scan[i] = by_warp[d][skewed];
     }
-    for (int i = 0; i < nf; ++i)
-      if (scan[i]) F[i]->buf_scanned = true;
   }
   refresh_btrees(F, nf, s, &scan);
+  for (int i = 0; i < nf; ++i) F[i]->in_call = F[i]->in_call || m[i] > 0;
+  for (int i = 0; i < nf; ++i)   // (a forest may take part more than once)
+    if (F[i]->in_call) {
+      F[i]->in_call = false;
+      count_knn_call(F[i]);
+    }
   std::vector<ForestView> views(nf);
   std::vector<KnnCall> calls;
   for (int i = 0; i < nf; ++i) {
@@ -1614,6 +1626,7 @@ static int knn_plan_make(bdl_forest *const *F, int nf, const int32_t *const *q, 
   }
   if (!same_device(F, nf)) return set_error(BDL_EINVAL, "forests on different devices");
   refresh_btrees(F, nf, s);
+  for (int i = 0; i < nf; ++i) F[i]->knn_calls = 2;   // (a plan is launched again and again)
   std::vector<ForestView> views(nf);
   std::vector<KnnCall> calls;
   size_t sort_bytes = 0;

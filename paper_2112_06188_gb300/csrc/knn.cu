@@ -1165,6 +1165,7 @@ extern "C" int bdl_knn_noalloc(bdl_forest *f, const int32_t *q, int64_t m, int k
   int st = knn_scratch_address(f->device, &scratch);
   if (!st) {
     ForestView fv = knn_view(f, false, s);   // never rebuilds (no allocation)
+    count_knn_call(f);
     int32_t *perm = nullptr;
     if (m >= kSortMinQueries) {
       perm = (int32_t *)scratch;
