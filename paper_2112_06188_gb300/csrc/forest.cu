@@ -1472,7 +1472,27 @@ static int reinsert_low(const std::vector<bdl_forest *> &fs, cudaStream_t s) {
   return st;
 }
 
-constexpr int64_t kScanPairs = (int64_t)16 << 20;   // most (query, buffer point) pairs of a scan
+// Whether a call's scans of its stale buffers cost less than building trees
+// over them.  A warp goes through a buffer 32 points at a time, however many
+// warps there are, and every query reads every point.  us more than with a
+// current tree, scan / build (forests of 100,000 points):
+//   2-D: 944 points, 100 queries 4 / 96; 1,478, 4,000 11 / 116; 4,500, 100
+//        47 / 173; 15,400, 100 192 / 160
+//   7-D: 1,337, 4,000 16 / 127; 4,780, 1,000 59 / 169; 15,400, 100 176 / 190
+//   10-D: 2,180, 4,000 73 / 146; 4,800, 1,000 76 / 174; 15,100, 1 258 / 205
+//   16-D: 1,060, 1,000 31 / 135; 1,350, 4,000 180 / 145; 4,500, 100 123 / 204;
+//        4,700, 1,000 173 / 207; 15,300, 100 438 / 273
+// The estimate below gives every one of these to the cheaper side but the last
+// but one (and 7-D at 15,400 points, where they are near each other).
+// pairs: queries times the buffer points each meets, over all forests of the
+// call (measured to 16M); nbuf: the largest buffer.
+constexpr int64_t kScanPairs = (int64_t)16 << 20;
+static bool scan_pays(int dim, int64_t nbuf, int64_t pairs) {
+  const double d = dim / 16.0;
+  const double per_point = std::max(0.012, 0.024 * d), per_mpair = dim <= 7 ? 2 : 28 * d * d * d;
+  const double build = 100 + 0.01 * (double)std::min<int64_t>(nbuf, 7000);
+  return pairs <= kScanPairs && per_point * (double)nbuf + per_mpair * 1e-6 * (double)pairs <= build;
+}
 
 // kNN_L on nf forests: stale buffer trees rebuilt in shared builds, then one
 // k-NN launch per dimension over every forest's queries.
@@ -1510,12 +1530,17 @@ static int knn_many(bdl_forest *const *F, int nf, const int32_t *const *q, const
   // the buffer: the whole step 493 -> 435 us.
   std::vector<char> scan(nf, 0);
   if (!counts) {
-    int64_t pairs = 0, md[kMaxDim + 1] = {};
+    int64_t pairs = 0, most = 0, md[kMaxDim + 1] = {};
+    int dmax = 1;
     double mn[kMaxDim + 1] = {}, nd[kMaxDim + 1] = {};   // the size of forest that a query meets, times md; all points
     bool stats[kMaxDim + 1] = {};
     for (int i = 0; i < nf; ++i) {
       const int d = F[i]->dim;
-      pairs += F[i]->buf_dirty ? m[i] * F[i]->nbuf : 0;
+      if (F[i]->buf_dirty && m[i] > 0) {
+        pairs += m[i] * F[i]->nbuf;
+        most = std::max(most, F[i]->nbuf);
+        dmax = std::max(dmax, d);
+      }
       md[d] += m[i];
       mn[d] += (double)m[i] * (double)F[i]->live;
       nd[d] += (double)F[i]->live;
@@ -1523,7 +1548,8 @@ static int knn_many(bdl_forest *const *F, int nf, const int32_t *const *q, const
     }
     signed char by_warp[kMaxDim + 1][2];   // the rule's answers so far (it takes logarithms)
     memset(by_warp, -1, sizeof(by_warp));
-    for (int i = 0; i < nf && pairs <= kScanPairs; ++i) {
+    const bool pays = scan_pays(dmax, most, pairs);
+    for (int i = 0; i < nf && pays; ++i) {
       const bdl_forest *f = F[i];
       const int d = f->dim;
       scan[i] = f->buf_dirty && f->asks_once && f->knn_calls == 0 && f->nbuf > 0 && m[i] > 0 && !stats[d];

@@ -120,3 +120,17 @@ def test_one_call_per_change_scans():
     assert c.plan()
     c.change()
     assert c.ask()                                         # a plan counts as many calls
+
+
+# on either side of where a scan costs more than the tree: by the buffer's points
+# (12 ns each, 24 in 16 dimensions) and by the pairs of query and point in high dimensions
+@pytest.mark.parametrize("dim,m,nbuf,builds", [(2, 200, 8_000, False), (2, 200, 15_000, True), (7, 4_000, 2_000, False),
+                                               (16, 1_000, 700, False), (16, 4_000, 1_400, True), (10, 40, 14_000, True),
+                                               (3, 6_000, 5_000, True)])
+def test_scan_where_it_pays(dim, m, nbuf, builds):
+    c = Case(dim, m=m, X=16_384, nbuf=nbuf)
+    assert c.ask()
+    for _ in range(2):
+        c.change()
+        assert c.ask() == builds
+    assert c.ask() != builds
