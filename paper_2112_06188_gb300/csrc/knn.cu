@@ -38,9 +38,15 @@ constexpr uint64_t kNone = ~0ull;
 // instance compiled for exactly that launch; every other shape (KnnShape:
 // 64, 128 or 256 threads, 32, 64 or 128 queries per warp) runs the general
 // instance, compiled for blocks of up to 256 threads with the same register
-// budget (256 x 6 = 128 x 12 threads per SM).
+// budget.
 constexpr int kKnnThreads = 128;
 constexpr int kKnnMaxThreads = 256;
+// Resident blocks per SM, which set that budget: 40 registers a thread up to 3
+// dimensions, 64 above, where a record's 40 to 72 words spill with fewer.  us at
+// 40 / 48 / 64 registers: 1M 4-D points, 200K queries, k = 16 2,098 / 1,874 / 1,722;
+// 200,000 5-D points in 100 clusters, 500K, k = 8 2,157 / 1,901 / 1,943; 200,000
+// 6-D ones, 500K, k = 1 1,142 / 1,079 / 999; 20,000 7-D ones, 500K, k = 1 551 / 473 / 459.
+constexpr int knn_blocks(int dim, bool gen) { return dim >= 1 && dim <= 3 ? (gen ? 6 : 12) : (gen ? 4 : 8); }
 
 // The k best candidates of one query, sorted by (d2, id), live in shared
 // memory with a warp's 32 lanes in consecutive words, so that its accesses
@@ -574,7 +580,7 @@ __device__ __forceinline__ void knn_query(const KnnJob &J, const TreeView *trees
 // of its job (in the job's processing order), 32 at a time; every round ends
 // with the warp converged.  GEN false: the default shape (qpw = 32).
 template <int D, bool STATS, bool GEN>
-__global__ void __launch_bounds__(GEN ? kKnnMaxThreads : kKnnThreads, GEN ? 6 : 12)
+__global__ void __launch_bounds__(GEN ? kKnnMaxThreads : kKnnThreads, knn_blocks(D, GEN))
     k_knn(const KnnJob *jobs, const int64_t *job_warp, int njobs, int k, int qpw, unsigned long long *stats) {
   // the warp's job, copied into shared memory: its fields are read where
   // used instead of held in registers through the walk
@@ -598,7 +604,7 @@ __global__ void __launch_bounds__(GEN ? kKnnMaxThreads : kKnnThreads, GEN ? 6 : 
 
 // One forest: its job and tree views travel as kernel parameters.
 template <int D, bool STATS, bool GEN>
-__global__ void __launch_bounds__(GEN ? kKnnMaxThreads : kKnnThreads, GEN ? 6 : 12)
+__global__ void __launch_bounds__(GEN ? kKnnMaxThreads : kKnnThreads, knn_blocks(D, GEN))
     k_knn_one(const __grid_constant__ KnnOne P, int k, int qpw, unsigned long long *stats) {
   if (!GEN) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
