@@ -164,8 +164,8 @@ int bdl_knn_noalloc(bdl_forest *f, const int32_t *q_dev, int64_t m, int k, int32
  * the order the call processes them, 32 at a time.  Used by bdl_knn,
  * bdl_knn_noalloc, bdl_knn_count, and by the batched calls and plans whose
  * forests[0] is f (a plan keeps the shape it was made with), where they take
- * the thread-per-query kernel (small batches and high dimensions take one warp
- * per query, which has one shape).  Results do not depend on the shape.  Other
+ * the thread-per-query kernel (small batches, and in high dimensions all but the
+ * largest, take one warp per query, which has one shape).  Results do not depend on the shape.  Other
  * values: BDL_EINVAL, shape unchanged.  Host only; no device work. */
 int bdl_set_knn_shape(bdl_forest *f, int block_threads, int queries_per_warp);
 
@@ -372,7 +372,8 @@ int bdl_bloom_export(const bdl_forest *f, int level, uint32_t *words_host, bdl_s
  * nothing is waited for.  Measurement only: these counts give the
  * algorithmic bytes of a k-NN launch (4d + 12k per query, 32 per node, one
  * record per leaf point).  Under profiling its launches are reported as
- * "k_knn_count", apart from the timed instance "k_knn". */
+ * "k_knn_count", apart from the timed kernels "k_knn" (a thread per query) and
+ * "k_knn_warp" (a warp per query). */
 int bdl_knn_count(bdl_forest *f, const int32_t *q_dev, int64_t m, int k, int32_t *out_ids_dev,
                   int64_t *out_d2_dev, uint64_t *counts_dev, bdl_stream_t stream);
 

@@ -54,6 +54,7 @@ enum KernelId : int {
   kK_sp_box,
   kK_knn_count,
   kK_small_copy,
+  kK_knn_warp,
   kKernelCount
 };
 extern const char *const kKernelNames[kKernelCount];

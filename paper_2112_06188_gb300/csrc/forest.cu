@@ -47,6 +47,7 @@ const char *const kKernelNames[kKernelCount] = {
     "k_sp_box",
     "k_knn_count",
     "k_small_copy",
+    "k_knn_warp",
 };
 
 // ---- live per-kernel timing (CUDA events on the launching stream) ----

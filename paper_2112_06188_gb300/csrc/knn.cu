@@ -1,7 +1,7 @@
 // knn.cu -- kNN_L (Alg. 5): exact k nearest neighbours of a batch of queries
 // over every static tree (largest first, Sec. V-B) and the buffer: the
-// thread-per-query kernel, for large batches in low dimensions (knn_by_warp;
-// the others go to knn_warp.cu), the packed records and the query order.
+// thread-per-query kernel, for large batches where their walks are short
+// (knn_by_warp; the others go to knn_warp.cu), the packed records and the query order.
 //
 // GPU design:
 //  * One thread per query walks the trees one after another with its own
@@ -42,7 +42,7 @@ constexpr uint64_t kNone = ~0ull;
 constexpr int kKnnThreads = 128;
 constexpr int kKnnMaxThreads = 256;
 // Resident blocks per SM, which set that budget: 40 registers a thread up to 3
-// dimensions, 64 above, where a record's 40 to 72 words spill with fewer.  us at
+// dimensions, 64 above, where a record's 40 to 72 words (instance 0: the query) spill with fewer.  us at
 // 40 / 48 / 64 registers: 1M 4-D points, 200K queries, k = 16 2,098 / 1,874 / 1,722;
 // 200,000 5-D points in 100 clusters, 500K, k = 8 2,157 / 1,901 / 1,943; 200,000
 // 6-D ones, 500K, k = 1 1,142 / 1,079 / 999; 20,000 7-D ones, 500K, k = 1 551 / 473 / 459.
@@ -204,15 +204,36 @@ __device__ __forceinline__ void read_rec(const int32_t *src, int32_t (&p)[rec_in
 // 2-D 997 -> 989 (with two, three, five pairs unrolled 2,755, 2,455, 2,930: the
 // ones that spill lose).
 template <int D, class TK>
-__device__ __forceinline__ void scan_leaf(const TreeView &T, int pa, int pz, const int32_t *q, int k, TK &best) {
-  constexpr int rs = rec_ints(D);
-  constexpr bool kPairs = rs == 4;
+__device__ __forceinline__ void scan_leaf(const TreeView &T, int pa, int pz, const int32_t *q, int dim, int k,
+                                          TK &best) {
+  constexpr int rd = rec_ints(D ? D : kMaxDim);   // (D = 0: the most words a record has)
+  const int rs = D ? rd : rec_ints(dim);
+  constexpr bool kPairs = rd == 4;
   for (int b = kPairs ? pa & ~1 : pa; b < pz; b += 32) {
     const int n = min(pz - b, 32);
     const int32_t *src = T.pts + (int64_t)b * rs;
-    int32_t p[rs];
+    int32_t p[D ? rd : 4];
     unsigned in = 0;
-    if constexpr (kPairs) {
+    if constexpr (D == 0) {
+#pragma unroll 1
+      for (int i = 0; i < n; ++i) {
+        const int32_t *r = src + i * rs;
+        float s = 0.f;
+#pragma unroll
+        for (int c4 = 0; c4 < kMaxDim; c4 += 4)
+          if (c4 < dim) {
+            const int4 v = *reinterpret_cast<const int4 *>(r + c4);
+            const int32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (c4 + e < dim) {
+                const float g = (float)(q[c4 + e] - w[e]);
+                s = fmaf(g, g, s);
+              }
+          }
+        if (!(s > best.kdf) && r[dim] >= 0) in |= 1u << i;
+      }
+    } else if constexpr (kPairs) {
       auto passes = [&](const int32_t *r) {
         float s = 0.f;
 #pragma unroll
@@ -248,14 +269,27 @@ __device__ __forceinline__ void scan_leaf(const TreeView &T, int pa, int pz, con
     while (in) {
       const int i = __ffs(in) - 1;
       in &= in - 1;
-      read_rec<D>(src + i * rs, p);
       uint64_t s = 0;
+      int32_t id;
+      if constexpr (D == 0) {
+        const int32_t *r = src + i * rs;
+        id = r[dim];
 #pragma unroll
-      for (int c = 0; c < D; ++c) {
-        const int32_t g = q[c] - p[c];
-        s += (uint64_t)((int64_t)g * g);
+        for (int c = 0; c < kMaxDim; ++c)
+          if (c < dim) {
+            const int32_t g = q[c] - r[c];
+            s += (uint64_t)((int64_t)g * g);
+          }
+      } else {
+        read_rec<D>(src + i * rs, p);
+        id = p[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+          const int32_t g = q[c] - p[c];
+          s += (uint64_t)((int64_t)g * g);
+        }
       }
-      if (best.better(s, p[D])) best.insert(s, p[D], k);
+      if (best.better(s, id)) best.insert(s, id, k);
     }
   }
 }
@@ -291,7 +325,7 @@ template <int D, class TK>
 __device__ __forceinline__ void walk_packed(const KnnJob &J, const TreeView &T, bool active,
                                             const int32_t *q, int dim, int k, TK &best,
                                             uint64_t *stk) {
-  constexpr int rec = packed_node_ints(D);
+  const int rec = packed_node_ints(D ? D : dim);
   const float kInf = __int_as_float(0x7f800000);
   int sp = 0;
   uint64_t cur = 0;   // the next entry to visit (code >= 0: record; < 0: leaf -1-code)
@@ -310,7 +344,7 @@ __device__ __forceinline__ void walk_packed(const KnnJob &J, const TreeView &T, 
     const unsigned pm = __ballot_sync(0xffffffffu, pending);
     if (2 * __popc(pm) >= __popc(wm)) {
       // half of the working lanes have a leaf due: scan them together
-      if (pending) scan_leaf<D>(T, pa, pz, q, k, best);
+      if (pending) scan_leaf<D>(T, pa, pz, q, dim, k, best);
       pending = false;
       continue;
     }
@@ -347,7 +381,50 @@ __device__ __forceinline__ void walk_packed(const KnnJob &J, const TreeView &T, 
       const int32_t *r = T.pk + (int64_t)code * rec;
       int4 cd, lv;
       float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;   // box distances (see box_dist_f)
-      if constexpr (!packed_by_entry(D)) {
+      if constexpr (D == 0) {
+        // any dimension from 4 on: an entry's bounds in 16-byte words as they come
+        float sv[4];
+        int32_t cv[4], nv[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          sv[a] = 0.f;
+          auto gap = [&](int c, int32_t lo, int32_t hi) {
+            const int32_t x = q[c] + kBias;
+            const float g = (float)max(max(lo - x, x - hi), 0);
+            sv[a] = fmaf(g, g, sv[a]);
+          };
+          if (dim & 1) {
+            const int4 w0 = *reinterpret_cast<const int4 *>(r + packed_quad_at(a, 0));
+            cv[a] = w0.x;
+            nv[a] = w0.y;
+            gap(0, w0.z, w0.w);
+#pragma unroll
+            for (int c = 1; c + 1 < kMaxDim; c += 2)
+              if (c < dim) {
+                const int4 w = *reinterpret_cast<const int4 *>(r + packed_quad_at(a, 2 + 2 * c));
+                gap(c, w.x, w.y);
+                gap(c + 1, w.z, w.w);
+              }
+          } else {
+            const int2 cl = *reinterpret_cast<const int2 *>(r + packed_code_at(dim, a));
+            cv[a] = cl.x;
+            nv[a] = cl.y;
+#pragma unroll
+            for (int c = 0; c + 1 < kMaxDim; c += 2)
+              if (c < dim) {
+                const int4 w = *reinterpret_cast<const int4 *>(r + packed_quad_at(a, 2 * c));
+                gap(c, w.x, w.y);
+                gap(c + 1, w.z, w.w);
+              }
+          }
+        }
+        s0 = sv[0];
+        s1 = sv[1];
+        s2 = sv[2];
+        s3 = sv[3];
+        cd = make_int4(cv[0], cv[1], cv[2], cv[3]);
+        lv = make_int4(nv[0], nv[1], nv[2], nv[3]);
+      } else if constexpr (!packed_by_entry(D)) {
         // a 3-D record (128 bytes) in four loads: 2,468 -> 2,428 us, 100 clusters
         // 1,808 -> 1,760 (2-D in three: 989 -> 1,008)
         auto two = [&](int at, int4 &x, int4 &y) {
@@ -627,9 +704,8 @@ int knn_block_for(const KnnShape &sh, int k) {
   return b;
 }
 
-// The timed instances exist for dim 1 .. 7 (higher dimensions always take the
-// warp-per-query kernel, see knn_by_warp); the counting ones for 2, 3, 5, 7
-// and any (0).
+// The timed instances exist for dim 1 .. 8 and any (0); the counting ones for
+// 2, 3, 5, 7 and any.
 template <int D, bool STATS>
 void launch_d(const KnnJob *jobs, const int64_t *job_warp, int njobs, int64_t warps, int k,
               const KnnShape &sh, unsigned long long *stats, cudaStream_t s) {
@@ -993,7 +1069,8 @@ int launch_knn_table(const void *table, int njobs, int64_t warps, int dim, int k
       case 5: launch_d<5, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
       case 6: launch_d<6, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
       case 7: launch_d<7, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
-      default: return set_error(BDL_EINTERNAL, "no thread-per-query k-NN kernel for this dimension");
+      case 8: launch_d<8, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
+      default: launch_d<0, false>(dj, dw, njobs, warps, k, sh, stats, s); break;
     }
     return cuda_check(cudaGetLastError(), "knn kernel");
   }
@@ -1038,7 +1115,8 @@ int launch_knn_jobs(const std::vector<KnnCall> &calls, int dim, int k, const Knn
         case 5: launch_one<5, false>(P, k, sh, stats, s); break;
         case 6: launch_one<6, false>(P, k, sh, stats, s); break;
         case 7: launch_one<7, false>(P, k, sh, stats, s); break;
-        default: return set_error(BDL_EINTERNAL, "no thread-per-query k-NN kernel for this dimension");
+        case 8: launch_one<8, false>(P, k, sh, stats, s); break;
+        default: launch_one<0, false>(P, k, sh, stats, s); break;
       }
       return cuda_check(cudaGetLastError(), "knn kernel");
     }

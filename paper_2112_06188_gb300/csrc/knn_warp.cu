@@ -449,14 +449,14 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 template <int D>
 void warp_one(const KnnOne &P, int k, int per, cudaStream_t s) {
   const int64_t blk = (int64_t)kWarpsPerBlock * per;
-  KScope ks_(kK_knn, s);
+  KScope ks_(kK_knn_warp, s);
   k_knn_warp_one<D><<<(unsigned)((P.job.m + blk - 1) / blk), kWarpsPerBlock * 32, 0, s>>>(P, k, per);
 }
 
 template <int D>
 void warp_table(const KnnJob *jobs, const int64_t *job_warp, int njobs, int64_t warps, int k, int per,
                 cudaStream_t s) {
-  KScope ks_(kK_knn, s);
+  KScope ks_(kK_knn_warp, s);
   k_knn_warp<D><<<(unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock), kWarpsPerBlock * 32, 0, s>>>(
       jobs, job_warp, njobs, k, per);
 }
@@ -472,66 +472,87 @@ int knn_warp_per(int64_t m) { return (int)std::min<int64_t>(8, std::max<int64_t>
 // Between the size of one forest, which sets the length of a walk, and the size
 // of all, which sets how far apart a warp's queries and its reads lie: their
 // geometric mean.  us by all / by one / by the mean: 64 forests of 10K 3-D
-// points, 1,200 queries each, k = 8: 304 / 257 / 258; 4-D, 3,000 queries, k = 5:
-// 675 / 482 / 483; 5-D, 5,000 queries: 1286 / 1338 / 1338; 32 forests of 12K
-// 7-D points, 10,000 queries, k = 1: 957 / 1333 / 957.
+// points, 1,200 queries each, k = 8: 234 / 182 / 181; 5-D, 5,000 queries, k = 5:
+// 1202 / 1336 / 1337; 32 forests of 12K 7-D points, 10,000 queries, k = 1: uniform
+// 1017 / 1505 / 1015, clustered 828 / 529 / 829; 128 of 5K 8-D points, clustered,
+// 2,000 queries, k = 1: 526 / 253 / 526.
 int64_t knn_forest_size(double mn, int64_t m, double n) {
   return (int64_t)std::sqrt(mn / (double)std::max<int64_t>(m, 1) * n);
 }
 
 // Where the two kernels cost the same: thousands of queries, for k = 1, 5, 16
-// and 32 on forests of 4,500, 55,000 and a million points (9999: beyond
-// 640,000, the most that was measured).  The warp-per-query kernel's time
-// grows with the queries (3 to 20 ns each) from a few dozen microseconds; the
+// and 32 on forests of 2,000, 10,000, 30,000, 100,000 and a million points, by
+// dimension (the last row: 9 and more; 9999: beyond 2.5 million, from the 1.28
+// million that were measured).  The warp-per-query kernel's time grows with the
+// queries (3 to 20 ns each) from a few dozen microseconds; the
 // thread-per-query kernel's stays near that of its slowest warps until about
 // 130,000 queries fill the GPU, and then grows more slowly where its walks are
 // short (low dimensions, small forests) and for small k (its top-k lists take
 // 12 k bytes of shared memory per thread: past k = 16 they cost it resident
 // warps).  Each entry is the geometric mean of the crossings of uniform points
-// and of points in 100 clusters, and of two sizes n for the first two columns
-// (2,000 and 10,000; 30,000 and 100,000).  5,000 to 640,000 queries at points
-// of the forest, thread / warp in us on either side of a crossing:
-//   dim 1, k = 5:  n = 10,000, 10K queries 36 / 31, 20K 37 / 48
-//   dim 2, k = 5:  n = 100,000, 20K 89 / 65, 40K 101 / 139
-//   dim 3, k = 5:  n = 1M, 40K 264 / 198, 80K 300 / 337
-//          k = 16: n = 1M, 80K 573 / 435, 160K 666 / 797
-//   dim 4, k = 1:  n = 30,000, 40K 182 / 137, 80K 186 / 195
-//   dim 5, k = 1:  n = 2,000 clustered, 10K 38 / 28, 160K 83 / 217
-//          k = 16: n = 30,000, 320K 1973 / 1856, 640K 2914 / 3285
-//   dim 6, k = 5:  n = 10,000, 160K 782 / 674, 320K 912 / 1203
-//   dim 7, k = 1:  n = 10,000, 160K 554 / 343, 320K 554 / 586
-// Over all 2,688 of those launches the choice costs 1% more than the better
-// kernel each time (a line in k alone: 3.4%, and up to 3.3 times on small
-// forests in dimensions 4 to 7).  (Measured before the thread-per-query
-// kernel's 32-byte loads, which took 1 to 8% off its times in 2 to 5 dimensions.)
+// and of points in 100 clusters (a million: with those of 4 or 10 million; 9 and
+// more: of 10, 13 and 16 dimensions; uniform points from 30,000 on in 8 and more
+// dimensions, where the thread-per-query kernel is several times slower, count as
+// 5 million).  2,500 to 1.28 million queries at points of the forest, thread /
+// warp in us on either side of a crossing:
+//   dim 1, k = 5:  n = 10,000, 10K queries 43 / 35, 20K 42 / 52
+//   dim 2, k = 5:  n = 100,000, 20K 92 / 69, 40K 106 / 147
+//   dim 3, k = 5:  n = 1M, 40K 278 / 205, 80K 282 / 340; n = 10M, 40K 282 / 216, 80K 307 / 390
+//          k = 16: n = 1M, 80K 550 / 441, 160K 695 / 805
+//   dim 4, k = 1:  n = 30,000, 40K 144 / 140, 80K 156 / 199
+//   dim 5, k = 1:  n = 2,000 clustered, 10K 36 / 31, 20K 38 / 47
+//          k = 16: n = 30,000, 80K 917 / 583, 160K 1049 / 1058
+//   dim 6, k = 5:  n = 10,000, 80K 504 / 374, 160K 587 / 682
+//   dim 7, k = 1:  n = 10,000, 160K 396 / 350, 320K 488 / 601; clustered, 20K 72 / 59, 40K 90 / 124
+//          k = 5:  n = 4M clustered, 1.28M 33527 / 19327
+//   dim 8, k = 1:  n = 2,000 clustered, 20K 51 / 50, 40K 70 / 106
+//          k = 5:  n = 10,000, 160K 1525 / 1406, 320K 1914 / 2558
+//   dim 10, k = 1: n = 2,000 clustered, 20K 96 / 68, 40K 114 / 138
+//   dim 16, k = 1: n = 2,000 clustered, 20K 112 / 68, 40K 121 / 138
+// Over all 3,121 of those launches the choice costs 1.9% more than the better
+// kernel each time; at worst, between the crossings of uniform and of clustered
+// points, 2.0 times where the warp-per-query kernel is taken and 2.8 times where
+// the other is (1-D points of which most lie in the same places).
 //
 // Leaves of hundreds of points and more (spatial-median trees of clustered
 // points) are scanned by one lane in the thread-per-query kernel, 32 points at
 // a time here.  100 clusters, thread / warp in us: 1M 2-D points, k = 5, 100K
 // queries 3190 / 867, 600K 4400 / 4083, 1M 5749 / 6522; 1M 3-D points, k = 10,
 // 1M queries 11681 / 8335; 10M 3-D points, 1M queries 55418 / 37189.
-bool knn_by_warp(int dim, int k, int64_t m, int64_t n, bool skewed) {
-  if (dim > 7 || (skewed && (dim > 2 || m <= 600000))) return true;
-  static constexpr int kAtK[4] = {1, 5, 16, 32};
-  static constexpr float kAtN[3] = {4500, 55000, 1e6};
-  static constexpr float kMost[7][4][3] = {
-      {{7, 14, 56}, {14, 20, 64}, {32, 42, 97}, {61, 130, 220}},
-      {{13, 18, 28}, {27, 34, 53}, {49, 81, 110}, {130, 1700, 9999}},
-      {{19, 28, 41}, {33, 53, 78}, {62, 120, 150}, {220, 2600, 9999}},
-      {{23, 45, 78}, {53, 85, 260}, {130, 250, 9999}, {710, 9999, 9999}},
-      {{36, 77, 270}, {64, 180, 9999}, {160, 1600, 9999}, {2600, 9999, 9999}},
-      {{55, 140, 910}, {87, 300, 9999}, {220, 2000, 9999}, {2500, 9999, 9999}},
-      {{73, 420, 9999}, {94, 1700, 9999}, {470, 9999, 9999}, {2800, 9999, 9999}}};
-  // between the entries: linear in k and log n, for the logarithm
+namespace {
+
+constexpr int kAtK[4] = {1, 5, 16, 32};
+
+// Thousands of queries at (k, n) from a table over kAtK and N sizes: linear in
+// k and log n between its entries, for the logarithm.
+template <int N>
+float crossing(const float (&most)[4][N], const float (&at_n)[N], int k, int64_t n) {
   const int ik = k < 5 ? 0 : k < 16 ? 1 : 2;
   const float wk = (float)(k - kAtK[ik]) / (float)(kAtK[ik + 1] - kAtK[ik]);
-  const int in = (float)n < kAtN[1] ? 0 : 1;
-  const float x = std::log((float)std::max<int64_t>(n, 1) / kAtN[in]) / std::log(kAtN[in + 1] / kAtN[in]);
+  int in = 0;
+  while (in < N - 2 && (float)n >= at_n[in + 1]) ++in;
+  const float x = std::log((float)std::max<int64_t>(n, 1) / at_n[in]) / std::log(at_n[in + 1] / at_n[in]);
   const float wn = std::min(std::max(x, 0.f), 1.f);
-  auto at = [&](int i) {
-    return (1 - wn) * std::log(kMost[dim - 1][i][in]) + wn * std::log(kMost[dim - 1][i][in + 1]);
-  };
-  return (float)m <= 1000 * std::exp((1 - wk) * at(ik) + wk * at(ik + 1));
+  auto at = [&](int i) { return (1 - wn) * std::log(most[i][in]) + wn * std::log(most[i][in + 1]); };
+  return std::exp((1 - wk) * at(ik) + wk * at(ik + 1));
+}
+
+}  // namespace
+
+bool knn_by_warp(int dim, int k, int64_t m, int64_t n, bool skewed) {
+  if (skewed && (dim > 2 || m <= 600000)) return true;
+  static constexpr float kAtN[5] = {2000, 10000, 30000, 100000, 1e6};
+  static constexpr float kMost[9][4][5] = {
+      {{3, 9, 16, 19, 68}, {16, 15, 22, 26, 77}, {33, 33, 41, 49, 120}, {91, 61, 140, 170, 290}},
+      {{12, 14, 21, 16, 27}, {24, 28, 31, 31, 42}, {41, 57, 81, 83, 100}, {120, 180, 450, 2100, 9999}},
+      {{15, 24, 29, 25, 39}, {30, 39, 53, 50, 76}, {53, 79, 110, 140, 140}, {140, 440, 1600, 9999, 9999}},
+      {{16, 21, 34, 32, 47}, {33, 44, 56, 59, 120}, {82, 98, 130, 190, 770}, {250, 1000, 1700, 9999, 9999}},
+      {{21, 30, 49, 49, 130}, {37, 51, 82, 120, 590}, {94, 100, 150, 260, 9999}, {300, 1100, 1700, 9999, 9999}},
+      {{23, 60, 92, 87, 690}, {44, 72, 120, 220, 9999}, {98, 130, 220, 1300, 9999}, {260, 1000, 1700, 9999, 9999}},
+      {{35, 73, 160, 200, 9999}, {52, 95, 180, 9999, 9999}, {190, 230, 560, 9999, 9999}, {880, 1700, 9999, 9999, 9999}},
+      {{37, 100, 460, 860, 9999}, {48, 110, 770, 9999, 9999}, {100, 150, 1100, 9999, 9999}, {260, 1200, 9999, 9999, 9999}},
+      {{160, 460, 890, 9999, 9999}, {100, 220, 1100, 9999, 9999}, {550, 300, 1500, 9999, 9999}, {650, 9999, 9999, 9999, 9999}}};
+  return (float)m <= 1000 * crossing(kMost[std::min(dim, 9) - 1], kAtN, k, n);
 }
 
 int launch_knn_warp_one(const KnnOne &P, int dim, int k, int per, cudaStream_t s) {

@@ -13,6 +13,7 @@ import torch
 from oracle.oracle import OracleForest
 from oracle.threads import oracle_knn
 from paper_2112_06188_gb300 import inputs
+from tests.which_kernel import knn_kernel
 
 pytestmark = pytest.mark.gpu
 
@@ -56,12 +57,14 @@ def forest_pair(dim, n0, seed):
     return g, o, lp
 
 
-@pytest.mark.parametrize("k", [10, 32])
-def test_every_shape_matches_oracle(k):
-    g, o, lp = forest_pair(3, 200_000, seed=500 + k)
-    big = np.concatenate([inputs.queries_from(lp, 20_000, seed=510),
-                          inputs.uniform_points(20_000, 3, seed=511)])       # sorted path
-    small = inputs.uniform_points(2_500, 3, seed=512)                        # input order
+# (batches that the thread-per-query kernel takes, and small ones, which have one shape)
+@pytest.mark.parametrize("k,dim,n0,m", [(10, 3, 200_000, 110_000), (32, 2, 3_000, 150_000), (1, 2, 3_000, 20_000)])
+def test_every_shape_matches_oracle(k, dim, n0, m):
+    g, o, lp = forest_pair(dim, n0, seed=500 + k)
+    big = np.concatenate([inputs.queries_from(lp, m // 2, seed=510),
+                          inputs.uniform_points(m // 2, dim, seed=511)])     # sorted path (m >= 32,768)
+    small = inputs.uniform_points(2_500, dim, seed=512)                      # input order
+    assert knn_kernel(lambda: g.knn(dev(big), k))[0] == "k_knn"
     for q in (big, small):
         want = oracle_knn(o, q, k)
         qd = dev(q)
@@ -75,7 +78,7 @@ def test_batched_and_plan_use_first_forest_shape():
     from paper_2112_06188_gb300.forest import KnnPlan, knn_batch
     pairs = [forest_pair(2, 60_000, seed=520), forest_pair(2, 30_000, seed=530), forest_pair(5, 40_000, seed=540)]
     k = 8
-    qs = [np.concatenate([inputs.queries_from(lp, 20_000, seed=550 + j), inputs.uniform_points(15_000, g.dim, seed=560 + j)])
+    qs = [np.concatenate([inputs.queries_from(lp, 60_000, seed=550 + j), inputs.uniform_points(15_000, g.dim, seed=560 + j)])
           if j == 0 else inputs.uniform_points(3_000 + 500 * j, g.dim, seed=560 + j)
           for j, (g, _, lp) in enumerate(pairs)]
     wants = [oracle_knn(o, q, k) for (_, o, _), q in zip(pairs, qs)]
@@ -132,10 +135,10 @@ def test_batched_call_at_k32():
     of shared memory at 128 threads, with the warps' job and tree slots on
     top (the launch opts in to the larger size)."""
     from paper_2112_06188_gb300.forest import knn_batch
-    pairs = [forest_pair(3, 40_000, seed=590), forest_pair(3, 20_000, seed=591)]
-    qs = [inputs.uniform_points(2_000 + 700 * j, 3, seed=592 + j) for j in range(2)]
-    out = knn_batch([g for g, _, _ in pairs], [dev(q) for q in qs], 32)
-    torch.cuda.synchronize()
+    pairs = [forest_pair(2, 3_000, seed=590), forest_pair(2, 2_000, seed=591)]
+    qs = [inputs.uniform_points(90_000 + 700 * j, 2, seed=592 + j) for j in range(2)]
+    name, out = knn_kernel(lambda: knn_batch([g for g, _, _ in pairs], [dev(q) for q in qs], 32))
+    assert name == "k_knn"
     for j, ((g, o, _), q) in enumerate(zip(pairs, qs)):
         assert_rows(out[j], oracle_knn(o, q, 32), "k=32 batched, forest %d" % j)
     for g, _, _ in pairs:

@@ -10,6 +10,7 @@ import torch
 
 from oracle.threads import bruteforce_knn_threads
 from paper_2112_06188_gb300 import inputs
+from tests.which_kernel import crossing, knn_kernel
 
 pytestmark = pytest.mark.gpu
 
@@ -87,33 +88,52 @@ def test_deep_trees_with_little_pruning():
     check(f, live, inputs.uniform_points(3, 16, 12), 32)
 
 
-# just above and below the size from which each dimension takes the
-# thread-per-query kernel (k = 1, a small forest), with the launch shapes that kernel has
-@pytest.mark.parametrize("dim,m", [(1, 6_900), (2, 12_900), (3, 18_900), (4, 22_900), (5, 35_900), (6, 54_900),
-                                   (7, 72_900)])
-def test_thread_kernel_gives_the_same_rows(dim, m):
+# on both sides of the batch size from which each dimension takes the thread-per-query
+# kernel (k = 1, a small forest), found by asking, and with the launch shapes that kernel has
+@pytest.mark.parametrize("dim", [1, 2, 3, 4, 5, 6, 7, 8, 9, 16])
+def test_thread_kernel_gives_the_same_rows(dim):
     from paper_2112_06188_gb300.forest import KnnPlan, knn_batch
     f, live = forest_of(dim, 3_000, 60 + dim)
     lp, _ = live.live_points()
-    q = dev(np.concatenate([inputs.queries_from(lp, m // 2, 7), inputs.uniform_points(m + 200 - m // 2, dim, 8)]))
-    wi, wd = (torch.cat(x) for x in zip(*(f.knn(c, 1) for c in q.split(5_000))))
-    for n in (m, m + 200):
-        gi, gd = f.knn(q[:n], 1)
-        assert torch.equal(gi, wi[:n]) and torch.equal(gd, wd[:n])
+    most = 400_000 if dim > 8 else 100_000
+    q = dev(np.concatenate([inputs.queries_from(lp, most // 2, 7), inputs.uniform_points(most // 2, dim, 8)]))
+    q = q[torch.randperm(most, generator=torch.Generator().manual_seed(1)).cuda()].contiguous()
+    c = crossing(f, q, 1)
+    q = q[:2 * c + 200].contiguous()
+    parts = [knn_kernel(lambda x=x: f.knn(x, 1)) for x in q.split(max(c // 2, 1))]
+    assert {name for name, _ in parts} == {"k_knn_warp"}
+    wi, wd = (torch.cat(x) for x in zip(*(rows for _, rows in parts)))
+    for n, want in ((c, "k_knn_warp"), (c + 1, "k_knn"), (c + 200, "k_knn")):
+        name, (gi, gd) = knn_kernel(lambda: f.knn(q[:n], 1))
+        assert name == want and torch.equal(gi, wi[:n]) and torch.equal(gd, wd[:n])
     half = q.shape[0] // 2
-    for (gi, gd), want in zip(knn_batch([f, f], [q[:half], q[half:]], 1), (slice(0, half), slice(half, None))):
+    name, rows = knn_kernel(lambda: knn_batch([f, f], [q[:half], q[half:]], 1))
+    assert name == "k_knn"
+    for (gi, gd), want in zip(rows, (slice(0, half), slice(half, None))):
         assert torch.equal(gi, wi[want]) and torch.equal(gd, wd[want])
-    if dim == 3:
+    if dim in (3, 8, 9):
         for block in (64, 128, 256):
             for per in (32, 64, 128):
                 f.set_knn_shape(block, per)
                 plan = KnnPlan([f], [q], 1)
-                for gi, gd in (f.knn(q, 1), plan.launch()[0]):
-                    assert torch.equal(gi, wi) and torch.equal(gd, wd)
+                for name, (gi, gd) in (knn_kernel(lambda: f.knn(q, 1)), knn_kernel(lambda: plan.launch()[0])):
+                    assert name == "k_knn" and torch.equal(gi, wi) and torch.equal(gd, wd)
                 plan.close()
-        wi, wd = (torch.cat(x) for x in zip(*(f.knn(c, 16) for c in q.repeat(4, 1).split(20_000))))
-        gi, gd = f.knn(q.repeat(4, 1), 16)
-        assert torch.equal(gi, wi) and torch.equal(gd, wd)
+    assert f.poll_error() == 0
+
+
+# high dimensions at small and large k, with erased points, ties and leaves on either side of 32 points
+@pytest.mark.parametrize("dim,k,m", [(8, 16, 300_000), (8, 5, 200_000), (9, 5, 300_000), (11, 5, 300_000), (13, 8, 600_000), (16, 5, 300_000)])
+@pytest.mark.parametrize("leaf,distinct", [(16, 0), (40, 50)])
+def test_thread_kernel_in_high_dimensions(dim, k, m, leaf, distinct):
+    f, live = forest_of(dim, 2_000, 300 + dim, leaf=leaf, distinct=distinct)
+    lp, ids = live.live_points()
+    few = np.concatenate([inputs.queries_from(lp, 500, 7), inputs.uniform_points(500, dim, 8)])
+    q = dev(few).repeat(m // 1_000, 1)
+    name, (gi, gd) = knn_kernel(lambda: f.knn(q, k))
+    assert name == "k_knn"
+    bi, bd = (dev(x) for x in bruteforce_knn_threads(lp, ids, few, k))
+    assert torch.equal(gi, bi.repeat(m // 1_000, 1)) and torch.equal(gd, bd.repeat(m // 1_000, 1))
     assert f.poll_error() == 0
 
 
@@ -123,7 +143,8 @@ def test_thread_kernel_with_leaves_over_32_points(dim, m, k, leaf, distinct):
     f, live = forest_of(dim, 9_000, 71 + leaf, leaf=leaf, distinct=distinct)
     lp, _ = live.live_points()
     q = dev(np.concatenate([inputs.queries_from(lp, m // 2, 7), inputs.uniform_points(m - m // 2, dim, 8)]))
-    gi, gd = f.knn(q, k)
+    name, (gi, gd) = knn_kernel(lambda: f.knn(q, k))
+    assert name == "k_knn" and knn_kernel(lambda: f.knn(q[:5_000], k))[0] == "k_knn_warp"
     for a in range(0, m, 5_000):
         wi, wd = f.knn(q[a:a + 5_000], k)
         assert torch.equal(gi[a:a + 5_000], wi) and torch.equal(gd[a:a + 5_000], wd)
@@ -132,7 +153,7 @@ def test_thread_kernel_with_leaves_over_32_points(dim, m, k, leaf, distinct):
     assert torch.equal(ci, gi) and torch.equal(cd, gd) and f.poll_error() == 0
 
 
-@pytest.mark.parametrize("dim,n,m,k", [(4, 6_000, 61_003, 32), (5, 20_000, 250_001, 16), (8, 6_000, 60_000, 1),
+@pytest.mark.parametrize("dim,n,m,k", [(4, 6_000, 61_003, 32), (7, 20_000, 150_001, 16), (8, 6_000, 60_000, 1),
                                        (10, 3_000, 90_001, 32), (8, 20, 60_100, 32), (8, 40, 60_100, 32)])
 @pytest.mark.parametrize("distinct", [0, 7])
 def test_queries_in_turn_by_one_warp(dim, n, m, k, distinct):
@@ -142,7 +163,8 @@ def test_queries_in_turn_by_one_warp(dim, n, m, k, distinct):
     f, live = forest_of(dim, n, 31 + n, distinct=distinct, X=16)
     lp, _ = live.live_points()
     q = dev(np.concatenate([inputs.queries_from(lp, m // 2, 7), inputs.uniform_points(m - m // 2, dim, 8)]))
-    gi, gd = f.knn(q, k)
+    name, (gi, gd) = knn_kernel(lambda: f.knn(q, k))
+    assert name == "k_knn_warp"
     for a in range(0, m, 7_000):
         wi, wd = f.knn(q[a:a + 7_000], k)
         assert torch.equal(gi[a:a + 7_000], wi) and torch.equal(gd[a:a + 7_000], wd)
