@@ -516,9 +516,14 @@ int64_t knn_forest_size(double mn, int64_t m, double n) {
 //
 // Leaves of hundreds of points and more (spatial-median trees of clustered
 // points) are scanned by one lane in the thread-per-query kernel, 32 points at
-// a time here.  100 clusters, thread / warp in us: 1M 2-D points, k = 5, 100K
-// queries 3190 / 867, 600K 4400 / 4083, 1M 5749 / 6522; 1M 3-D points, k = 10,
-// 1M queries 11681 / 8335; 10M 3-D points, 1M queries 55418 / 37189.
+// a time here.  The second table, for 10,000, 100,000, 1 and 10 million points,
+// stands where it is the higher one; it hardly depends on the dimension (1 to 5
+// measured).  100 clusters, thread / warp in us:
+//   dim 2, k = 1:  n = 100,000, 40K queries 224 / 166, 160K 287 / 403
+//          k = 5:  n = 1M, 160K 2580 / 1255, 640K 3057 / 3947; n = 10M, 640K 14439 / 11371, 1.28M 17280 / 19153
+//   dim 3, k = 5:  n = 100,000, 80K 436 / 303, 160K 464 / 542
+//          k = 1:  n = 10M, 640K 18455 / 13107, 1.28M 23134 / 21732
+// Over 796 such launches from 10,000 points on: 1.3% more than the better kernel.
 namespace {
 
 constexpr int kAtK[4] = {1, 5, 16, 32};
@@ -540,7 +545,6 @@ float crossing(const float (&most)[4][N], const float (&at_n)[N], int k, int64_t
 }  // namespace
 
 bool knn_by_warp(int dim, int k, int64_t m, int64_t n, bool skewed) {
-  if (skewed && (dim > 2 || m <= 600000)) return true;
   static constexpr float kAtN[5] = {2000, 10000, 30000, 100000, 1e6};
   static constexpr float kMost[9][4][5] = {
       {{3, 9, 16, 19, 68}, {16, 15, 22, 26, 77}, {33, 33, 41, 49, 120}, {91, 61, 140, 170, 290}},
@@ -552,7 +556,12 @@ bool knn_by_warp(int dim, int k, int64_t m, int64_t n, bool skewed) {
       {{35, 73, 160, 200, 9999}, {52, 95, 180, 9999, 9999}, {190, 230, 560, 9999, 9999}, {880, 1700, 9999, 9999, 9999}},
       {{37, 100, 460, 860, 9999}, {48, 110, 770, 9999, 9999}, {100, 150, 1100, 9999, 9999}, {260, 1200, 9999, 9999, 9999}},
       {{160, 460, 890, 9999, 9999}, {100, 220, 1100, 9999, 9999}, {550, 300, 1500, 9999, 9999}, {650, 9999, 9999, 9999, 9999}}};
-  return (float)m <= 1000 * crossing(kMost[std::min(dim, 9) - 1], kAtN, k, n);
+  static constexpr float kAtSkewedN[4] = {1e4, 1e5, 1e6, 1e7};
+  static constexpr float kMostSkewed[4][4] = {
+      {26, 65, 300, 2000}, {40, 130, 500, 3000}, {110, 270, 900, 9999}, {450, 9999, 9999, 9999}};
+  float most = crossing(kMost[std::min(dim, 9) - 1], kAtN, k, n);
+  if (skewed) most = std::max(most, crossing(kMostSkewed, kAtSkewedN, k, n));
+  return (float)m <= 1000 * most;
 }
 
 int launch_knn_warp_one(const KnnOne &P, int dim, int k, int per, cudaStream_t s) {

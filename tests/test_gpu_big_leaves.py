@@ -1,14 +1,16 @@
 """Spatial-median trees whose leaves hold far more points than a warp has
 lanes (the rule bounds the depth, not the leaves): erases that find their ids
-in such leaves, the leaves' boxes, and k-NN on both sides of the batch size
-from which well-filled trees take another kernel, all against the oracle."""
+in such leaves and the leaves' boxes against the oracle, and k-NN by either
+kernel (the size of the leaves moves the choice) against the other and, for a
+sample, brute force."""
 import numpy as np
 import pytest
 import torch
 
 from oracle.oracle import OracleForest
-from oracle.threads import oracle_knn
+from oracle.threads import bruteforce_knn_threads, oracle_knn
 from paper_2112_06188_gb300 import inputs
+from tests.which_kernel import knn_kernel
 
 pytestmark = pytest.mark.gpu
 
@@ -54,15 +56,24 @@ def test_erase_and_boxes(dim, clumps, spread):
         assert np.array_equal(gi.cpu().numpy(), oi) and np.array_equal(gd.cpu().numpy(), od)
 
 
-@pytest.mark.parametrize("clumps", [5, 20_000])
-def test_knn_of_skewed_and_even_leaves(clumps):
+@pytest.mark.parametrize("clumps,m", [(5, 150_000), (20_000, 60_000)])
+def test_knn_of_skewed_and_even_leaves(clumps, m):
     from paper_2112_06188_gb300.forest import Forest
     rng = np.random.default_rng(clumps)
     centre = rng.integers(0, inputs.GRID, size=(clumps, 2))
+    pts = centre[rng.integers(0, clumps, size=20_000)].astype(np.int32)
     f = Forest(2, split="spatial")
-    f.insert(dev(centre[rng.integers(0, clumps, size=20_000)].astype(np.int32)))
+    f.insert(dev(pts))
     torch.cuda.synchronize()
-    q = dev(inputs.uniform_points(40_000, 2, 9))
-    gi, gd = f.knn(q, 3)
-    wi, wd = (torch.cat(x) for x in zip(*(f.knn(c, 3) for c in q.split(4_000))))
+    q = inputs.uniform_points(m, 2, 9)
+    name, (gi, gd) = knn_kernel(lambda: f.knn(dev(q), 3))
+    assert name == "k_knn"
+    parts = [knn_kernel(lambda c=c: f.knn(c, 3)) for c in dev(q).split(4_000)]
+    assert {name for name, _ in parts} == {"k_knn_warp"}
+    wi, wd = (torch.cat(x) for x in zip(*(rows for _, rows in parts)))
     assert torch.equal(gi, wi) and torch.equal(gd, wd)
+    bi, bd = bruteforce_knn_threads(pts, np.arange(20_000, dtype=np.int32), q[:300], 3)
+    assert np.array_equal(gi[:300].cpu().numpy(), bi) and np.array_equal(gd[:300].cpu().numpy(), bd)
+    # leaves of thousands of points move the choice: the same batch on even leaves goes to the other kernel
+    name, _ = knn_kernel(lambda: f.knn(dev(q[:35_000]), 3))
+    assert name == ("k_knn_warp" if clumps == 5 else "k_knn")
