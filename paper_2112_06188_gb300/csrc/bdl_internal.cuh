@@ -265,27 +265,6 @@ __host__ __device__ inline int64_t quad_count(int H) {   // (4^H - 1) / 3 nodes 
   return (((int64_t)1 << (2 * H)) - 1) / 3;
 }
 
-// Position of node (level u, index i) in the vEB order of a complete 4-ary
-// tree of H levels, split into top and bottom levels as veb_slot does.
-__host__ __device__ inline int64_t veb4_slot(int H, int u, int64_t i) {
-  int64_t off = 0;
-  while (H > 1) {
-    const int Hb = veb_bottom(H);
-    const int Ht = H - Hb;
-    if (u < Ht) {
-      H = Ht;
-    } else {
-      const int uu = u - Ht;
-      const int64_t j = i >> (2 * uu);
-      off += quad_count(Ht) + j * quad_count(Hb);
-      i &= ((int64_t)1 << (2 * uu)) - 1;
-      u = uu;
-      H = Hb;
-    }
-  }
-  return off;
-}
-
 // Records of a tree with h internal levels.
 __host__ __device__ inline int64_t packed_nrec(int h) {
   if (h <= 0) return 0;
@@ -296,20 +275,12 @@ __host__ __device__ inline int64_t packed_nrec(int h) {
 // Levels from the record of a node at depth t down to its entries.
 __host__ __device__ inline int packed_step(int h, int t) { return ((h & 1) && t == 0) ? 1 : 2; }
 
-// Slot of the record of the node at depth t, index i.  Even h: the records
-// form one complete 4-ary tree, in vEB order.  Odd h: the root's record, then
-// the 4-ary trees under its two children, each in vEB order.
-__host__ __device__ inline int64_t packed_slot(int h, int t, int64_t i) {
-  if (!(h & 1)) return veb4_slot(h / 2, t / 2, i);
-  if (t == 0) return 0;
-  const int64_t sub = i >> (t - 1), il = i & (((int64_t)1 << (t - 1)) - 1);
-  return 1 + sub * quad_count((h - 1) / 2) + veb4_slot((h - 1) / 2, (t - 1) / 2, il);
-}
-
-// veb4_slot and packed_slot in 32-bit arithmetic.  (4^H - 1) / 3 is every
-// other bit of 2 H.
+// The same count in 32-bit arithmetic (H < 16), for the kernels: every other bit
+// of 2 H.
 __host__ __device__ inline int quad_count32(int H) { return (int)(0x55555555u & ((1u << (2 * H)) - 1)); }
 
+// Position of node (level u, index i) in the vEB order of a complete 4-ary
+// tree of H levels, split into top and bottom levels as veb_slot does.
 __host__ __device__ inline int veb4_slot32(int H, int u, int i) {
   int off = 0;
   while (H > 1) {
@@ -327,6 +298,9 @@ __host__ __device__ inline int veb4_slot32(int H, int u, int i) {
   return off;
 }
 
+// Slot of the record of the node at depth t, index i.  Even h: the records
+// form one complete 4-ary tree, in vEB order.  Odd h: the root's record, then
+// the 4-ary trees under its two children, each in vEB order.
 __host__ __device__ inline int packed_slot32(int h, int t, int i) {
   if (!(h & 1)) return veb4_slot32(h / 2, t / 2, i);
   if (t == 0) return 0;
@@ -334,8 +308,8 @@ __host__ __device__ inline int packed_slot32(int h, int t, int i) {
   return 1 + sub * quad_count32((h - 1) / 2) + veb4_slot32((h - 1) / 2, (t - 1) / 2, il);
 }
 
-// packed_record_of in 32-bit arithmetic: level u of the (1 + odd) 4-ary trees
-// starts after (1 + odd) (4^u - 1) / 3 records.
+// The g-th record in level order: depth t and index i of its node.  Level u of
+// the (1 + odd) 4-ary trees starts after (1 + odd) (4^u - 1) / 3 records.
 __host__ __device__ inline void packed_record_of32(int h, int g, int &t, int &i) {
   const int odd = h & 1;
   if (odd && g == 0) {
@@ -349,24 +323,6 @@ __host__ __device__ inline void packed_record_of32(int h, int g, int &t, int &i)
   i = y - (quad_count32(u) << odd);
 }
 
-// The g-th record in level order: depth t and index i of its node.
-__host__ __device__ inline void packed_record_of(int h, int64_t g, int &t, int64_t &i) {
-  const int odd = h & 1;
-  if (odd && g == 0) {
-    t = 0;
-    i = 0;
-    return;
-  }
-  int64_t y = odd ? g - 1 : g;
-  int u = 0;
-  while (y >= ((int64_t)(1 + odd) << (2 * u))) {   // 2 * 4^u (odd h) or 4^u nodes on level u
-    y -= (int64_t)(1 + odd) << (2 * u);
-    ++u;
-  }
-  t = 2 * u + odd;
-  i = y;
-}
-
 struct TreeView {          // one static tree, device pointers
   int32_t *pts;            // [size][rec_ints(dim)]: coordinates, id (erased: id | kTomb)
   const Node *node;        // [nnodes]
@@ -374,7 +330,7 @@ struct TreeView {          // one static tree, device pointers
   int32_t *live;           // [nnodes]
   const int32_t *leaf_off; // [2^h + 1]
   const uint32_t *bloom;   // [blocks * 8] or nullptr
-  int32_t *pk;             // packed k-NN node records (packed_slot order)
+  int32_t *pk;             // packed k-NN node records (packed_slot32 order)
   int64_t size;
   int64_t nnodes;
   int64_t bloom_blocks;
@@ -604,10 +560,9 @@ bool skewed_leaves(const bdl_forest *f);
 ForestView forest_view(const bdl_forest *f);
 // A k-NN call on the forest, for the choice of whether to build the buffer's tree.
 inline void count_knn_call(bdl_forest *f) { f->knn_calls = std::min(f->knn_calls + 1, 2); }
-// The view k-NN uses: the static trees plus the buffer's kd-tree.  With
-// build = true a stale buffer tree is rebuilt first (this allocates); with
-// build = false a stale one is left alone and the buffer is scanned instead.
-ForestView knn_view(bdl_forest *f, bool build, cudaStream_t s);
+// The view k-NN uses: the static trees plus the buffer's kd-tree, or, where
+// that is stale, the buffer's points to be scanned.
+ForestView knn_view(bdl_forest *f);
 // BDL_DEBUG_CHECK: wait for the call's kernels and report a bounds-check hit.
 int finish_call(bdl_forest *f, cudaStream_t s, int status);
 constexpr int64_t kSortMinQueries = 1 << 15;   // smaller batches run in input order ...

@@ -261,7 +261,7 @@ __device__ void level_hist(const LvParams &P, int64_t b, uint32_t (*h)[kHistBins
 __device__ void hist_rank_bin(const uint32_t *h, uint32_t r, int *out_bin, uint32_t *out_below,
                               uint32_t *out_cnt) {
   __shared__ uint32_t wsum[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int per = kHistBins / blockDim.x;   // 4
   uint32_t v[4] = {0, 0, 0, 0}, sum = 0;
   if (per == 4) {
@@ -278,7 +278,6 @@ __device__ void hist_rank_bin(const uint32_t *h, uint32_t r, int *out_bin, uint3
   __syncthreads();
   uint32_t base = 0;
   for (int w = 0; w < warp; ++w) base += wsum[w];
-  (void)nwarps;
   uint32_t below = base + inc - sum;
   if (below < r && r <= below + sum) {
     for (int j = 0; j < 4; ++j) {
@@ -613,13 +612,13 @@ struct LevelsParams {
   int64_t pool_total;               // pool entries
   const LevelWork *lv;              // [nlev]
   int nlev;
-  unsigned *bar;                    // grid barrier state (2 words, zeroed)
+  unsigned *bar;                    // grid barrier's count of arrivals (zeroed)
   unsigned long long *err;          // where a barrier that gave up is recorded
 };
 
 __global__ void __launch_bounds__(kCoopThreads, 2) k_build_levels(const LevelsParams B) {
-  // shared buffers for the phases' big arrays (histograms, candidate keys,
-  // the partition's staging; the next level's histograms), 16 KB each
+  // shared buffers for the phases' big arrays (histograms, candidate keys; the
+  // next level's histograms), 16 KB each
   __shared__ __align__(16) uint32_t s_big[2 * kHistBins];
   __shared__ __align__(16) uint32_t s_next[2 * kHistBins];
   unsigned epoch = 0;
@@ -1951,7 +1950,7 @@ int build_trees_object(bdl_forest *af, int dim, std::vector<BuildTree> &bt,
   uint32_t *hist = (uint32_t *)p; p += hist_bytes;   // the next one's states and its own
   unsigned long long *cursor = (unsigned long long *)p; p += cursor_bytes;   // histograms
   unsigned char *plan = p;
-  unsigned *bar = (unsigned *)((unsigned char *)cursor + align256((size_t)ntree * 8));   // [0..1] levels, [2..3] boxes
+  unsigned *bar = (unsigned *)((unsigned char *)cursor + align256((size_t)ntree * 8));   // [0] levels, [2] boxes
   const DTree *d_tree = (const DTree *)(plan + o_dt);
   const int32_t *d_act = (const int32_t *)(plan + o_act);
   const int64_t *d_pre = (const int64_t *)(plan + o_pre);

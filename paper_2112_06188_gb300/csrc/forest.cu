@@ -902,8 +902,7 @@ static void refresh_btrees(bdl_forest *const *F, int nf, cudaStream_t s, const s
   }
 }
 
-ForestView knn_view(bdl_forest *f, bool build, cudaStream_t s) {
-  if (build && f->buf_dirty) refresh_btrees(&f, 1, s);
+ForestView knn_view(bdl_forest *f) {
   ForestView fv = forest_view(f);
   if (f->btree && !f->buf_dirty && fv.ntrees < kMaxLevel) {
     TreeView &tv = fv.tree[fv.ntrees++];
@@ -1571,7 +1570,7 @@ static int knn_many(bdl_forest *const *F, int nf, const int32_t *const *q, const
   std::vector<KnnCall> calls;
   for (int i = 0; i < nf; ++i) {
     if (m[i] == 0) continue;
-    views[i] = knn_view(F[i], false, s);
+    views[i] = knn_view(F[i]);
     calls.push_back(KnnCall{&views[i], q[i], perm[i], m[i], oi[i], od[i], skewed_leaves(F[i])});
   }
   int st = BDL_OK;
@@ -1659,7 +1658,7 @@ static int knn_plan_make(bdl_forest *const *F, int nf, const int32_t *const *q, 
   size_t sort_bytes = 0;
   for (int i = 0; i < nf; ++i) {
     if (m[i] == 0) continue;
-    views[i] = knn_view(F[i], false, s);
+    views[i] = knn_view(F[i]);
     if (m[i] >= kSortMinQueries) sort_bytes += a256(query_sort_bytes(m[i], F[i]->dim));
     calls.push_back(KnnCall{&views[i], q[i], nullptr, m[i], oi[i], od[i], skewed_leaves(F[i])});
   }

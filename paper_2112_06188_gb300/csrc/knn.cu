@@ -1248,7 +1248,7 @@ extern "C" int bdl_knn_noalloc(bdl_forest *f, const int32_t *q, int64_t m, int k
   void *scratch = nullptr;
   int st = knn_scratch_address(f->device, &scratch);
   if (!st) {
-    ForestView fv = knn_view(f, false, s);   // never rebuilds (no allocation)
+    ForestView fv = knn_view(f);   // (the buffer's tree is not rebuilt: no allocation)
     count_knn_call(f);
     int32_t *perm = nullptr;
     if (m >= kSortMinQueries) {

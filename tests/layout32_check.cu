@@ -1,9 +1,9 @@
 // The 32-bit forms of the layout arithmetic that the kernels use, on the host:
-// equal to the 64-bit ones at every node of small trees, at every level's ends
-// and at places spread over the tallest trees there can be.
+// equal to the 64-bit ones (layout64.h) at every node of small trees, at every
+// level's ends and at places spread over the tallest trees there can be (30 levels).
 #include <cstdio>
 
-#include "../paper_2112_06188_gb300/csrc/bdl_internal.cuh"
+#include "layout64.h"
 
 using namespace bdl;
 
@@ -18,10 +18,10 @@ int main() {
     for (int t = 0; t <= h; ++t) {
       const int64_t n = (int64_t)1 << t, step = n <= 4096 ? 1 : n / 4093;
       for (int64_t i = 0; i < n; i += step) {
-        CHECK(veb_slot(h + 1, t, i) == (h < 30 ? veb_slot32(h + 1, t, (int)i) : veb_slot(h + 1, t, i)));
+        CHECK(veb_slot(h + 1, t, i) == veb_slot32(h + 1, t, (int)i));
         if (t < h && (t == 0 || ((h - t) & 1) == 0)) CHECK(packed_slot(h, t, i) == packed_slot32(h, t, (int)i));
       }
-      CHECK(h == 30 || veb_slot(h + 1, t, n - 1) == veb_slot32(h + 1, t, (int)(n - 1)));
+      CHECK(veb_slot(h + 1, t, n - 1) == veb_slot32(h + 1, t, (int)(n - 1)));
     }
     const int64_t n = packed_nrec(h), step = n <= 50000 ? 1 : n / 49999;
     for (int64_t g = 0; g < n; g += step) {

@@ -1,11 +1,12 @@
 // Host-side check of the library's layout arithmetic (bdl_internal.cuh):
 // the binary vEB slots, the segments of a level, the tree height, the bloom
 // hash's SplitMix64 mixer, and the packed k-NN records' level order, slots
-// and entries.  Prints the number of violations; exit status 0 when there are none.
+// and entries (layout64.h, which layout32_check.cu compares the kernels' forms
+// with).  Prints the number of violations; exit status 0 when there are none.
 #include <cstdio>
 #include <vector>
 
-#include "../paper_2112_06188_gb300/csrc/bdl_internal.cuh"
+#include "layout64.h"
 
 using namespace bdl;
 

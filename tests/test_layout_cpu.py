@@ -2,7 +2,8 @@
 the host: the vEB slot function against the paper's worked example and as a
 bijection, the segments of a level (left child ceil(m/2), reading G3), the
 tree height, and the packed k-NN record numbering (every record once,
-entries that are records or leaves two levels down)."""
+entries that are records or leaves two levels down) in the 64-bit form that
+test_layout32_cpu.py compares the kernels' own with."""
 import os
 import shutil
 import subprocess
