@@ -642,7 +642,6 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   const size_t b_i32 = al256((size_t)Nmax * 4), b_i64 = al256((size_t)Nmax * 8);
   const size_t b_tr = al256(ntree * sizeof(SpTree)), b_ga = al256(ga.size() * sizeof(SpGather));
   const size_t b_gpre = al256(gpre.size() * 8), b_lpre = al256(leaf_pre.size() * 8);
-  const size_t b_huge = al256((size_t)(S / kHugeLeaf + 1) * sizeof(HugeLeaf));
   // zeroed: gather cursors, sums of squared leaf sizes, the two barriers, the number of huge leaves
   const size_t b_cur = 2 * al256((size_t)ntree * 8) + 256;
   std::vector<int64_t> depth(std::max(hmax, 1), 0);
@@ -661,7 +660,7 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   }
   const size_t b_pk = al256(pk.size() * sizeof(TreeSeg)), b_pkpre = al256(pk_pre.size() * 8);
   const size_t total = 2 * b_stg + 2 * b_seg + 6 * b_i32 + 2 * (b_i64 + b_i32) + b_tr + b_ga + b_gpre + b_lpre +
-                       b_cur + b_pk + b_pkpre + 2 * b_depth + b_huge;
+                       b_cur + b_pk + b_pkpre + 2 * b_depth;
   void *block = nullptr;
   int st = dev_alloc(af, &block, total, s);
   if (st) return st;
@@ -688,7 +687,6 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
   nn[0] = (int32_t *)take(b_i32);
   lo[1] = (int64_t *)take(b_i64);
   nn[1] = (int32_t *)take(b_i32);
-  HugeLeaf *huge = (HugeLeaf *)take(b_huge);
   // the tables, in one upload
   std::vector<unsigned char> img;
   unsigned char *const tables = p;
@@ -748,7 +746,7 @@ int build_trees_spatial(bdl_forest *af, int dim, std::vector<BuildTree> &bt, con
     P.leaf_pre = d_lpre;
     P.depth = d_depth;
     P.sq = sq;
-    P.huge = huge;
+    P.huge = (HugeLeaf *)stg[0];   // (staging is free again; S / kHugeLeaf entries at most)
     P.nhuge = bar + 16;
     P.ntree = ntree;
     P.dim = dim;
