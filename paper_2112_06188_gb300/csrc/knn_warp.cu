@@ -27,13 +27,14 @@
 // (a dependent L2 read each); large ones by instruction issue (about 3,900
 // warp instructions per query on 2M 3-D points, 9,500 on 2M 7-D ones, 67 to
 // 75% of the issue slots) and by the shared/L1 data pipe (53 to 59%).
-// Measured against the thread-per-query kernel (1M 5-D points, k = 10, 316
-// queries: 1,014 -> 47 us; 50K 16-D points, k = 8, 1,000 queries: 1,495 -> 52;
-// 500K 4-D points, k = 32, 100K queries: 3,620 -> 768; 10M 7-D points of 100
-// clusters, k = 5, 1M queries: 31.4 -> 17.8 ms).
-// Without the starting bound and the narrow first rounds, and with them: those
-// four 50.5 -> 47, 55 -> 52, 840 -> 768 us and 20.3 -> 17.8 ms; 10M 3-D points,
-// k = 10, 30K queries 235 -> 202 us; 1M 2-D points of 100 clusters, spatial
+// Measured against the thread-per-query kernel as it was when this one came,
+// whole calls: 1M 5-D points, k = 10, 316 queries 1,212 -> 51 us (the kernel 43 to
+// 67 by the inputs: its longest chain); 50K 16-D points, k = 8, 1,000 queries 1,526
+// -> 48; 500K 4-D points, k = 32, 100K queries 3,644 -> 779; 10M 7-D points of 100
+// clusters, k = 5, 1M queries 31.4 -> 17.9 ms.
+// Without the starting bound and the narrow first rounds, and with them, in one
+// run: those four 50.5 -> 47, 55 -> 52, 840 -> 768 us and 20.3 -> 17.8 ms; 10M 3-D
+// points, k = 10, 30K queries 235 -> 202 us; 1M 2-D points of 100 clusters, spatial
 // median, k = 5, 100K queries 1,057 -> 865 us.
 #include "bdl_internal.cuh"
 
