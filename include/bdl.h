@@ -33,7 +33,7 @@
  *    skips the access and sets a bit in the forest's device error word (1 child
  *    slot, 2 leaf range, 4 traversal stack, 8 partition, 16 gather, 32 a packed
  *    k-NN record's live count differs from its node's, 64 a grid barrier of a
- *    build gave up after ten seconds).  bdl_insert and
+ *    build gave up after a minute).  bdl_insert and
  *    bdl_erase read the word at the waits they make and return BDL_EINTERNAL
  *    when a bit is set, with the bits in bdl_last_error(); bdl_poll_error reads
  *    it on demand.  With the environment variable BDL_DEBUG_CHECK=1 (read at

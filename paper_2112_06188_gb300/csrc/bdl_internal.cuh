@@ -371,12 +371,13 @@ enum : unsigned long long {
 // over the block's writes, and another after the wait).
 //
 // The wait is bounded by time: between two barriers a block may have much to
-// do (a select over hundreds of millions of equal coordinates in one block
-// takes about a second), so a block gives up after kBarrierNs, far above
+// do.  The longest is a median among points that are equal in the split
+// coordinate, which one block selects: 10M take 30 ms, 40M 220, 6 ns each, so
+// that 2^31 would take 13 s.  A block gives up after kBarrierNs, far above
 // that.  It then sets kErrBarrier in *err, lets every later wait of the launch
 // through (kBarrierOpen stands above any count of arrivals) and goes on, so a
 // lost block never hangs the GPU; the call then fails with BDL_EINTERNAL.
-constexpr unsigned long long kBarrierNs = 10000000000ull;
+constexpr unsigned long long kBarrierNs = 60000000000ull;
 constexpr unsigned kBarrierOpen = 1u << 30;
 __device__ __forceinline__ unsigned long long now_ns() {
   unsigned long long t;

@@ -47,6 +47,9 @@ int main() {
   for (int t = 0; t < kMaxHeight; t += packed_step(kMaxHeight, t)) ++levels;
   CHECK(kWWide - 8 + 32 + 3 * levels <= kWStack);
   CHECK(kMaxLevel + 1 + 32 <= kWWide);   // (the walk starts with every tree's root)
+  // a grid barrier waits several times as long as the longest phase of a build
+  // can take: one block's select over the most points there can be, 6 ns each
+  CHECK(kBarrierNs >= 4 * 6 * (unsigned long long)INT32_MAX);
   puts(bad ? "BAD" : "ok");
   return bad != 0;
 }
